@@ -213,6 +213,16 @@ cudaError_t launch_wfa(const WfaPlan& plan, int group, const PairsView& P, const
                        uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms, cudaStream_t st,
                        int* warps_used);
 
+// the form of wfa_ring.cu (state in shared memory): whether the costs and lengths allow it, whether a launch with G
+// lanes per pair (1..32) fits shared memory and the scratch, the lanes suited to a batch (0: does not fit), one launch
+// over all pairs, or over the queue range bounds[0..1] of order
+bool ring_ok(const WfaPlan& p, uint32_t max_length);
+bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_bytes);
+int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes);
+cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, const LimitView& L, const OutView& O,
+                            const uint32_t* order, const uint32_t* bounds, uint8_t* scratch, size_t scratch_bytes,
+                            uint32_t* counters, int num_sms, cudaStream_t st, int* warps_used);
+
 // GenASM (windowed bitap): scratch per warp for windows of W bases under the largest threshold max_limit
 size_t genasm_warp_bytes(int W, int64_t max_limit, uint32_t max_length);
 cudaError_t launch_genasm(int W, int O, const PairsView& P, const LimitView& L, const OutView& Ov, int64_t max_limit,

@@ -183,6 +183,14 @@ int align_packed(aim_ctx* ctx, const aim::PairsView& P, int algo, const aim_pena
                                           &w2);
                 if (err == cudaSuccess && w2 == 0) warps = 0;
             }
+        } else if (const int ring = !aim::ring_ok(plan, P.max_length) ? 0
+                                    : !ctx->wfa_group ? aim::ring_group(plan, P.max_length, P.num_pairs, ctx->num_sms,
+                                                                        scratch_bytes)
+                                    : aim::ring_fits(plan, ctx->wfa_group, P.max_length, scratch_bytes) ? ctx->wfa_group
+                                                                                                         : 0) {
+            slot = time_begin(ctx, 1, st);
+            err = aim::launch_wfa_ring(plan, ring, P, r.lim, O, nullptr, nullptr, scratch, scratch_bytes, counter,
+                                       ctx->num_sms, st, &warps);
         } else {
             const int group = fit_group(plan, ctx->wfa_group ? ctx->wfa_group
                                                              : aim::wfa_default_group(plan, P.max_length));

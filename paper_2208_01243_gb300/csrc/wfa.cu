@@ -61,6 +61,7 @@
 #include <vector>
 
 #include "aim_internal.cuh"
+#include "wfa_common.cuh"
 
 namespace aim {
 namespace {
@@ -207,32 +208,6 @@ __device__ __forceinline__ int extend(const PairSeqs<STAGE>& q, int n, int m, in
     }
     return h;
 }
-
-// 32 bases ending at base p (inclusive) with base p in the low two bits; for
-// p < 31 only bases 0..p are present (in the low bits).
-__device__ __forceinline__ uint64_t window_ending(const uint64_t* w, uint32_t nwords, int p) {
-    if (p >= 31) return window32(w, nwords, (uint32_t)(p - 31));
-    return window32(w, nwords, 0) >> (2 * (31 - p));
-}
-
-// number of consecutive matches P[v-1-i] == T[h-1-i], i = 0, 1, ... (at most min(v, h))
-__device__ __forceinline__ int match_run_back(const uint64_t* Pw, uint32_t nwP, int v, const uint64_t* Tw,
-                                              uint32_t nwT, int h) {
-    int run = 0;
-    for (;;) {
-        const int pv = v - 1 - run, ph = h - 1 - run;
-        if (pv < 0 || ph < 0) break;
-        const uint64_t d = window_ending(Pw, nwP, pv) ^ window_ending(Tw, nwT, ph);
-        const int avail = min(min(pv, ph) + 1, 32);
-        int z = d ? ((__ffsll((long long)d) - 1) >> 1) : 32;
-        if (z > avail) z = avail;
-        run += z;
-        if (z < 32) break;
-    }
-    return run;
-}
-
-enum : int { kRun = 0, kDone = 1, kRejected = 2, kCap = 3, kBad = 4, kIdle = 5 };
 
 // Collectives of one group.  G <= 32: a warp holds 32/G groups that run in lockstep, so loop
 // conditions are warp-wide and group results come from masked ballots and butterflies.  G == 256:
@@ -987,30 +962,6 @@ __device__ __noinline__ uint32_t traceback_compact(const WfaArgs& a, uint8_t* re
     wr.finish();
     ok = ok && wr.n <= wr.cap;
     return wr.n;
-}
-
-// Result of a finished pair: score, flags, run count, and its runs (staged end-first) copied start-first by
-// lanes gl, gl + G, ... of its group; every lane of the group calls this with the same values.
-__device__ __forceinline__ void emit_done(const WfaArgs& a, uint32_t pi, int final_s, uint32_t nruns, bool ok,
-                                          const uint32_t* staged, int gl, int G) {
-    const int32_t score = final_s * a.g;
-    uint8_t flags = ok ? 0 : AIM_F_STEP_CAP;
-    if (ok && a.O.cigars && a.O.cigar_off) {
-        const uint64_t off = a.O.cigar_off[pi];
-        const uint64_t cap = a.O.cigar_off[pi + 1] - off;
-        if (nruns <= cap) {
-            for (uint32_t j = (uint32_t)gl; j < nruns; j += (uint32_t)G) a.O.cigars[off + j] = staged[nruns - 1 - j];
-        } else {
-            flags |= AIM_F_CIGAR_OVERFLOW;
-        }
-    }
-    if (gl == 0) write_header(a.O, pi, ok ? score : -1, flags, nruns);
-}
-
-// One lane: result of a pair that ended without an alignment.
-__device__ __forceinline__ void emit_failed(const WfaArgs& a, uint32_t pi, int status) {
-    const uint8_t f = status == kBad ? AIM_F_BAD_PAIR : status == kRejected ? AIM_F_REJECTED : AIM_F_STEP_CAP;
-    write_header(a.O, pi, -1, f, 0);
 }
 
 // finished pairs awaiting their traceback: G records per group, 32 per warp (pair, final score, region

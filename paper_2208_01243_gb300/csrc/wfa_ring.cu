@@ -1,0 +1,595 @@
+// Gap-affine wavefront alignment with the running state in shared memory: the form for thresholds whose wavefronts
+// are narrow enough to hold a pair's last few wavefronts beside its sequences (see ring_ok).
+//
+// G lanes align one pair and a warp runs P = 32 / G pairs in lockstep, G = 1 being one pair per lane.  Lane
+// l = gl * P + g is lane gl of pair g, and every per-pair array in shared memory is interleaved by pair (element j of
+// pair g at [j * P + g]), so whatever the diagonal, the 32 lanes of an access touch 32 consecutive words.
+//
+// Scores are scaled as in wfa.cu (X, OE = O + E, and E == 1 here).  Instead of reading M~[s-OE] and I~[s-E] from
+// stored wavefronts, the pass carries, per diagonal k,
+//   mh[k]  M~[s-1..s-4, k], four 16-bit values in one 64-bit word that shifts by one value per score,
+//   jd[k]  J = max(M~[s-O, k], I~[s, k]) and K = max(M~[s-O, k], D~[s, k]), two 16-bit values,
+// so that   I~[s, k] = J[s-1, k+1],   D~[s, k] = K[s-1, k-1] + 1   and M~[s-X, k], M~[s-O, k] come out of mh by one
+// byte permute each: three shared loads and two stores per entry, with no test against any wavefront's range.
+// An invalid value is -1; a candidate is dropped when it would leave the matrix, as in wfa.cu.
+//
+// Ranges.  Row s covers the diagonals that can lie on an alignment within the limit S: at most s - O from diagonal
+// 0, at most S - s from the end diagonal kend, and inside the window [kmin, kmax] outside which even a gap out and a
+// gap back cost more than S (2 O + |k| + |k - kend| > S).  The ranges are arithmetic in s, so no per-score record is
+// read or reduced.  Dropping the other diagonals changes no result: a value that would have come from outside lies on
+// no alignment of cost <= S, and the traceback reads entries on optimal paths only.  Every pair walks its own row; the
+// warp walks as many entries as its widest row.  The positions just outside a row read as invalid in the next one.
+//
+// History for the traceback: row s is one run of entries in the warp's scratch, written 32 consecutive entries at a
+// time, at a fixed distance from the row before: (M~, I~, D~) + 1 in 10 bits each for reads up to 1,022 bp, three
+// 16-bit values beyond.  A round of P pairs leaves its history in the warp's arena; after G rounds (or when the
+// arena may not hold another) the 32 lanes trace back one pair each, by the tests of wfa.cu.
+//
+// What bounds it: instruction issue.  1M pairs of 150 bp at 6 edits take 900 warp instructions a pair at 2.7 per
+// cycle (wfa.cu's 4-lane groups: 1,790 at 2.2), 1.03 ms against 2.43 ms; 250 bp, band 25, 25 edits 9.6 ms against
+// 21.4 ms (all on one launch, packing apart).
+#include <algorithm>
+#include <cstdint>
+#include <type_traits>
+
+#include "wfa_common.cuh"
+
+namespace aim {
+namespace {
+
+constexpr int kWarpsPerBlock = 4;
+constexpr int kMhDepth = 4;               // scores of M~ held per diagonal
+constexpr uint32_t kNarrowLength = 1022;  // longest read whose offsets + 1 fit 10 bits
+
+struct RingArgs {
+    WfaArgs w;
+    uint32_t width;          // diagonals per pair in shared memory, two of them padding
+    uint32_t seq_words;      // 32-bit words per sequence in shared memory
+    uint32_t seq_rounds;     // rounds whose copies are kept: G, or 1 and the traceback reads the packed sequences
+    uint32_t smem_warp;      // bytes of shared memory per warp
+    uint32_t stage_shared;   // runs are staged in shared memory
+    size_t round_bytes;      // history of one round, worst case
+    uint32_t sel_x, sel_o;   // byte permute selectors of M~[s-X], M~[s-O] in mh
+};
+
+__device__ __forceinline__ int prmt(uint32_t a, uint32_t b, uint32_t sel) {   // sign-replicating byte permute
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return (int)r;
+}
+
+// history entries: 10 bits of value + 1 for each of M~, I~, D~, or three int16
+template <typename E>
+struct Entry;
+template <>
+struct Entry<uint32_t> {
+    static constexpr uint32_t kBias = 1u | (1u << 10) | (1u << 20);
+    static __device__ __forceinline__ uint32_t make(int m, int i, int d) {
+        return (uint32_t)m + ((uint32_t)i << 10) + ((uint32_t)d << 20);   // each value + 1 once kBias is added
+    }
+    static __device__ __forceinline__ int m(uint32_t e) { return (int)((e + kBias) & 1023u) - 1; }
+    static __device__ __forceinline__ int i(uint32_t e) { return (int)(((e + kBias) >> 10) & 1023u) - 1; }
+    static __device__ __forceinline__ int d(uint32_t e) { return (int)((e + kBias) >> 20) - 1; }
+    static __device__ __forceinline__ uint32_t none() { return 0u - kBias; }
+};
+template <>
+struct Entry<uint64_t> {
+    static __device__ __forceinline__ uint64_t make(int m, int i, int d) {
+        return (uint64_t)(uint32_t)prmt((uint32_t)m, (uint32_t)i, 0x5410u) | ((uint64_t)(uint32_t)d << 32);
+    }
+    static __device__ __forceinline__ int m(uint64_t e) { return (int16_t)(uint16_t)e; }
+    static __device__ __forceinline__ int i(uint64_t e) { return (int16_t)(uint16_t)(e >> 16); }
+    static __device__ __forceinline__ int d(uint64_t e) { return (int16_t)(uint16_t)(e >> 32); }
+    static __device__ __forceinline__ uint64_t none() { return ~0ull; }
+};
+
+// 16 bases from position pos of a sequence copy (32-bit word i of the pair at [i * P])
+template <int P>
+__device__ __forceinline__ uint32_t window16(const uint32_t* s, int pos) {
+    const uint32_t* w = s + (pos >> 4) * P;
+    return __funnelshift_l(w[P], w[0], 2 * pos);   // the shift is taken modulo 32
+}
+
+// the match run from (v, h) on, 32 bases a turn: at most rem
+template <int P>
+__device__ __forceinline__ int match_on(const uint32_t* sp, const uint32_t* st, int v, int h, int rem) {
+    int run = 0;
+    const uint32_t* p = sp + (v >> 4) * P;
+    const uint32_t* t = st + (h >> 4) * P;
+    uint32_t a = p[0], c = t[0];
+    do {
+        const uint32_t b = p[P], d = t[P];
+        const uint32_t x = __funnelshift_l(b, a, 2 * v) ^ __funnelshift_l(d, c, 2 * h);
+        if (x || run + 16 >= rem) { run += __clz((int)x) >> 1; break; }   // __clz(0) = 32
+        a = p[2 * P]; c = t[2 * P];
+        const uint32_t y = __funnelshift_l(a, b, 2 * v) ^ __funnelshift_l(c, d, 2 * h);
+        run += 16 + (__clz((int)y) >> 1);
+        if (y) break;
+        p += 2 * P; t += 2 * P;
+    } while (run < rem);
+    return min(run, rem);
+}
+
+// runs in end-first order, every `stride` words
+struct RunStage {
+    uint32_t* runs;
+    uint32_t stride, cap, n, op, len;
+    __device__ __forceinline__ void flush() {
+        if (len) {
+            if (n < cap) runs[n * stride] = (len << 4) | op;
+            ++n;
+        }
+    }
+    __device__ __forceinline__ void put(uint32_t o, uint32_t l) {
+        if (o == op) { len += l; return; }
+        flush();
+        op = o; len = l;
+    }
+};
+
+// A pair's ring: diagonal k at position k - koff, position 1 the window's first diagonal and `last` its last one;
+// diagonal 0 at `zero`, the end diagonal at `end`.  Row s covers lo(s) .. hi(s).
+struct Window {
+    int koff, last, zero, end, S;
+    __device__ __forceinline__ int lo(int s, int O) const { return max(max(zero - max(s - O, 0), end - (S - s)), 1); }
+    __device__ __forceinline__ int hi(int s, int O) const { return min(min(zero + max(s - O, 0), end + (S - s)), last); }
+};
+
+// What the traceback of a lane's pair needs.
+struct Pending {
+    uint32_t pi;
+    int final_s;             // < 0: none
+    int koff, last, S;       // its Window
+    uint32_t base, stride;   // its round's history: 256-byte units from the arena's rounds, entries per row
+    int round;
+};
+
+// Canonical traceback of one finished pair by one lane (the tests of wfa.cu's traceback).  Every step issues all its
+// loads at once: the four entries and both sequences' windows ending at (v, h), whose XOR gives the match run.
+// The rows' ranges are those of the forward pass, by arithmetic: no table is read.
+// seqs_kept: the pair's copies in shared memory (words [i * P]); otherwise the packed sequences are read.
+template <int P, typename E>
+__device__ uint32_t ring_traceback(const WfaArgs& a, const uint8_t* rounds, const Pending& q, int g, bool seqs_kept,
+                                   const uint32_t* sp, const uint32_t* st, RunStage& wr, bool& ok) {
+    const E* hist = reinterpret_cast<const E*>(rounds + ((size_t)q.base << 8)) + g;
+    const int n = (int)a.P.read_len[q.pi], m = (int)a.P.target_len[q.pi];
+    const uint64_t* Pg = read_words(a.P, q.pi);
+    const uint64_t* Tg = target_words(a.P, q.pi);
+    const uint32_t nwP = (uint32_t)(n + 31) >> 5, nwT = (uint32_t)(m + 31) >> 5;
+    const int X = a.X, OE = a.OE, O = OE - 1;
+    const Window w{q.koff, q.last, -q.koff, m - n - q.koff, q.S};
+    auto entry = [&](int c, int j) -> E {
+        const int lo = w.lo(c, O);
+        if (c < 0 || j < lo || j > w.hi(c, O)) return Entry<E>::none();
+        return hist[(size_t)(uint32_t)c * q.stride + (uint32_t)((j - lo) * P)];
+    };
+    int v = n, h = m, cM = q.final_s, cI = q.final_s, cD = q.final_s;
+    while (v > 0 || h > 0) {
+        const int j = h - v - q.koff;
+        const E eX = entry(cM - X, j), eI = entry(cI, j), eD = entry(cD, j), eM = entry(cM, j);
+        const int avail = min(v, h);
+        int same;   // matching bases back from (v, h), as far as the window shows
+        if (seqs_kept) {   // 16 bases back; before the start the window's earlier bases are not looked at
+            const int back = min(avail, 16);
+            const uint32_t x = window16<P>(sp, max(v - 16, 0)) >> (v < 16 ? 2 * (16 - v) & 31 : 0);
+            const uint32_t y = window16<P>(st, max(h - 16, 0)) >> (h < 16 ? 2 * (16 - h) & 31 : 0);
+            const uint32_t d = x ^ y;
+            same = min(d ? (__ffs((int)d) - 1) >> 1 : 16, back);
+        } else {
+            const int back = min(avail, 32);
+            const uint64_t d = back ? window_ending(Pg, nwP, v - 1) ^ window_ending(Tg, nwT, h - 1) : 1ull;
+            same = min(d ? (__ffsll((long long)d) - 1) >> 1 : 32, back);
+        }
+        const bool diag = avail > 0, match = same > 0;
+        if (diag && !match && Entry<E>::m(eX) >= h - 1) {
+            cM = cI = cD = cM - X; --v; --h;
+            wr.put(kOpMismatch, 1);
+        } else if (v > 0 && Entry<E>::i(eI) >= h) {
+            const int c = cI;
+            cM = cD = c - OE; cI = c - 1; --v;
+            wr.put(kOpIns, 1);
+        } else if (h > 0 && Entry<E>::d(eD) >= h) {
+            const int c = cD;
+            cM = cI = c - OE; cD = c - 1; --h;
+            wr.put(kOpDel, 1);
+        } else if (match && Entry<E>::m(eM) >= h - 1) {
+            // a longer run is taken window by window: I~ and D~ of this score stop it at the same offset
+            const int run = min(same, h - max(Entry<E>::i(eM), Entry<E>::d(eM)));
+            if (run < 1) { ok = false; break; }
+            v -= run; h -= run;
+            cI = cD = cM;
+            wr.put(kOpMatch, (uint32_t)run);
+        } else {
+            ok = false;
+            break;
+        }
+    }
+    wr.flush();
+    ok = ok && wr.n <= wr.cap;
+    return wr.n;
+}
+
+extern __shared__ __align__(16) uint8_t s_ring[];
+
+template <int G, typename E>
+__global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs r) {
+    constexpr int P = 32 / G;
+    constexpr int kRows = G == 1 ? 1 : 2;   // jd rows: one lane per pair updates its row in place
+    const WfaArgs& a = r.w;
+    const int lane = (int)(threadIdx.x & 31);
+    const int g = lane % P, gl = lane / P;
+    const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (gwarp >= a.nwarps) return;
+    const uint32_t W = r.width;
+    uint8_t* sm = s_ring + (size_t)(threadIdx.x >> 5) * r.smem_warp;
+    uint2* mh = reinterpret_cast<uint2*>(sm);                            // [W][P]
+    uint32_t* jd = reinterpret_cast<uint32_t*>(sm + (size_t)W * P * 8);  // [kRows][W][P]
+    // copies of a round's reads, then of its targets, [seq_words][P] each; of every round awaiting its traceback
+    // when seq_rounds says so
+    uint32_t* seq = jd + (size_t)kRows * W * P;
+    const uint32_t seq_round = 2 * r.seq_words * P;
+    const bool seqs_kept = r.seq_rounds == (uint32_t)G;
+    uint8_t* arena = a.scratch + (size_t)gwarp * a.warp_bytes;
+    uint8_t* rounds = arena + 32 * a.runs_bytes;
+    const size_t rounds_bytes = a.warp_bytes - 32 * a.runs_bytes;
+    const int O = a.OE - 1;
+    const uint32_t begin = a.bounds ? a.bounds[0] : 0;
+    const uint32_t end = a.bounds ? a.bounds[1] : a.P.num_pairs;
+    unsigned long long st_cells = 0, st_windows = 0;
+    uint32_t st_pairs = 0;
+
+    Pending pend{0, -1, 0, 0, 0, 0, 0, 0};
+    int round = 0;
+    size_t used = 0;   // arena bytes of the rounds awaiting their traceback
+    auto finish = [&]() {
+        __syncwarp();
+        // runs staged where the forward pass kept its state, lane l's i-th run at [33 i + l], or in the arena
+        uint32_t* stage = r.stage_shared ? reinterpret_cast<uint32_t*>(sm) + lane
+                                         : reinterpret_cast<uint32_t*>(arena + (size_t)lane * a.runs_bytes);
+        RunStage wr{stage, r.stage_shared ? 33u : 1u, a.runs_cap, 0, 0, 0};
+        bool ok = pend.final_s >= 0;
+        uint64_t off = 0;
+        uint32_t copy = 0;
+        if (ok) {
+            const uint32_t* sp = seq + (seqs_kept ? (uint32_t)pend.round * seq_round : 0u) + g;
+            const uint32_t nruns = ring_traceback<P, E>(a, rounds, pend, g, seqs_kept, sp, sp + r.seq_words * P, wr, ok);
+            uint8_t flags = ok ? 0 : AIM_F_STEP_CAP;
+            if (ok && a.O.cigars) {
+                off = a.O.cigar_off[pend.pi];
+                if (nruns <= a.O.cigar_off[pend.pi + 1] - off) copy = nruns;
+                else flags = AIM_F_CIGAR_OVERFLOW;
+            }
+            write_header(a.O, pend.pi, ok ? pend.final_s * a.g : -1, flags, nruns);
+        }
+        __syncwarp();
+        if (a.O.cigars) {   // half a warp copies one pair's runs, start first
+            const int hl = lane & 15;
+            for (int q = lane >> 4; q < 32; q += 2) {
+                const uint32_t cnt = __shfl_sync(kFull, copy, q);
+                const uint64_t at = __shfl_sync(kFull, off, q);
+                const uint32_t* from = r.stage_shared ? reinterpret_cast<const uint32_t*>(sm) + q
+                                                      : reinterpret_cast<const uint32_t*>(arena + (size_t)q * a.runs_bytes);
+                const uint32_t step = r.stage_shared ? 33u : 1u;
+                for (uint32_t i = (uint32_t)hl; i < cnt; i += 16) a.O.cigars[at + i] = from[(cnt - 1 - i) * step];
+            }
+        }
+        __syncwarp();
+        pend.final_s = -1;
+        round = 0;
+        used = 0;
+    };
+
+    for (;;) {
+        uint32_t pos = 0;
+        if (lane == 0) pos = atomicAdd(a.counters, (uint32_t)P);
+        pos = __shfl_sync(kFull, pos, 0);
+        if (pos >= end - begin || end <= begin) break;
+        if (round == G || rounds_bytes - used < r.round_bytes) finish();
+
+        // ---- the round's pairs
+        const uint32_t q = begin + pos + (uint32_t)g;
+        int status = kIdle, n = 0, m = 0, S = 0, kend = 0;
+        uint32_t pi = 0;
+        bool skip = q >= end;
+        if (!skip) {
+            pi = a.order ? a.order[q] : q;
+            skip = a.retry_only && a.O.flags[pi] != AIM_F_STEP_CAP;
+        }
+        if (!skip) {
+            n = (int)a.P.read_len[pi];
+            m = (int)a.P.target_len[pi];
+            kend = m - n;
+            const int64_t lim = pair_limit(a.L, pi);
+            if (gl == 0) ++st_pairs;
+            if (pair_bad(a.P, pi) || (uint32_t)n > a.P.max_length || (uint32_t)m > a.P.max_length || lim == -2) {
+                status = kBad;
+            } else {
+                const int64_t S64 = lim / a.g;
+                S = (int)(S64 > a.smax ? a.smax : S64);
+                if (a.bound) {   // a bound pass found an alignment of this score: the optimum is at most that
+                    const int ub = a.bound[pi];
+                    if (ub >= 0 && ub < S) S = ub;
+                }
+                // rejected at once: the end diagonal outside the band, or its gap alone above the limit
+                const bool far = a.band >= 0 && (kend > a.band || -kend > a.band);
+                status = far || S < 0 || (kend != 0 && abs(kend) + O > S) ? kRejected : kRun;
+            }
+        }
+        bool run = status == kRun;
+        Window win{0, 0, 0, 0, S};
+        if (run) {
+            // the window: 2 O + k + (k - kend) <= S beyond both 0 and kend, and likewise on the other side
+            int right = min(max(max(0, kend), (S - 2 * O + kend) >> 1), m);
+            int left = min(max(max(0, -kend), (S - 2 * O - kend) >> 1), n);
+            if (a.band >= 0) { right = min(right, a.band); left = min(left, a.band); }
+            win = Window{-left - 1, left + right + 1, left + 1, kend + left + 1, S};
+        }
+        const int wide = __reduce_max_sync(kFull, win.last);   // 0: no pair to run
+        // entry (s, t-th of its row) of the history at [s * stride + t * P]
+        const uint32_t stride = ((uint32_t)wide * P + 31u) & ~31u;
+        int final_s = -1, s = 0;
+        if (wide) {
+            uint32_t* dp = seq + (seqs_kept ? (uint32_t)round * seq_round : 0u) + g;
+            uint32_t* dt = dp + r.seq_words * P;
+            const uint32_t* sp = dp;
+            const uint32_t* st = dt;
+            // nothing is reachable yet
+            for (int i = lane; i < (wide + 2) * P; i += 32) {
+                mh[i] = make_uint2(~0u, ~0u);
+                jd[i] = ~0u;
+                if (kRows == 2) jd[i + W * P] = ~0u;
+            }
+            if (run) {
+                const uint64_t* Pw = read_words(a.P, pi);
+                const uint64_t* Tw = target_words(a.P, pi);
+                for (int w = gl; w < (n + 31) >> 5; w += G) {
+                    const uint64_t x = __ldg(Pw + w);
+                    dp[2 * w * P] = (uint32_t)(x >> 32); dp[(2 * w + 1) * P] = (uint32_t)x;
+                }
+                for (int w = gl; w < (m + 31) >> 5; w += G) {
+                    const uint64_t x = __ldg(Tw + w);
+                    dt[2 * w * P] = (uint32_t)(x >> 32); dt[(2 * w + 1) * P] = (uint32_t)x;
+                }
+            }
+            __syncwarp();
+            uint32_t cells = 0, windows = 0;
+            E* hrow = reinterpret_cast<E*>(rounds + used) + lane;   // row s, this lane's first entry
+            // row 0: diagonal 0 from offset 0
+            if (run && gl == 0) {
+                const int m0 = match_on<P>(sp, st, 0, 0, min(n, m));
+                mh[win.zero * P + g] = make_uint2((uint32_t)m0 | 0xffff0000u, ~0u);
+                hrow[0] = Entry<E>::make(m0, -1, -1);
+                ++cells; ++windows;
+            }
+            for (;;) {
+                // the row just computed ends the pair if it reaches the end of the end diagonal
+                if (G > 1) __syncwarp();
+                if (run && (int)(mh[win.end * P + g].x & 0xffffu) == m) { status = kDone; final_s = s; run = false; }
+                ++s;
+                if (run && s > S) { status = kRejected; run = false; }
+                if (!__any_sync(kFull, run)) break;
+                hrow += stride;
+                const int jlo = win.lo(s, O), jhi = win.hi(s, O);
+                const int w = run ? max(jhi - jlo + 1, 0) : 0;
+                const int rows = __reduce_max_sync(kFull, w);
+                const uint32_t odd = (uint32_t)(s & 1);
+                const uint32_t at = (uint32_t)(jlo * P + g);       // the row's first position
+                uint2* mhr = mh + at;
+                uint32_t* jw = (kRows == 2 ? jd + odd * (W * P) : jd) + at;                // this row
+                const uint32_t* jr = (kRows == 2 ? jd + (odd ^ 1u) * (W * P) : jd) + at;   // row s-1
+                const int kb = jlo + win.koff;                     // the row's first diagonal
+                uint32_t before = 0, here = 0;   // G == 1: jd of positions j-1 and j in row s-1
+                // U entries of every lane at a time: the loads and the first 16 bases of each overlap
+                auto step = [&](const int tb, auto count) {
+                    constexpr int U = decltype(count)::value;
+                    int mv[U], ins[U], del[U], mo[U], hmax[U];
+                    uint32_t x[U];
+                    uint2 h4[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int t = min(tb + u * G + (G > 1 ? gl : 0), w - 1);   // a lane past its row repeats the last
+                        uint32_t left, right;
+                        if (G == 1) {
+                            left = before;
+                            right = jr[(t + 1) * P];
+                            before = here;
+                            here = right;
+                        } else {
+                            left = jr[(t - 1) * P]; right = jr[(t + 1) * P];
+                        }
+                        h4[u] = mhr[t * P];
+                        const int k = kb + t;
+                        hmax[u] = min(m, n + k);   // >= 0 inside the window
+                        mo[u] = prmt(h4[u].x, h4[u].y, r.sel_o);
+                        int mis = prmt(h4[u].x, h4[u].y, r.sel_x);
+                        ins[u] = prmt(right, 0u, 0x9910u);
+                        del[u] = prmt(left, 0u, 0xbb32u);
+                        mis = (unsigned)mis < (unsigned)hmax[u] ? mis + 1 : -1;
+                        del[u] = (unsigned)del[u] < (unsigned)hmax[u] ? del[u] + 1 : -1;
+                        ins[u] = ins[u] <= hmax[u] ? ins[u] : -1;   // (an invalid -1 stays)
+                        mv[u] = max(mis, max(ins[u], del[u]));
+                        // an invalid entry reads words before its copies, inside the warp's shared memory, and
+                        // matches nothing
+                        x[u] = (window16<P>(sp, mv[u] - k) ^ window16<P>(st, mv[u])) | (uint32_t)(mv[u] >> 31);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int t = tb + u * G + (G > 1 ? gl : 0);
+                        const int rem = hmax[u] - mv[u];   // bases left on both sequences
+                        int len = min(__clz((int)x[u]) >> 1, rem);
+                        if (t < w) windows += 1 + (mv[u] >> 31);
+                        if (x[u] == 0 && rem > 16) {
+                            len = 16 + match_on<P>(sp, st, mv[u] - kb - min(t, w - 1) + 16, mv[u] + 16, rem - 16);
+                            if (t < w) windows += (uint32_t)len >> 5;
+                        }
+                        mv[u] += len;
+                        if (t < w) {
+                            mhr[t * P] =
+                                make_uint2((uint32_t)prmt((uint32_t)mv[u], h4[u].x, 0x5410u),
+                                           (uint32_t)prmt(h4[u].x, h4[u].y, 0x5432u));
+                            jw[t * P] = (uint32_t)prmt((uint32_t)max(mo[u], ins[u]), (uint32_t)max(mo[u], del[u]), 0x5410u);
+                            hrow[(tb + u * G) * P] = Entry<E>::make(mv[u], ins[u], del[u]);
+                        }
+                    }
+                };
+                if (w > 0) {   // lanes whose pair has ended have no row
+                    if (G == 1) { before = jr[-P]; here = jr[0]; }
+                    int t = 0;
+                    for (; t + G < rows; t += 2 * G) step(t, std::integral_constant<int, 2>{});
+                    if (t < rows) step(t, std::integral_constant<int, 1>{});
+                }
+                if (gl == 0 && w > 0) {   // just outside the row: invalid
+                    jw[-P] = ~0u;
+                    jw[w * P] = ~0u;
+                    cells += (uint32_t)w;
+                }
+            }
+            st_cells += cells;
+            st_windows += windows;
+        }
+        if (gl == 0 && (status == kRejected || status == kBad)) emit_failed(a, pi, status);
+        // lane round * P + g will trace pair g of this round
+        const int src = lane % P;
+        const uint32_t p_pi = __shfl_sync(kFull, pi, src);
+        const int p_s = __shfl_sync(kFull, final_s, src), p_koff = __shfl_sync(kFull, win.koff, src);
+        const int p_last = __shfl_sync(kFull, win.last, src), p_S = __shfl_sync(kFull, S, src);
+        if (lane / P == round) pend = Pending{p_pi, p_s, p_koff, p_last, p_S, (uint32_t)(used >> 8), stride, round};
+        if (wide) {
+            used += ((size_t)s * stride * sizeof(E) + 255) & ~(size_t)255;
+            ++round;
+        }
+    }
+    finish();
+    warp_stat_add(a.O.stats, 0, st_cells, (uint32_t)lane);
+    warp_stat_add(a.O.stats, 1, st_windows, (uint32_t)lane);
+    warp_stat_add(a.O.stats, 3, st_pairs, (uint32_t)lane);
+}
+
+template <typename E>
+void (*ring_kernel_for(int G))(RingArgs) {
+    switch (G) {
+        case 1: return wfa_ring_kernel<1, E>;
+        case 2: return wfa_ring_kernel<2, E>;
+        case 4: return wfa_ring_kernel<4, E>;
+        case 8: return wfa_ring_kernel<8, E>;
+        case 16: return wfa_ring_kernel<16, E>;
+        default: return wfa_ring_kernel<32, E>;
+    }
+}
+
+// Lanes per pair: the fewest whose warps fit an SM at least 16 at a time (14 KB of shared memory each), since one lane
+// per pair wastes no lane on a row's end and shares a row's fixed work between the most pairs; more when the batch
+// would otherwise give the device less than 8 warps per SM, where the pair's own serial chain is what counts.
+// Measured, ms at 1 / 2 / 4 / 8 / 16 lanes: 1M x 150 bp, 6 edits (12 KB at 1 lane) 1.15 / 1.24 / 1.50 / 1.99 / 2.89;
+// 1M x 250 bp, 25 edits, band 25 (12 KB at 4) 13.4 / 10.7 / 9.8 / 10.4 / 12.8; 300k x 300 bp, 30 edits (11 KB at 8)
+// 12.6 / 12.2 / 5.7 / 4.6 / 4.9; 10k x 150 bp 0.080 / 0.067 / 0.060 / 0.064 / 0.073; 61 x 150 bp 0.072 / 0.056 /
+// 0.045 / 0.039 / 0.037.
+constexpr size_t kGoodSmem = 14u << 10;
+constexpr int kGoodWarps = 8;
+constexpr size_t kMaxSmem = 227u << 10;   // shared memory a block may use
+
+size_t entry_bytes(uint32_t max_length) { return max_length <= kNarrowLength ? 4 : 8; }
+
+// diagonals per pair: the widest window (2 O + 2 k - kend <= S on both sides, or just 0 .. kend: S - O + 1), the
+// band's or the matrix's, and the two padding positions
+int64_t ring_width(const WfaPlan& p, uint32_t max_length) {
+    const int64_t O = p.oe - p.e;
+    int64_t w = p.smax - O + 1;
+    if (p.band >= 0) w = std::min<int64_t>(w, 2 * (int64_t)p.band + 1);
+    return std::max<int64_t>(std::min<int64_t>(w, 2 * (int64_t)max_length + 1), 1) + 2;
+}
+
+uint32_t seq_words(uint32_t max_length) { return 2 * ((max_length + 31) / 32) + 2; }
+
+}  // namespace
+
+namespace {
+
+// bytes of the copies of `pairs` pairs' sequences
+size_t seq_bytes(uint32_t max_length, size_t pairs) { return pairs * 2 * seq_words(max_length) * 4; }
+
+// the copies of every round are kept for the traceback while they take no more than this
+constexpr size_t kKeepBytes = 5u << 10;
+
+}  // namespace
+
+size_t ring_smem_per_warp(const WfaPlan& p, int G, uint32_t max_length) {
+    const size_t P = 32 / G, W = (size_t)ring_width(p, max_length);
+    const size_t kept = seq_bytes(max_length, 32) <= kKeepBytes ? 32 : P;
+    return align_up(P * W * (8 + (G == 1 ? 4 : 8)) + seq_bytes(max_length, kept), 16);
+}
+
+size_t ring_warp_bytes(const WfaPlan& p, int G, uint32_t max_length) {
+    const size_t P = 32 / G, W = (size_t)ring_width(p, max_length);
+    const size_t hist = ((size_t)p.smax + 1) * ((W * P + 31) / 32 * 32) * entry_bytes(max_length);
+    return align_up(32 * p.runs_bytes + hist + 256, 256);
+}
+
+bool ring_ok(const WfaPlan& p, uint32_t max_length) {
+    const int O = p.oe - p.e;
+    return p.adapt_min_len < 0 && !p.bound_pass && p.e == 1 && O >= 1 && O <= kMhDepth && p.x <= kMhDepth &&
+           max_length <= kMaxWfaLength16 && ring_width(p, max_length) < 32768 && p.smax < (1 << 20);
+}
+
+bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_bytes) {
+    return G <= 32 && ring_ok(p, max_length) && kWarpsPerBlock * ring_smem_per_warp(p, G, max_length) <= kMaxSmem &&
+           kWarpsPerBlock * ring_warp_bytes(p, G, max_length) <= scratch_bytes;
+}
+
+int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes) {
+    int G = 1;
+    while (G < 32 && (ring_smem_per_warp(p, G, max_length) > kGoodSmem ||
+                      (uint64_t)num_pairs * G < (uint64_t)num_sms * kGoodWarps * 32))
+        G *= 2;
+    while (G <= 32 && !ring_fits(p, G, max_length, scratch_bytes)) G *= 2;
+    return G <= 32 ? G : 0;
+}
+
+cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, const LimitView& L, const OutView& O,
+                            const uint32_t* order, const uint32_t* bounds, uint8_t* scratch, size_t scratch_bytes,
+                            uint32_t* counters, int num_sms, cudaStream_t st, int* warps_used) {
+    *warps_used = 0;
+    if (P.num_pairs == 0) return cudaSuccess;
+    RingArgs r{};
+    WfaArgs& a = r.w;
+    a.X = plan.x; a.OE = plan.oe; a.E = plan.e; a.g = plan.g; a.smax = plan.smax; a.band = plan.band;
+    a.P = P; a.L = L; a.O = O;
+    a.scratch = scratch;
+    a.runs_bytes = plan.runs_bytes; a.runs_cap = (uint32_t)plan.runs_cap;
+    a.order = order; a.bounds = bounds; a.counters = counters; a.nbuckets = 1;
+    a.bound = plan.bound; a.retry_only = plan.retry_only;
+    const uint32_t len = P.max_length;
+    const size_t e_bytes = entry_bytes(len);
+    r.width = (uint32_t)ring_width(plan, len);
+    r.seq_words = seq_words(len);
+    r.smem_warp = (uint32_t)ring_smem_per_warp(plan, G, len);
+    r.seq_rounds = seq_bytes(len, 32) <= kKeepBytes ? (uint32_t)G : 1u;
+    r.stage_shared = (size_t)plan.runs_cap * 33 * 4 <= (size_t)r.width * (32 / G) * (8 + (G == 1 ? 4 : 8));
+    const size_t min_warp = ring_warp_bytes(plan, G, len);
+    r.round_bytes = min_warp - 32 * plan.runs_bytes;
+    // value d scores back: bytes 2 (d - 1) and 2 (d - 1) + 1 of mh, the sign replicated above them
+    auto sel = [](int d) { const uint32_t b = 2u * (uint32_t)(d - 1); return b | ((b + 1) << 4) | ((b + 9) << 8) | ((b + 9) << 12); };
+    r.sel_x = sel(plan.x);
+    r.sel_o = sel(plan.oe - plan.e);
+    void (*kernel)(RingArgs) = e_bytes == 4 ? ring_kernel_for<uint32_t>(G) : ring_kernel_for<uint64_t>(G);
+    const size_t smem = (size_t)kWarpsPerBlock * r.smem_warp;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    if (e != cudaSuccess) return e;
+    int bps = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, 32 * kWarpsPerBlock, smem);
+    if (e != cudaSuccess) return e;
+    if (bps < 1) return cudaSuccess;
+    size_t warps = (size_t)num_sms * bps * kWarpsPerBlock;
+    warps = std::min(warps, scratch_bytes / min_warp);
+    if (!bounds) warps = std::min(warps, ((size_t)P.num_pairs * G + 31) / 32);
+    if (warps == 0) return cudaSuccess;
+    a.nwarps = (uint32_t)warps;
+    // a warp's arena: its share of the scratch, up to G worst-case rounds
+    a.warp_bytes = std::min(scratch_bytes / warps & ~(size_t)255, min_warp + (size_t)(G - 1) * r.round_bytes);
+    kernel<<<(unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock), 32 * kWarpsPerBlock, smem, st>>>(r);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) *warps_used = (int)warps;
+    return e;
+}
+
+}  // namespace aim

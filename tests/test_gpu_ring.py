@@ -1,0 +1,75 @@
+"""The shared-memory wavefront form (wfa_ring.cu) against the oracle, for every number of lanes per pair: at lengths
+around a packed word and around the 10-bit history's limit, at thresholds of one gap up to wide windows, with a band,
+with thresholds that differ from pair to pair, and over end diagonals far from 0."""
+import numpy as np
+import pytest
+
+import gen
+from devutil import assert_same, device_results, oracle_results
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def aligner():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2208_01243_gb300 as aim
+    al = aim.Aligner(0, 256 << 20)
+    yield al
+    al.close()
+
+
+def _mixed(lengths, seed):
+    """Related pairs, unrelated pairs and pairs whose targets are cut short or run on, at each length."""
+    rng = np.random.default_rng(seed)
+    reads, targets = [], []
+    for n in lengths:
+        for rate in (0.0, 0.03, 0.1, 1.0):
+            r = rng.integers(0, 4, n)
+            t = []
+            for b in r:
+                u = rng.random()
+                if u < rate / 3:
+                    t += [(b + rng.integers(1, 4)) % 4]
+                elif u < 2 * rate / 3:
+                    t += [rng.integers(0, 4), b]
+                elif u >= rate or rate == 0.0:
+                    t += [b]
+            for cut in (0, 1, 7):
+                reads.append(bytes(b"ACGT"[x] for x in r))
+                targets.append(bytes(b"ACGT"[x] for x in t[cut:]))
+            reads.append(bytes(b"ACGT"[x] for x in r[: n - n // 8]))
+            targets.append(bytes(b"ACGT"[x] for x in t))
+    return gen.from_strings(reads, targets)
+
+
+@pytest.mark.parametrize("lanes", [1, 2, 4, 8, 16, 32])
+@pytest.mark.parametrize("penalties,max_edits,band", [((0, 4, 6, 2), 6, -1), ((0, 3, 4, 1), 8, -1),
+                                                      ((0, 4, 6, 2), 1, -1), ((0, 2, 3, 1), 12, 5),
+                                                      ((0, 4, 4, 4), 9, 0), ((0, 4, 6, 2), 20, 15)])
+def test_ring_matches_oracle(aligner, lanes, penalties, max_edits, band):
+    import paper_2208_01243_gb300 as aim
+    lengths = [1, 15, 16, 17, 31, 32, 33, 63, 64, 97, 150] if max_edits < 20 else [64, 250, 300]
+    p = _mixed(lengths, 7 * lanes + max_edits)
+    per_pair = np.random.default_rng(lanes).integers(0, max_edits + 1, len(p)).astype(np.int32)
+    per_pair[::3] = max_edits
+    x, o, e = penalties[1:]
+    lim = per_pair.astype(np.int64) * max(x, o + e)
+    aim.aim_set_wfa_group(aligner.ctx, lanes)
+    try:
+        dev = device_results(p, "wfa", penalties, max_edits, per_pair=per_pair, band=band, aligner=aligner)
+    finally:
+        aim.aim_set_wfa_group(aligner.ctx, 0)
+    assert_same(dev, oracle_results(p, penalties, lim, band=band), what=f"ring, {lanes} lanes")
+
+
+@pytest.mark.parametrize("length", [1000, 1022, 1023, 1500])
+def test_ring_at_the_narrow_history_limit(aligner, length):
+    """max_length up to 1,022 keeps 10-bit history fields, beyond it 16-bit ones."""
+    w = gen.Workload("ring_edge", 91, 40, length, length, 0.01, 0.01, 0.2, "wfa", (0, 4, 6, 2), 15)
+    p = gen.generate(w)
+    keep = p.target_len <= length
+    p = gen.from_strings([p.read(i) for i in np.nonzero(keep)[0]], [p.target(i) for i in np.nonzero(keep)[0]])
+    dev = device_results(p, "wfa", w.penalties, 15, max_length=length, aligner=aligner)
+    assert_same(dev, oracle_results(p, w.penalties, np.full(len(p), 120, np.int64)), what=f"ring, {length} bp")
