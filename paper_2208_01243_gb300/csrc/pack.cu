@@ -1,139 +1,174 @@
-// 2-bit packer: ASCII A/C/G/T -> 0/1/2/3, first base in the top two bits of each 64-bit word.
+// 2-bit packer: ASCII A/C/G/T -> 0/1/2/3, first base in the top two bits of each 64-bit word; sequences at any byte
+// offset, word offsets given or i * stride.
 //
-// Fixed slots (every sequence at word i * stride, the form the ASCII entry points use): one thread per output
-// word.  It reads the word's 32 bytes as aligned 4-byte loads (each load holds at least one byte of the word, so
-// none crosses into another page), lines them up with funnel shifts, and converts four bytes at a time:
-// ((c >> 1) ^ (c >> 2)) & 3 maps A, C, G, T (0x41, 0x43, 0x47, 0x54) to 0, 1, 2, 3; a byte whose code's letter
-// (looked up for four bytes by one byte permute) is not the byte itself flags the pair; one multiply gathers the
-// four 2-bit codes into a byte, first base on top.  The slot of a thread comes from a multiply, not a division.
+// A warp takes a batch of up to 32 sequences, one per lane for their offsets and lengths, and walks the words of all
+// of them as one list, a word per lane whatever the sequences' lengths (a scan over the batch gives each sequence's
+// place, five shuffles find a word's sequence), so lanes stay busy over uneven reads and the offsets are read once,
+// coalesced.  A lane reads its word's 32 bytes as two aligned 16-byte chunks, converts them as they lie (bytes outside
+// the sequence read as 'A', code 0), takes the code bits of the next chunk from the next lane, and shifts the 96 bits
+// by the sequence's offset inside its first chunk: the alignment costs two funnel shifts on codes instead of eight on
+// bytes and nine 4-byte loads.  Each sequence has one item more than words, which only supplies that next chunk.
+// Every chunk read holds a byte of its sequence, so no read crosses into another page.
 //
-// Explicit word offsets (aim_pack_2bit): one warp per sequence; each lane converts one byte per 32-base word
-// and the warp ORs the lanes' 2-bit codes together (two 32-bit halves).  Lane w%32 keeps word w and the warp
-// stores 32 words at a time with one coalesced store.
-#include <type_traits>
+// (c >> 1) & 3 maps A, C, T, G (0x41, 0x43, 0x54, 0x47) to 0, 1, 2, 3; a byte is one of the four exactly when it equals
+// "ACTG" at that value, looked up for four bytes by one byte permute; one multiply lines the values up as the permute's
+// selector, another gathers them into a byte, and one XOR over 16 bases turns 2 and 3 into the codes of T and G.
+// Bytes next to a sequence are converted like its own: the shift drops those before it and a mask those after it;
+// only a chunk that shows a byte other than the four is looked at again, with the bytes outside the sequence masked.
+//
+// What bounds it: the latency of the 16-byte loads and the integer pipe (58 % busy) about evenly; 40 registers, for 48
+// warps on an SM, measured better than more registers or loads issued a turn ahead (136 us with 55 registers, 132 us
+// with the loads ahead).  1M sequences of 100-1,000 bp (391 MB) in 123 us, 4.2 TB/s of 6.8, from 901 us with a warp
+// per sequence and a byte per lane; 1M of 150 bp 62 us (from 392 us; a thread per word in fixed slots 63 us, and 105
+// us over uneven lengths against 54 us here).
+#include <algorithm>
 
 #include "aim_internal.cuh"
 
 namespace aim {
 namespace {
 
-__device__ __forceinline__ uint32_t ascii_code(uint32_t c, bool& ok) {
-    // A 0x41, C 0x43, G 0x47, T 0x54
-    uint32_t code = (c == 'C') ? 1u : (c == 'G') ? 2u : (c == 'T') ? 3u : 0u;
-    ok = (c == 'A') | (c == 'C') | (c == 'G') | (c == 'T');
-    return code;
+constexpr int kPackWarps = 8;   // per block
+
+// four bytes (first in the low byte) -> (c >> 1) & 3 of each, the first's in the top two bits of the top byte; diff
+// collects bytes that are none of the four letters
+__device__ __forceinline__ uint32_t gather4(uint32_t x, uint32_t& diff) {
+    const uint32_t y = (x >> 1) & 0x03030303u;
+    const uint32_t sel = __byte_perm(y * 0x110u, 0u, 0x4431u);   // y_0 | y_1 << 4 in byte 1 of the product, y_2, y_3 in 3
+    diff |= __byte_perm(0x47544341u, 0u, sel) ^ x;                // "ACTG"[y_k] against the byte
+    return y * 0x40100401u;   // 2^30 + 2^20 + 2^10 + 1: no carries into the top byte
 }
 
-__global__ void __launch_bounds__(256) pack_kernel(const uint8_t* __restrict__ ascii,
-                                                   const uint64_t* __restrict__ char_off,
-                                                   const uint32_t* __restrict__ len, uint32_t count,
-                                                   uint64_t* __restrict__ packed,
-                                                   const uint64_t* __restrict__ word_off, uint64_t word_stride,
-                                                   uint8_t* __restrict__ bad) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t i = warp; i < count; i += nwarps) {
-        const uint8_t* s = ascii + __ldg(char_off + i);
-        const uint32_t L = __ldg(len + i);
-        uint64_t* out = packed + (word_off ? __ldg(word_off + i) : (uint64_t)i * word_stride);
-        const uint32_t nw = (L + 31) >> 5;
-        if (!word_off && nw > word_stride) {   // longer than the fixed per-sequence slot: flag, write nothing
-            if (bad && lane == 0) bad[i] = 1;
-            continue;
-        }
-        bool any_bad = false;
-        uint64_t mine = 0;
-        for (uint32_t w = 0; w < nw; ++w) {
-            const uint32_t pos = (w << 5) + lane;
-            uint32_t code = 0;
-            if (pos < L) {
-                bool ok;
-                code = ascii_code(__ldg(s + pos), ok);
-                any_bad |= !ok;
-            }
-            const uint32_t hi = __reduce_or_sync(0xffffffffu, lane < 16 ? code << (30 - 2 * lane) : 0u);
-            const uint32_t lo = __reduce_or_sync(0xffffffffu, lane >= 16 ? code << (30 - 2 * (lane - 16)) : 0u);
-            if (lane == (w & 31)) mine = ((uint64_t)hi << 32) | lo;
-            if ((w & 31) == 31 || w + 1 == nw) {
-                const uint32_t first = w & ~31u;
-                if (first + lane <= w) out[first + lane] = mine;
-            }
-        }
-        const bool b = __any_sync(0xffffffffu, any_bad);
-        if (bad && lane == 0) bad[i] = b ? 1 : 0;
+// 16 bytes -> 32 bits, first base on top; values of (c >> 1) & 3 (codes_of makes them codes)
+__device__ __forceinline__ uint32_t gather16(uint4 u, uint32_t& diff) {
+    const uint32_t a = gather4(u.x, diff), b = gather4(u.y, diff), c = gather4(u.z, diff), d = gather4(u.w, diff);
+    return __byte_perm(__byte_perm(d, c, 0x0073u), __byte_perm(b, a, 0x0073u), 0x5410u);
+}
+__device__ __forceinline__ uint32_t codes_of(uint32_t z) { return z ^ ((z >> 1) & 0x55555555u); }
+
+// the bytes of x that are A, C, G or T; the others as 'A'
+__device__ __forceinline__ uint32_t letters_only(uint32_t x) {
+    uint32_t r = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t c = (x >> (8 * k)) & 0xffu;
+        r |= (c == 'C' || c == 'G' || c == 'T' ? c : (uint32_t)'A') << (8 * k);
     }
+    return r;
 }
 
-// four ASCII bytes (first in the low byte) -> their 2-bit codes, first base in bits 7..6; *bad: a byte in `keep`
-// (0xff per byte to look at) that is not A, C, G or T.  Every byte c gets the code ((c >> 1) ^ (c >> 2)) & 3,
-// and c is one of the four letters exactly when it equals the letter of its code, "ACGT"[code]: one byte
-// permute looks the four letters up, with the codes as its selector nibbles.
-__device__ __forceinline__ uint32_t pack4(uint32_t x, uint32_t keep, bool& bad) {
-    const uint32_t codes = ((x >> 1) ^ (x >> 2)) & 0x03030303u;   // byte k: code of byte k
-    const uint32_t pairs = codes | (codes >> 4);                   // byte 0: c0 | c1 << 4; byte 2: c2 | c3 << 4
-    const uint32_t sel = __byte_perm(pairs, 0u, 0x4420u);          // nibble k: c_k
-    const uint32_t letters = __byte_perm(0x54474341u, 0u, sel);    // byte k: "ACGT"[c_k]
-    bad |= ((letters ^ x) & keep) != 0;
-    // byte k holds code k; times 2^30 + 2^20 + 2^10 + 1 puts code k at bits 30-2k..31-2k with no carries
-    return ((codes & keep) * 0x40100401u) >> 24;
+// a chunk that showed some other byte: the bytes outside the sequence (not in m) count as 'A'; any left inside is
+// bad, code 0
+__device__ __noinline__ uint32_t gather16_checked(uint4 u, uint4 m, bool& bad) {
+    auto keep = [](uint32_t k, uint32_t x) { return (x & k) | (0x41414141u & ~k); };
+    u = make_uint4(keep(m.x, u.x), keep(m.y, u.y), keep(m.z, u.z), keep(m.w, u.w));
+    uint32_t diff = 0;
+    uint32_t z = gather16(u, diff);
+    if (diff) {
+        bad = true;
+        z = gather16(make_uint4(letters_only(u.x), letters_only(u.y), letters_only(u.z), letters_only(u.w)), diff);
+    }
+    return z;
 }
 
-// g / d for any 32-bit g, by a multiply: with s = ceil(log2 d) and M = ceil(2^(32+s) / d) = 2^32 + m (d <= 2^s
-// puts M in [2^32, 2^33)), g * M / 2^(32+s) = g / d + g (M d - 2^(32+s)) / (d 2^(32+s)), and the second term
-// is below 1 / d since M d - 2^(32+s) < d <= 2^s and g < 2^32: its floor is g / d rounded down.
-struct Divider {
-    uint32_t m, s;
-    __device__ uint32_t div(uint32_t g) const { return (uint32_t)(((uint64_t)__umulhi(g, m) + g) >> s); }
-};
-
-Divider make_divider(uint32_t d) {   // 1 <= d <= 2^31
-    uint32_t s = 0;
-    while (((uint64_t)1 << s) < d) ++s;
-    const uint64_t M = (((uint64_t)1 << (32 + s)) + d - 1) / d;
-    return Divider{(uint32_t)(M - ((uint64_t)1 << 32)), s};
+__device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t s) {   // 0 for s >= 32
+    uint32_t r;
+    asm("shr.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));
+    return r;
 }
 
-template <bool WIDE>
-__global__ void __launch_bounds__(256) pack_words_kernel(const uint8_t* __restrict__ ascii,
-                                                         const uint64_t* __restrict__ char_off,
-                                                         const uint32_t* __restrict__ len, uint32_t count,
-                                                         uint64_t* __restrict__ packed, uint32_t stride,
-                                                         Divider by_stride, uint8_t* __restrict__ bad) {
-    using Index = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
-    const Index total = (Index)count * stride;
-    for (Index g = (Index)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += (Index)gridDim.x * blockDim.x) {
-        const uint32_t i = WIDE ? (uint32_t)(g / stride) : by_stride.div((uint32_t)g);
-        const uint32_t w = (uint32_t)(g - (Index)i * stride);
-        const uint32_t L = __ldg(len + i);
-        const uint32_t nw = (L + 31) >> 5;
-        if (nw > stride) {   // longer than the fixed per-sequence slot: flag, write nothing
-            if (bad && w == 0) bad[i] = 1;
-            continue;
+// parts: warps that share a batch (word lists of few, long sequences), each taking every parts-th turn; then `bad` is
+// zero at launch
+__global__ void __launch_bounds__(32 * kPackWarps, 6) pack_kernel(const uint8_t* __restrict__ ascii,
+                                                               const uint64_t* __restrict__ char_off,
+                                                               const uint32_t* __restrict__ len, uint32_t count,
+                                                               uint32_t batch, uint32_t parts,
+                                                               uint64_t* __restrict__ packed,
+                                                               const uint64_t* __restrict__ word_off,
+                                                               uint64_t word_stride, uint8_t* __restrict__ bad) {
+    __shared__ uint4 s_first[17];   // [h]: ones in the first h bytes of a chunk
+    if (threadIdx.x < 17) {
+        auto word = [&](int q) -> uint32_t {
+            const int h = (int)threadIdx.x - 4 * q;
+            return h >= 4 ? 0xffffffffu : h <= 0 ? 0u : (1u << (8 * h)) - 1u;
+        };
+        s_first[threadIdx.x] = make_uint4(word(0), word(1), word(2), word(3));
+    }
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint64_t nbatches = (count + batch - 1) / batch;
+    for (uint64_t work = warp; work < nbatches * parts; work += nwarps) {
+        const uint32_t first = (uint32_t)(work / parts) * batch, part = (uint32_t)(work % parts);
+        // this lane's sequence
+        const bool have = lane < batch && lane < count - first;
+        uint32_t L = 0, items = 0;
+        uint64_t from = 0, to = 0;
+        if (have) {
+            const uint32_t i = first + lane;
+            L = __ldg(len + i);
+            from = reinterpret_cast<uint64_t>(ascii) + __ldg(char_off + i);
+            to = word_off ? __ldg(word_off + i) : i * word_stride;
+            const uint32_t nw = (L + 31) >> 5;
+            const bool fits = word_off || nw <= word_stride;   // longer than the fixed slot: flag, write nothing
+            items = fits && nw ? nw + 1 : 0;
+            if (bad && part == 0) {
+                if (!fits) bad[i] = 1;
+                else if (parts == 1) bad[i] = 0;
+            }
         }
-        if (w >= nw) continue;
-        // first byte of this word; alignment is taken from the address itself (the buffer may start anywhere)
-        const uintptr_t at = reinterpret_cast<uintptr_t>(ascii) + __ldg(char_off + i) + 32ull * w;
-        const uint32_t nb = min(32u, L - 32u * w);              // bytes of this word
-        const uint32_t* base = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
-        const uint32_t sh = 8u * (uint32_t)(at & 3);
-        const uint32_t last = (uint32_t)(((at & 3) + nb - 1) >> 2);     // last aligned word holding a byte
-        uint32_t u[9];
+        __syncwarp();   // bad[] starts at 0 before any lane sets it
+        // all sequences at once, or one by one where the list's length might leave 32 bits (over 2 G bases in one)
+        const bool huge = __any_sync(kFull, items > (1u << 26));
+        for (uint32_t todo = __ballot_sync(kFull, items != 0); todo;) {
+            const uint32_t take = huge ? todo & (0u - todo) : todo;
+            todo &= ~take;
+            const uint32_t mine = (take >> lane) & 1u ? items : 0u;
+            uint32_t upto = mine;   // items of this and the sequences before it
 #pragma unroll
-        for (int q = 0; q < 9; ++q) u[q] = (uint32_t)q <= last ? __ldg(base + q) : 0u;
-        bool b = false;
-        uint32_t hi = 0, lo = 0;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, upto, o);
+                if ((int)lane >= o) upto += t;
+            }
+            const uint32_t total = __shfl_sync(kFull, upto, 31);
+            const uint32_t before = upto - mine;
+            // 31 items a turn; lane 31 only supplies the next chunk to lane 30
+            for (uint32_t base = 31 * part; base < total; base += 31 * parts) {
+                const uint32_t it = base + lane;
+                uint32_t s = 0;   // sequences whose items all come before this one
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const uint32_t x = __funnelshift_r(u[q], u[q + 1], sh);
-            const int have = (int)nb - 4 * q;                       // bytes of this group inside the word
-            const uint32_t keep = have >= 4 ? 0xffffffffu : have <= 0 ? 0u : ((1u << (8 * have)) - 1u);
-            const uint32_t byte = pack4(x, keep, b);
-            if (q < 4) hi |= byte << (24 - 8 * q);
-            else lo |= byte << (24 - 8 * (q - 4));
+                for (int step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(kFull, upto, (int)(s + step - 1)) <= it) s += step;
+                const uint32_t sL = __shfl_sync(kFull, L, s), w = it - __shfl_sync(kFull, before, s);
+                const uint64_t sfrom = __shfl_sync(kFull, from, s), sto = __shfl_sync(kFull, to, s);
+                const uint32_t phase = (uint32_t)sfrom & 15u, nw = (sL + 31) >> 5;
+                // the sequence's bytes from this item's chunks on, counted from the chunk's start
+                const int left = it >= total ? 0 : w + 2 < nw ? 64 : (int)(sL - 32 * w) + (int)phase;
+                const uint4* src = reinterpret_cast<const uint4*>(sfrom & ~15ull) + 2ull * w;
+                uint4 u0 = make_uint4(0x41414141u, 0x41414141u, 0x41414141u, 0x41414141u), u1 = u0;
+                if (left > 0) u0 = __ldg(src);
+                if (left > 16) u1 = __ldg(src + 1);
+                bool b = false;
+                uint32_t d0 = 0, d1 = 0;
+                uint32_t z0 = gather16(u0, d0), z1 = gather16(u1, d1);
+                if (d0 | d1) {
+                    uint4 m = s_first[min(max(left, 0), 16)];
+                    const uint4 l = s_first[w == 0 ? phase : 0u];
+                    m = make_uint4(m.x & ~l.x, m.y & ~l.y, m.z & ~l.z, m.w & ~l.w);
+                    z0 = gather16_checked(u0, m, b);
+                    z1 = gather16_checked(u1, s_first[min(max(left - 16, 0), 16)], b);
+                }
+                const uint32_t z2 = __shfl_down_sync(kFull, z0, 1);
+                if (lane < 31 && it < total && w < nw) {
+                    const uint32_t nb = min(sL - 32 * w, 32u);   // bases of this word
+                    const uint32_t hi = codes_of(__funnelshift_l(z1, z0, 2 * phase)) & ~shr_clamp(~0u, 2 * nb);
+                    const uint32_t lo = codes_of(__funnelshift_l(z2, z1, 2 * phase)) &
+                                        ~shr_clamp(~0u, 2 * max(nb, 16u) - 32);
+                    packed[sto + w] = ((uint64_t)hi << 32) | lo;
+                }
+                if (bad && b) bad[first + s] = 1;
+            }
         }
-        packed[g] = ((uint64_t)hi << 32) | lo;
-        if (bad && b) bad[i] = 1;
     }
 }
 
@@ -146,32 +181,20 @@ cudaError_t launch_pack(const uint8_t* ascii, const uint64_t* char_off, const ui
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (!word_off && word_stride > 0 && word_stride <= 0xffffffffull) {
-        // fixed slots: one thread per word; bad flags start at 0 and threads that see a bad byte set them
-        if (bad) {
-            const cudaError_t e = cudaMemsetAsync(bad, 0, count, st);
-            if (e != cudaSuccess) return e;
-        }
-        const uint64_t total = (uint64_t)count * word_stride;
-        uint64_t blocks = (total + 255) / 256;
-        const uint64_t cap = (uint64_t)sms * 32;   // grid-stride beyond 32 blocks of 256 per SM
-        if (blocks > cap) blocks = cap;
-        // the reciprocal needs 2^(32+s) in 64 bits (a stride up to 2^31); anything wider divides
-        const bool narrow = total <= 0xffffffffull && word_stride <= ((uint64_t)1 << 31);
-        const Divider by_stride = narrow ? make_divider((uint32_t)word_stride) : Divider{0u, 0u};
-        if (narrow)
-            pack_words_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(ascii, char_off, len, count, packed,
-                                                                        (uint32_t)word_stride, by_stride, bad);
-        else
-            pack_words_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(ascii, char_off, len, count, packed,
-                                                                       (uint32_t)word_stride, by_stride, bad);
-        return cudaGetLastError();
+    // batches of up to 32 sequences, smaller (and then shared by several warps) while that leaves SMs without 16 warps
+    const uint32_t want = (uint32_t)sms * 16;
+    uint32_t batch = 32, parts = 1;
+    while (batch > 1 && (count + batch - 1) / batch < want) batch /= 2;
+    const uint32_t batches = (count + batch - 1) / batch;
+    while (parts < 16 && batches * parts < want / 2) parts *= 2;
+    if (bad && parts > 1) {
+        const cudaError_t e = cudaMemsetAsync(bad, 0, count, st);
+        if (e != cudaSuccess) return e;
     }
-    const uint32_t warps_needed = count;
-    uint32_t blocks = (warps_needed + 7) / 8;
-    const uint32_t cap = (uint32_t)sms * 8;   // 8 blocks of 8 warps per SM, grid-stride beyond that
-    if (blocks > cap) blocks = cap;
-    pack_kernel<<<blocks, 256, 0, st>>>(ascii, char_off, len, count, packed, word_off, word_stride, bad);
+    const uint64_t warps = (uint64_t)batches * parts;
+    const uint64_t blocks = std::min<uint64_t>((warps + kPackWarps - 1) / kPackWarps, (uint64_t)sms * 32);
+    pack_kernel<<<(unsigned)blocks, 32 * kPackWarps, 0, st>>>(ascii, char_off, len, count, batch, parts, packed, word_off,
+                                                             word_stride, bad);
     return cudaGetLastError();
 }
 
