@@ -147,6 +147,9 @@ struct WfaPlan {
                          // exact launches take min(limit, bound) as the pair's limit when set (null: none)
     int bound_pass;      // the launch is a bound pass: pruned, no history, no traceback; writes bound
     int bound_min_len, bound_max_dist;   // the bound pass's pruning (as adapt_min_len, adapt_max_dist)
+    int64_t ring_diagonals, ring_scores; // wfa_ring.cu: no pair of the launch has a window of more diagonals, or a
+                                         // larger scaled limit, than these (0: only what smax, the band and the
+                                         // lengths say)
 };
 // the bound pass's pruning: wavefronts of at least kBoundMinLen diagonals keep those within kBoundMaxDist of the
 // diagonal closest to the end
@@ -214,7 +217,7 @@ cudaError_t launch_wfa(const WfaPlan& plan, int group, const PairsView& P, const
                        int* warps_used);
 
 // the form of wfa_ring.cu (state in shared memory): whether the costs and lengths allow it, whether a launch with G
-// lanes per pair (1..32) fits shared memory and the scratch, the lanes suited to a batch (0: does not fit), one launch
+// lanes per pair (1..32, 256: a block) fits shared memory and the scratch, the lanes suited to a batch (0: does not fit), one launch
 // over all pairs, or over the queue range bounds[0..1] of order
 bool ring_ok(const WfaPlan& p, uint32_t max_length);
 bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_bytes);

@@ -46,6 +46,7 @@
 // entry on an optimal path survive the clamp), so the tuner may add a bound
 // pass to any bucket it makes faster.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -168,6 +169,22 @@ size_t bucket_pair_bytes(const WfaPlan& plan, int b, int G) {
     return wfa_pair_bytes_capped(plan, G, hist);
 }
 
+// the plan with what bucket b says of its pairs for wfa_ring.cu.  With C = (S + 1) W < 2^(3 (kc + 1)) and the window at
+// most W: W is at most 64 / 128 / 256 in the narrower width classes, and at most sqrt(2 C) + 1 in the widest (W <= 2 S + 3
+// there, so C >= W (W - 1) / 2); S + 1 is C over the class's least W.
+WfaPlan bucket_plan(const WfaPlan& plan, int b) {
+    const int kc = kWorkClasses - 1 - b / kWidthClasses;
+    const int wc = kWidthClasses - 1 - b % kWidthClasses;
+    WfaPlan p = plan;
+    const int64_t cmax = ((int64_t)1 << (3 * (kc + 1))) - 2;
+    if (wc < kWidthClasses - 1) p.ring_diagonals = (int64_t)64 << wc;
+    else if (kc < kWorkClasses - 1) p.ring_diagonals = (int64_t)std::sqrt(2.0 * (double)cmax) + 2;
+    const int64_t wmin = wc == 0 ? 1 : ((int64_t)32 << wc) + 1;
+    // (E > 1 only narrows W for the same S; wfa_ring.cu needs E == 1)
+    if (kc < kWorkClasses - 1) p.ring_scores = std::max<int64_t>(cmax / wmin, 1);
+    return p;
+}
+
 constexpr int kCompactDiagonalsPerLane = 16;   // first-pass history: wavefronts of about 16 diagonals per lane
 constexpr int kBoundDefaultGroup = 4;          // lanes per pair of a forced bound pass
 constexpr float kBoundGain = 0.97f;            // a bound pass must save at least 3 % of the bucket's trial time
@@ -220,6 +237,7 @@ struct aim_batch {
     int ggroup[aim::kBuckets];          // lanes per pair of each group
     int gbound[aim::kBuckets];          // lanes per pair of each group's bound pass (0: none)
     size_t gwarp_bytes[aim::kBuckets];  // scratch per warp of each group
+    int64_t gdiagonals[aim::kBuckets], gscores[aim::kBuckets];   // each group's widest window and largest limit
     uint32_t host_counts[aim::kBuckets];
     aim::BucketParams bp;
     cudaStream_t stream;
@@ -271,6 +289,8 @@ cudaError_t enqueue_align(aim_batch* b, cudaStream_t st, int* warps) {
         for (int j = 0; j < b->bp.ngroups; ++j) {
             int w = 0;
             WfaPlan exact = b->plan;
+            exact.ring_diagonals = b->gdiagonals[j];
+            exact.ring_scores = b->gscores[j];
             if (b->gbound[j]) {
                 WfaPlan bp = b->plan;
                 bp.bound = b->bound;
@@ -362,6 +382,7 @@ int autotune(aim_batch* b) {
         const uint32_t tb[2] = {bounds[k], bounds[k] + sample};
         float best = 1e30f;
         int best_g = b->groups[k];
+        const WfaPlan exact = bucket_plan(b->plan, k);
         // lanes per pair worth trying for this width class: at most ~64 diagonals per lane and score step
         const int wc = kWidthClasses - 1 - k % kWidthClasses;
         const int gmin = wc == 0 ? 1 : wc == 1 ? 2 : wc == 2 ? 4 : 8;
@@ -371,7 +392,7 @@ int autotune(aim_batch* b) {
             const size_t wb = wfa_warp_bytes(G, bucket_pair_bytes(b->plan, k, G));
             if (wb * min_warps > b->scratch_bytes) continue;
             float ms = 0.f;
-            for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) e = trial(b, b->plan, tb, G, wb, t0, t1, &ms);
+            for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) e = trial(b, exact, tb, G, wb, t0, t1, &ms);
             if (e == cudaSuccess && ms < best) { best = ms; best_g = G; }
         }
         // compact first pass with fewer lanes, then the full-scratch pass over the pairs that outgrew it
@@ -393,7 +414,7 @@ int autotune(aim_batch* b) {
         // a bound pass, then the exact pass clamped at each pair's bound (only where no compact pass was chosen)
         int best_gb = 0;
         if (best_g1 == 0 && b->ctx->batch_bound != 2 && b->max_length <= kMaxWfaLength16) {
-            WfaPlan bp = b->plan, ep = b->plan;
+            WfaPlan bp = b->plan, ep = exact;
             bp.bound = ep.bound = b->bound;
             bp.bound_pass = 1;
             const size_t wb_full = wfa_warp_bytes(best_g, bucket_pair_bytes(b->plan, k, best_g));
@@ -578,10 +599,16 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
         int next = 0;
         for (int j = 0; j < ng; ++j) {
             b->bp.gstart[j] = (int8_t)next;
+            b->gdiagonals[j] = b->gscores[j] = 1;
             size_t wbj = 16;
             for (int k = 0; k < kBuckets; ++k) {
                 if (b->groups[k] != b->ggroup[j] || b->bound1[k] != b->gbound[j]) continue;
                 b->bp.perm[k] = (int8_t)next++;
+                // (a replay may put pairs into any bucket of the group; 0 is "no bound of its own")
+                const WfaPlan bk = bucket_plan(b->plan, k);
+                auto widen = [](int64_t& all, int64_t one) { all = all && one ? std::max(all, one) : 0; };
+                widen(b->gdiagonals[j], bk.ring_diagonals);
+                widen(b->gscores[j], bk.ring_scores);
                 wbj = std::max(wbj, wfa_warp_bytes(b->groups[k], bucket_pair_bytes(b->plan, k, b->groups[k])));
             }
             b->gwarp_bytes[j] = wbj;

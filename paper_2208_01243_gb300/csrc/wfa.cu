@@ -1246,6 +1246,7 @@ WfaPlan plan_wfa(const Costs& c, int band, uint32_t max_length, int64_t max_limi
     p.bound_pass = 0;
     p.bound_min_len = kBoundMinLen;
     p.bound_max_dist = kBoundMaxDist;
+    p.ring_diagonals = p.ring_scores = 0;
     return p;
 }
 
@@ -1295,6 +1296,13 @@ cudaError_t launch_wfa_buckets(const WfaPlan& plan, const PairsView& P, const Li
     *warps_used = 0;
     if (P.num_pairs == 0) return cudaSuccess;
     if (nbuckets < 1 || nbuckets > kMaxBuckets) return cudaErrorInvalidValue;
+    // one queue of an exact pass: the form with its state in shared memory, where the costs and widths allow it
+    if (nbuckets == 1 && !plan.bound_pass) {
+        const int G = groups[0] > 32 ? 256 : groups[0];
+        if (ring_fits(plan, G, P.max_length, scratch_bytes))
+            return launch_wfa_ring(plan, G, P, L, O, order, bounds, scratch, scratch_bytes, counters, num_sms, st,
+                                   warps_used);
+    }
     WfaArgs a;
     a.X = plan.x; a.OE = plan.oe; a.E = plan.e; a.g = plan.g; a.smax = plan.smax; a.band = plan.band;
     a.P = P; a.L = L; a.O = O;

@@ -20,10 +20,12 @@
 // no alignment of cost <= S, and the traceback reads entries on optimal paths only.  Every pair walks its own row; the
 // warp walks as many entries as its widest row.  The positions just outside a row read as invalid in the next one.
 //
-// History for the traceback: row s is one run of entries in the warp's scratch, written 32 consecutive entries at a
-// time, at a fixed distance from the row before: (M~, I~, D~) + 1 in 10 bits each for reads up to 1,022 bp, three
-// 16-bit values beyond.  A round of P pairs leaves its history in the warp's arena; after G rounds (or when the
-// arena may not hold another) the 32 lanes trace back one pair each, by the tests of wfa.cu.
+// History for the traceback, written 32 (or G) consecutive entries at a time.  Reads up to 1,022 bp: M~, I~ and D~,
+// each + 1 in 10 bits of a word.  Longer ones: M~ + 1 and two source bits in 16 bits (up to 16,382 bp) or 32, set when
+// J or K came from the extension (I~ > M~[s-O], D~ > M~[s-O]); the traceback follows them back to the gap's opening.
+// Row s starts at a fixed distance from row s-1, or, for a longer read alone in its unit, where row s-1 ends, and the
+// traceback computes where that is (RowMap).  A round of P pairs leaves its history in its unit's arena; after
+// 32 pairs (or when the arena may not hold another round) a lane each traces them back, by the tests of wfa.cu.
 //
 // What bounds it: instruction issue.  1M pairs of 150 bp at 6 edits take 900 warp instructions a pair at 2.7 per
 // cycle (wfa.cu's 4-lane groups: 1,790 at 2.2), 1.03 ms against 2.43 ms; 250 bp, band 25, 25 edits 9.6 ms against
@@ -58,29 +60,33 @@ __device__ __forceinline__ int prmt(uint32_t a, uint32_t b, uint32_t sel) {   //
     return (int)r;
 }
 
-// history entries: 10 bits of value + 1 for each of M~, I~, D~, or three int16
-template <typename E>
-struct Entry;
-template <>
-struct Entry<uint32_t> {
-    static constexpr uint32_t kBias = 1u | (1u << 10) | (1u << 20);
-    static __device__ __forceinline__ uint32_t make(int m, int i, int d) {
-        return (uint32_t)m + ((uint32_t)i << 10) + ((uint32_t)d << 20);   // each value + 1 once kBias is added
+// history forms
+enum : int { kWhole = 0, kBits16 = 1, kBits32 = 2 };
+template <int FMT>
+struct Entry {   // kBits16, kBits32
+    using T = typename std::conditional<FMT == kBits16, uint16_t, uint32_t>::type;
+    static constexpr int kBits = FMT == kBits16 ? 14 : 30;
+    static __device__ __forceinline__ T make(int m, int i, int d, int mo) {
+        return (T)((uint32_t)(m + 1) | ((uint32_t)(i > mo) << kBits) | ((uint32_t)(d > mo) << (kBits + 1)));
     }
-    static __device__ __forceinline__ int m(uint32_t e) { return (int)((e + kBias) & 1023u) - 1; }
-    static __device__ __forceinline__ int i(uint32_t e) { return (int)(((e + kBias) >> 10) & 1023u) - 1; }
-    static __device__ __forceinline__ int d(uint32_t e) { return (int)((e + kBias) >> 20) - 1; }
-    static __device__ __forceinline__ uint32_t none() { return 0u - kBias; }
+    static __device__ __forceinline__ T none() { return 0; }
+    static __device__ __forceinline__ int m(T e) { return (int)((uint32_t)e & ((1u << kBits) - 1)) - 1; }
+    static __device__ __forceinline__ bool from_ins(T e) { return ((uint32_t)e >> kBits) & 1u; }
+    static __device__ __forceinline__ bool from_del(T e) { return ((uint32_t)e >> (kBits + 1)) & 1u; }
 };
 template <>
-struct Entry<uint64_t> {
-    static __device__ __forceinline__ uint64_t make(int m, int i, int d) {
-        return (uint64_t)(uint32_t)prmt((uint32_t)m, (uint32_t)i, 0x5410u) | ((uint64_t)(uint32_t)d << 32);
+struct Entry<kWhole> {
+    using T = uint32_t;
+    static constexpr uint32_t kBias = 1u | (1u << 10) | (1u << 20);
+    static __device__ __forceinline__ T make(int m, int i, int d, int) {
+        return (uint32_t)m + ((uint32_t)i << 10) + ((uint32_t)d << 20);   // each value + 1 once kBias is added
     }
-    static __device__ __forceinline__ int m(uint64_t e) { return (int16_t)(uint16_t)e; }
-    static __device__ __forceinline__ int i(uint64_t e) { return (int16_t)(uint16_t)(e >> 16); }
-    static __device__ __forceinline__ int d(uint64_t e) { return (int16_t)(uint16_t)(e >> 32); }
-    static __device__ __forceinline__ uint64_t none() { return ~0ull; }
+    static __device__ __forceinline__ T none() { return 0u - kBias; }
+    static __device__ __forceinline__ int m(T e) { return (int)((e + kBias) & 1023u) - 1; }
+    static __device__ __forceinline__ int i(T e) { return (int)(((e + kBias) >> 10) & 1023u) - 1; }
+    static __device__ __forceinline__ int d(T e) { return (int)((e + kBias) >> 20) - 1; }
+    static __device__ __forceinline__ bool from_ins(T) { return false; }
+    static __device__ __forceinline__ bool from_del(T) { return false; }
 };
 
 // 16 bases from position pos of a sequence copy (32-bit word i of the pair at [i * P])
@@ -144,29 +150,99 @@ struct Pending {
     int round;
 };
 
-// Canonical traceback of one finished pair by one lane (the tests of wfa.cu's traceback).  Every step issues all its
-// loads at once: the four entries and both sequences' windows ending at (v, h), whose XOR gives the match run.
-// The rows' ranges are those of the forward pass, by arithmetic: no table is read.
+// Where entry (c, j) of a finished pair lies: row c at c * stride, or, with kDense, rows end to end, row c at the sum
+// of hi(i) - lo(i) + 1 over i < c.  lo(i) is zero - min(g, zero - 1), g = max(i - O, 0), up to row turn_lo and the
+// line end - S + i from there on (the first does not grow with i, the second does); hi(i) likewise.
+template <int P, bool kDense>
+struct RowMap {
+    Window w;
+    int O;
+    uint32_t stride;
+    int turn_lo, turn_hi, sum_lo, sum_hi;   // kDense: the sums of lo, hi up to those rows
+    // sum of min(t, a) over t = 1 .. u
+    static __device__ __forceinline__ int ramp(int u, int a) {
+        u = max(u, 0);
+        const int q = min(u, a);
+        return q * (q + 1) / 2 + (u - q) * a;
+    }
+    __device__ __forceinline__ int early_lo(int c) const { return c * w.zero - ramp(c - 1 - O, w.zero - 1); }
+    __device__ __forceinline__ int early_hi(int c) const { return c * w.zero + ramp(c - 1 - O, w.last - w.zero); }
+    __device__ __forceinline__ RowMap(const Window& win, int o, uint32_t st) : w(win), O(o), stride(st) {
+        if constexpr (kDense) {
+            const int S = w.S, z = w.zero, e = w.end;
+            turn_lo = max(min(z + S - e, (z + O + S - e) >> 1), 1 - e + S);
+            turn_hi = max(min(e + S - z, (e + S - z + O) >> 1), e + S - w.last);
+            sum_lo = early_lo(turn_lo + 1);
+            sum_hi = early_hi(turn_hi + 1);
+        }
+    }
+    __device__ __forceinline__ uint32_t start(int c) const {
+        if constexpr (!kDense) return (uint32_t)c * stride;
+        const int dl = c - 1 - turn_lo, dh = c - 1 - turn_hi;
+        const int lo = dl <= 0 ? early_lo(c) : sum_lo + dl * (w.end - w.S) + (int)((uint32_t)((c + turn_lo) * dl) >> 1);
+        const int hi = dh <= 0 ? early_hi(c) : sum_hi + dh * (w.end + w.S) - (int)((uint32_t)((c + turn_hi) * dh) >> 1);
+        return (uint32_t)(hi - lo + c);
+    }
+    template <typename H>
+    __device__ __forceinline__ typename H::T get(const typename H::T* hist, int c, int j) const {
+        const int lo = w.lo(c, O);
+        if (c < 0 || j < lo || j > w.hi(c, O)) return H::none();
+        return hist[(size_t)start(c) + (uint32_t)((j - lo) * P)];
+    }
+};
+
+template <int P, int FMT>
+constexpr bool kDenseRows = P == 1 && FMT != kWhole;
+
+// Canonical traceback of one finished pair by one lane (the tests of wfa.cu's traceback).  Every step issues its loads
+// at once: the entries of its tests and both sequences' windows ending at (v, h), whose XOR gives the match run.
 // seqs_kept: the pair's copies in shared memory (words [i * P]); otherwise the packed sequences are read.
-template <int P, typename E>
+template <int P, int FMT>
 __device__ uint32_t ring_traceback(const WfaArgs& a, const uint8_t* rounds, const Pending& q, int g, bool seqs_kept,
                                    const uint32_t* sp, const uint32_t* st, RunStage& wr, bool& ok) {
-    const E* hist = reinterpret_cast<const E*>(rounds + ((size_t)q.base << 8)) + g;
+    using H = Entry<FMT>;
+    const typename H::T* hist = reinterpret_cast<const typename H::T*>(rounds + ((size_t)q.base << 8)) + g;
     const int n = (int)a.P.read_len[q.pi], m = (int)a.P.target_len[q.pi];
     const uint64_t* Pg = read_words(a.P, q.pi);
     const uint64_t* Tg = target_words(a.P, q.pi);
     const uint32_t nwP = (uint32_t)(n + 31) >> 5, nwT = (uint32_t)(m + 31) >> 5;
     const int X = a.X, OE = a.OE, O = OE - 1;
-    const Window w{q.koff, q.last, -q.koff, m - n - q.koff, q.S};
-    auto entry = [&](int c, int j) -> E {
-        const int lo = w.lo(c, O);
-        if (c < 0 || j < lo || j > w.hi(c, O)) return Entry<E>::none();
-        return hist[(size_t)(uint32_t)c * q.stride + (uint32_t)((j - lo) * P)];
+    const RowMap<P, kDenseRows<P, FMT>> rows(Window{q.koff, q.last, -q.koff, m - n - q.koff, q.S}, O, q.stride);
+    auto entry = [&](int c, int j) { return rows.template get<H>(hist, c, j); };
+    // source-bit forms: I~[c, j] from the bit of (c-1, j+1) and M~ of (c-OE, j+1), loaded together, or further back
+    // along the gap; D~ likewise
+    auto ins_of = [&](int c, int j, typename H::T src, typename H::T opening) -> int {
+        const int hmax = min(m, n + j + q.koff);
+        for (int guard = n + m; H::from_ins(src) && guard > 0; --guard) {
+            --c; ++j;
+            src = entry(c - 1, j + 1);
+            opening = entry(c - OE, j + 1);
+        }
+        const int at = H::m(opening);
+        return at <= hmax ? at : -1;
+    };
+    auto del_of = [&](int c, int j, typename H::T src, typename H::T opening) -> int {
+        const int hmax = min(m, n + j + q.koff);
+        int more = 1;
+        for (int guard = n + m; H::from_del(src) && guard > 0; --guard) {
+            --c; --j; ++more;
+            src = entry(c - 1, j - 1);
+            opening = entry(c - OE, j - 1);
+        }
+        const int at = H::m(opening);
+        return at >= 0 && at + more <= hmax ? at + more : -1;
     };
     int v = n, h = m, cM = q.final_s, cI = q.final_s, cD = q.final_s;
     while (v > 0 || h > 0) {
         const int j = h - v - q.koff;
-        const E eX = entry(cM - X, j), eI = entry(cI, j), eD = entry(cD, j), eM = entry(cM, j);
+        const auto eX = entry(cM - X, j), eM = entry(cM, j);
+        typename H::T eI, eD, oI, oD;
+        if constexpr (FMT == kWhole) {
+            eI = entry(cI, j); eD = entry(cD, j);
+        } else {
+            eI = entry(cI - 1, j + 1); oI = entry(cI - OE, j + 1);
+            eD = entry(cD - 1, j - 1); oD = entry(cD - OE, j - 1);
+        }
         const int avail = min(v, h);
         int same;   // matching bases back from (v, h), as far as the window shows
         if (seqs_kept) {   // 16 bases back; before the start the window's earlier bases are not looked at
@@ -181,20 +257,30 @@ __device__ uint32_t ring_traceback(const WfaArgs& a, const uint8_t* rounds, cons
             same = min(d ? (__ffsll((long long)d) - 1) >> 1 : 32, back);
         }
         const bool diag = avail > 0, match = same > 0;
-        if (diag && !match && Entry<E>::m(eX) >= h - 1) {
+        if (diag && !match && H::m(eX) >= h - 1) {
             cM = cI = cD = cM - X; --v; --h;
             wr.put(kOpMismatch, 1);
-        } else if (v > 0 && Entry<E>::i(eI) >= h) {
+            continue;
+        }
+        int vI, vD;
+        if constexpr (FMT == kWhole) { vI = H::i(eI); vD = H::d(eD); }
+        else { vI = ins_of(cI, j, eI, oI); vD = del_of(cD, j, eD, oD); }
+        if (v > 0 && vI >= h) {
             const int c = cI;
             cM = cD = c - OE; cI = c - 1; --v;
             wr.put(kOpIns, 1);
-        } else if (h > 0 && Entry<E>::d(eD) >= h) {
+        } else if (h > 0 && vD >= h) {
             const int c = cD;
             cM = cI = c - OE; cD = c - 1; --h;
             wr.put(kOpDel, 1);
-        } else if (match && Entry<E>::m(eM) >= h - 1) {
+        } else if (match && H::m(eM) >= h - 1) {
             // a longer run is taken window by window: I~ and D~ of this score stop it at the same offset
-            const int run = min(same, h - max(Entry<E>::i(eM), Entry<E>::d(eM)));
+            if constexpr (FMT == kWhole) { vI = H::i(eM); vD = H::d(eM); }
+            else {
+                if (cI != cM) vI = ins_of(cM, j, entry(cM - 1, j + 1), entry(cM - OE, j + 1));
+                if (cD != cM) vD = del_of(cM, j, entry(cM - 1, j - 1), entry(cM - OE, j - 1));
+            }
+            const int run = min(same, h - max(vI, vD));
             if (run < 1) { ok = false; break; }
             v -= run; h -= run;
             cI = cD = cM;
@@ -211,25 +297,38 @@ __device__ uint32_t ring_traceback(const WfaArgs& a, const uint8_t* rounds, cons
 
 extern __shared__ __align__(16) uint8_t s_ring[];
 
-template <int G, typename E>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs r) {
-    constexpr int P = 32 / G;
+// threads of a block: four warps on their own, or, for G > 32, one group of G threads on one pair
+template <int G>
+constexpr int kBlockThreads = G > 32 ? G : 32 * kWarpsPerBlock;
+
+template <int G, int FMT>
+__global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) {
+    using E = typename Entry<FMT>::T;
+    constexpr bool kBlock = G > 32;
+    constexpr int P = kBlock ? 1 : 32 / G;
+    constexpr bool kDense = kDenseRows<P, FMT>;
+    constexpr int kRounds = 32 / P;          // rounds of P pairs until 32 tracebacks are due
     constexpr int kRows = G == 1 ? 1 : 2;   // jd rows: one lane per pair updates its row in place
     const WfaArgs& a = r.w;
-    const int lane = (int)(threadIdx.x & 31);
+    // lane of the unit (a warp, or the block), this thread's pair and its place among the pair's lanes
+    const int lane = kBlock ? (int)threadIdx.x : (int)(threadIdx.x & 31);
     const int g = lane % P, gl = lane / P;
-    const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gwarp >= a.nwarps) return;
+    const uint32_t unit = kBlock ? blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (unit >= a.nwarps) return;
+    auto sync = [] {
+        if constexpr (kBlock) __syncthreads();
+        else __syncwarp();
+    };
     const uint32_t W = r.width;
-    uint8_t* sm = s_ring + (size_t)(threadIdx.x >> 5) * r.smem_warp;
+    uint8_t* sm = s_ring + (kBlock ? 0 : (size_t)(threadIdx.x >> 5) * r.smem_warp);
     uint2* mh = reinterpret_cast<uint2*>(sm);                            // [W][P]
     uint32_t* jd = reinterpret_cast<uint32_t*>(sm + (size_t)W * P * 8);  // [kRows][W][P]
     // copies of a round's reads, then of its targets, [seq_words][P] each; of every round awaiting its traceback
     // when seq_rounds says so
     uint32_t* seq = jd + (size_t)kRows * W * P;
     const uint32_t seq_round = 2 * r.seq_words * P;
-    const bool seqs_kept = r.seq_rounds == (uint32_t)G;
-    uint8_t* arena = a.scratch + (size_t)gwarp * a.warp_bytes;
+    const bool seqs_kept = r.seq_rounds == (uint32_t)kRounds;
+    uint8_t* arena = a.scratch + (size_t)unit * a.warp_bytes;
     uint8_t* rounds = arena + 32 * a.runs_bytes;
     const size_t rounds_bytes = a.warp_bytes - 32 * a.runs_bytes;
     const int O = a.OE - 1;
@@ -238,21 +337,25 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
     unsigned long long st_cells = 0, st_windows = 0;
     uint32_t st_pairs = 0;
 
+    __shared__ int s_end[2];
     Pending pend{0, -1, 0, 0, 0, 0, 0, 0};
     int round = 0;
     size_t used = 0;   // arena bytes of the rounds awaiting their traceback
+    // the lane that traces pair g of round i: 32 in a warp, spread over the warps of a block
+    auto tracer = [&](int i) { return kBlock ? (i % (G / 32)) * 32 + i / (G / 32) : i * P + g; };
     auto finish = [&]() {
-        __syncwarp();
+        sync();
         // runs staged where the forward pass kept its state, lane l's i-th run at [33 i + l], or in the arena
-        uint32_t* stage = r.stage_shared ? reinterpret_cast<uint32_t*>(sm) + lane
-                                         : reinterpret_cast<uint32_t*>(arena + (size_t)lane * a.runs_bytes);
+        const int slot = kBlock ? pend.round : lane;
+        uint32_t* stage = r.stage_shared ? reinterpret_cast<uint32_t*>(sm) + slot
+                                         : reinterpret_cast<uint32_t*>(arena + (size_t)slot * a.runs_bytes);
         RunStage wr{stage, r.stage_shared ? 33u : 1u, a.runs_cap, 0, 0, 0};
         bool ok = pend.final_s >= 0;
         uint64_t off = 0;
         uint32_t copy = 0;
         if (ok) {
             const uint32_t* sp = seq + (seqs_kept ? (uint32_t)pend.round * seq_round : 0u) + g;
-            const uint32_t nruns = ring_traceback<P, E>(a, rounds, pend, g, seqs_kept, sp, sp + r.seq_words * P, wr, ok);
+            const uint32_t nruns = ring_traceback<P, FMT>(a, rounds, pend, g, seqs_kept, sp, sp + r.seq_words * P, wr, ok);
             uint8_t flags = ok ? 0 : AIM_F_STEP_CAP;
             if (ok && a.O.cigars) {
                 off = a.O.cigar_off[pend.pi];
@@ -264,16 +367,17 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
         __syncwarp();
         if (a.O.cigars) {   // half a warp copies one pair's runs, start first
             const int hl = lane & 15;
-            for (int q = lane >> 4; q < 32; q += 2) {
+            for (int q = (lane & 31) >> 4; q < 32; q += 2) {
                 const uint32_t cnt = __shfl_sync(kFull, copy, q);
                 const uint64_t at = __shfl_sync(kFull, off, q);
-                const uint32_t* from = r.stage_shared ? reinterpret_cast<const uint32_t*>(sm) + q
-                                                      : reinterpret_cast<const uint32_t*>(arena + (size_t)q * a.runs_bytes);
+                const int sl = __shfl_sync(kFull, slot, q);
+                const uint32_t* from = r.stage_shared ? reinterpret_cast<const uint32_t*>(sm) + sl
+                                                      : reinterpret_cast<const uint32_t*>(arena + (size_t)sl * a.runs_bytes);
                 const uint32_t step = r.stage_shared ? 33u : 1u;
                 for (uint32_t i = (uint32_t)hl; i < cnt; i += 16) a.O.cigars[at + i] = from[(cnt - 1 - i) * step];
             }
         }
-        __syncwarp();
+        sync();
         pend.final_s = -1;
         round = 0;
         used = 0;
@@ -281,10 +385,18 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
 
     for (;;) {
         uint32_t pos = 0;
-        if (lane == 0) pos = atomicAdd(a.counters, (uint32_t)P);
-        pos = __shfl_sync(kFull, pos, 0);
+        if constexpr (kBlock) {
+            __shared__ uint32_t s_pos;
+            if (lane == 0) s_pos = atomicAdd(a.counters, 1u);
+            __syncthreads();
+            pos = s_pos;
+            __syncthreads();
+        } else {
+            if (lane == 0) pos = atomicAdd(a.counters, (uint32_t)P);
+            pos = __shfl_sync(kFull, pos, 0);
+        }
         if (pos >= end - begin || end <= begin) break;
-        if (round == G || rounds_bytes - used < r.round_bytes) finish();
+        if (round == kRounds || rounds_bytes - used < r.round_bytes) finish();
 
         // ---- the round's pairs
         const uint32_t q = begin + pos + (uint32_t)g;
@@ -324,17 +436,18 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
             if (a.band >= 0) { right = min(right, a.band); left = min(left, a.band); }
             win = Window{-left - 1, left + right + 1, left + 1, kend + left + 1, S};
         }
-        const int wide = __reduce_max_sync(kFull, win.last);   // 0: no pair to run
+        const int wide = P == 1 ? win.last : __reduce_max_sync(kFull, win.last);   // 0: no pair to run
         // entry (s, t-th of its row) of the history at [s * stride + t * P]
         const uint32_t stride = ((uint32_t)wide * P + 31u) & ~31u;
         int final_s = -1, s = 0;
+        uint32_t entries = 0;   // of the round's history
         if (wide) {
             uint32_t* dp = seq + (seqs_kept ? (uint32_t)round * seq_round : 0u) + g;
             uint32_t* dt = dp + r.seq_words * P;
             const uint32_t* sp = dp;
             const uint32_t* st = dt;
             // nothing is reachable yet
-            for (int i = lane; i < (wide + 2) * P; i += 32) {
+            for (int i = lane; i < (wide + 2) * P; i += kBlock ? G : 32) {
                 mh[i] = make_uint2(~0u, ~0u);
                 jd[i] = ~0u;
                 if (kRows == 2) jd[i + W * P] = ~0u;
@@ -351,27 +464,38 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
                     dt[2 * w * P] = (uint32_t)(x >> 32); dt[(2 * w + 1) * P] = (uint32_t)x;
                 }
             }
-            __syncwarp();
+            sync();
             uint32_t cells = 0, windows = 0;
             E* hrow = reinterpret_cast<E*>(rounds + used) + lane;   // row s, this lane's first entry
+            uint32_t filled = 1;                                    // kDense: entries of the rows so far
             // row 0: diagonal 0 from offset 0
             if (run && gl == 0) {
                 const int m0 = match_on<P>(sp, st, 0, 0, min(n, m));
                 mh[win.zero * P + g] = make_uint2((uint32_t)m0 | 0xffff0000u, ~0u);
-                hrow[0] = Entry<E>::make(m0, -1, -1);
+                hrow[0] = Entry<FMT>::make(m0, -1, -1, -1);
+                if constexpr (kBlock) s_end[0] = win.zero == win.end ? m0 : -1;
                 ++cells; ++windows;
             }
             for (;;) {
                 // the row just computed ends the pair if it reaches the end of the end diagonal
-                if (G > 1) __syncwarp();
-                if (run && (int)(mh[win.end * P + g].x & 0xffffu) == m) { status = kDone; final_s = s; run = false; }
+                if (G > 1) sync();
+                int reached;   // M~ on the end diagonal
+                if constexpr (kBlock) reached = s_end[s & 1];
+                else reached = (int)(mh[win.end * P + g].x & 0xffffu);
+                if (G == 32) __syncwarp();   // every lane has read it before the next row is written (P > 1: the vote below)
+                if (run && reached == m) { status = kDone; final_s = s; run = false; }
                 ++s;
                 if (run && s > S) { status = kRejected; run = false; }
-                if (!__any_sync(kFull, run)) break;
-                hrow += stride;
+                if (P == 1 ? !run : !__any_sync(kFull, run)) break;
                 const int jlo = win.lo(s, O), jhi = win.hi(s, O);
                 const int w = run ? max(jhi - jlo + 1, 0) : 0;
-                const int rows = __reduce_max_sync(kFull, w);
+                const int rows = P == 1 ? w : __reduce_max_sync(kFull, w);
+                if constexpr (kDense) {
+                    hrow = reinterpret_cast<E*>(rounds + used) + filled + lane;
+                    filled += (uint32_t)w;
+                } else {
+                    hrow += stride;
+                }
                 const uint32_t odd = (uint32_t)(s & 1);
                 const uint32_t at = (uint32_t)(jlo * P + g);       // the row's first position
                 uint2* mhr = mh + at;
@@ -428,7 +552,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
                                 make_uint2((uint32_t)prmt((uint32_t)mv[u], h4[u].x, 0x5410u),
                                            (uint32_t)prmt(h4[u].x, h4[u].y, 0x5432u));
                             jw[t * P] = (uint32_t)prmt((uint32_t)max(mo[u], ins[u]), (uint32_t)max(mo[u], del[u]), 0x5410u);
-                            hrow[(tb + u * G) * P] = Entry<E>::make(mv[u], ins[u], del[u]);
+                            hrow[(tb + u * G) * P] = Entry<FMT>::make(mv[u], ins[u], del[u], mo[u]);
                         }
                     }
                 };
@@ -438,6 +562,11 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
                     for (; t + G < rows; t += 2 * G) step(t, std::integral_constant<int, 2>{});
                     if (t < rows) step(t, std::integral_constant<int, 1>{});
                 }
+                if constexpr (kBlock) {   // the end diagonal's M~ for the check above, in a place of the row's parity
+                    const int te = win.end - jlo;
+                    const bool in_row = te >= 0 && te < w;
+                    if (gl == (in_row ? te % G : 0)) s_end[odd] = in_row ? (int)(mhr[te].x & 0xffffu) : -1;
+                }
                 if (gl == 0 && w > 0) {   // just outside the row: invalid
                     jw[-P] = ~0u;
                     jw[w * P] = ~0u;
@@ -446,34 +575,42 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) wfa_ring_kernel(RingArgs 
             }
             st_cells += cells;
             st_windows += windows;
+            entries = kDense ? filled : (uint32_t)s * stride;
         }
         if (gl == 0 && (status == kRejected || status == kBad)) emit_failed(a, pi, status);
-        // lane round * P + g will trace pair g of this round
-        const int src = lane % P;
-        const uint32_t p_pi = __shfl_sync(kFull, pi, src);
-        const int p_s = __shfl_sync(kFull, final_s, src), p_koff = __shfl_sync(kFull, win.koff, src);
-        const int p_last = __shfl_sync(kFull, win.last, src), p_S = __shfl_sync(kFull, S, src);
-        if (lane / P == round) pend = Pending{p_pi, p_s, p_koff, p_last, p_S, (uint32_t)(used >> 8), stride, round};
-        if (wide) {
-            used += ((size_t)s * stride * sizeof(E) + 255) & ~(size_t)255;
+        // the pair's tracer takes what it needs (P == 1: every lane has it)
+        if constexpr (P == 1) {
+            if (lane == tracer(round))
+                pend = Pending{pi, final_s, win.koff, win.last, S, (uint32_t)(used >> 8), stride, round};
+        } else {
+            const int src = lane % P;
+            const uint32_t p_pi = __shfl_sync(kFull, pi, src);
+            const int p_s = __shfl_sync(kFull, final_s, src), p_koff = __shfl_sync(kFull, win.koff, src);
+            const int p_last = __shfl_sync(kFull, win.last, src), p_S = __shfl_sync(kFull, S, src);
+            if (lane == tracer(round)) pend = Pending{p_pi, p_s, p_koff, p_last, p_S, (uint32_t)(used >> 8), stride, round};
+        }
+        if (wide && (P > 1 || final_s >= 0)) {   // (a single pair that was rejected leaves nothing to trace)
+            used += ((size_t)entries * sizeof(E) + 255) & ~(size_t)255;
             ++round;
         }
     }
     finish();
-    warp_stat_add(a.O.stats, 0, st_cells, (uint32_t)lane);
-    warp_stat_add(a.O.stats, 1, st_windows, (uint32_t)lane);
-    warp_stat_add(a.O.stats, 3, st_pairs, (uint32_t)lane);
+    const uint32_t wl = threadIdx.x & 31;
+    warp_stat_add(a.O.stats, 0, st_cells, wl);
+    warp_stat_add(a.O.stats, 1, st_windows, wl);
+    warp_stat_add(a.O.stats, 3, st_pairs, wl);
 }
 
-template <typename E>
+template <int FMT>
 void (*ring_kernel_for(int G))(RingArgs) {
     switch (G) {
-        case 1: return wfa_ring_kernel<1, E>;
-        case 2: return wfa_ring_kernel<2, E>;
-        case 4: return wfa_ring_kernel<4, E>;
-        case 8: return wfa_ring_kernel<8, E>;
-        case 16: return wfa_ring_kernel<16, E>;
-        default: return wfa_ring_kernel<32, E>;
+        case 1: return wfa_ring_kernel<1, FMT>;
+        case 2: return wfa_ring_kernel<2, FMT>;
+        case 4: return wfa_ring_kernel<4, FMT>;
+        case 8: return wfa_ring_kernel<8, FMT>;
+        case 16: return wfa_ring_kernel<16, FMT>;
+        case 32: return wfa_ring_kernel<32, FMT>;
+        default: return wfa_ring_kernel<256, FMT>;
     }
 }
 
@@ -486,17 +623,30 @@ void (*ring_kernel_for(int G))(RingArgs) {
 // 0.045 / 0.039 / 0.037.
 constexpr size_t kGoodSmem = 14u << 10;
 constexpr int kGoodWarps = 8;
-constexpr size_t kMaxSmem = 227u << 10;   // shared memory a block may use
+constexpr size_t kBlockSmem = 20u << 10;   // a whole block per pair where a warp's state takes more
+constexpr size_t kMaxSmem = 226u << 10;   // dynamic shared memory a block may use (227 KB, less its static few bytes)
 
-size_t entry_bytes(uint32_t max_length) { return max_length <= kNarrowLength ? 4 : 8; }
+int entry_form(uint32_t max_length) {
+    return max_length <= kNarrowLength ? kWhole : max_length <= kMaxWfaLength16c ? kBits16 : kBits32;
+}
+size_t entry_bytes(uint32_t max_length) { return entry_form(max_length) == kBits16 ? 2 : 4; }
+
+// pairs of a warp, or 1 where a block works on one
+size_t pairs_of(int G) { return G > 32 ? 1 : 32 / G; }
 
 // diagonals per pair: the widest window (2 O + 2 k - kend <= S on both sides, or just 0 .. kend: S - O + 1), the
-// band's or the matrix's, and the two padding positions
+// band's or the matrix's, or what the caller knows of its pairs, and the two padding positions
 int64_t ring_width(const WfaPlan& p, uint32_t max_length) {
     const int64_t O = p.oe - p.e;
     int64_t w = p.smax - O + 1;
     if (p.band >= 0) w = std::min<int64_t>(w, 2 * (int64_t)p.band + 1);
+    if (p.ring_diagonals) w = std::min<int64_t>(w, p.ring_diagonals);
     return std::max<int64_t>(std::min<int64_t>(w, 2 * (int64_t)max_length + 1), 1) + 2;
+}
+
+// rows 0 .. S of a pair
+size_t ring_rows(const WfaPlan& p) {
+    return (size_t)(p.ring_scores ? std::min(p.ring_scores, p.smax) : p.smax) + 1;
 }
 
 uint32_t seq_words(uint32_t max_length) { return 2 * ((max_length + 31) / 32) + 2; }
@@ -514,15 +664,22 @@ constexpr size_t kKeepBytes = 5u << 10;
 }  // namespace
 
 size_t ring_smem_per_warp(const WfaPlan& p, int G, uint32_t max_length) {
-    const size_t P = 32 / G, W = (size_t)ring_width(p, max_length);
+    const size_t P = pairs_of(G), W = (size_t)ring_width(p, max_length);
     const size_t kept = seq_bytes(max_length, 32) <= kKeepBytes ? 32 : P;
     return align_up(P * W * (8 + (G == 1 ? 4 : 8)) + seq_bytes(max_length, kept), 16);
 }
 
 size_t ring_warp_bytes(const WfaPlan& p, int G, uint32_t max_length) {
-    const size_t P = 32 / G, W = (size_t)ring_width(p, max_length);
-    const size_t hist = ((size_t)p.smax + 1) * ((W * P + 31) / 32 * 32) * entry_bytes(max_length);
-    return align_up(32 * p.runs_bytes + hist + 256, 256);
+    const size_t P = pairs_of(G), W = (size_t)ring_width(p, max_length);
+    size_t entries = 0;
+    if (P > 1 || entry_form(max_length) == kWhole) {
+        entries = ring_rows(p) * ((W * P + 31) / 32 * 32);
+    } else {   // row s: at most s - O diagonals from 0, at most S - s from the end diagonal, the window
+        const int64_t O = p.oe - p.e, S = (int64_t)ring_rows(p) - 1;
+        for (int64_t s = 0; s <= S; ++s)
+            entries += (size_t)std::min(std::min(2 * std::max<int64_t>(s - O, 0), 2 * (S - s)) + 1, (int64_t)W - 2);
+    }
+    return align_up(32 * p.runs_bytes + entries * entry_bytes(max_length) + 512, 256);
 }
 
 bool ring_ok(const WfaPlan& p, uint32_t max_length) {
@@ -531,9 +688,12 @@ bool ring_ok(const WfaPlan& p, uint32_t max_length) {
            max_length <= kMaxWfaLength16 && ring_width(p, max_length) < 32768 && p.smax < (1 << 20);
 }
 
+// units (warps, or blocks for G > 32) of a block
+static size_t units_of(int G) { return G > 32 ? 1 : kWarpsPerBlock; }
+
 bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_bytes) {
-    return G <= 32 && ring_ok(p, max_length) && kWarpsPerBlock * ring_smem_per_warp(p, G, max_length) <= kMaxSmem &&
-           kWarpsPerBlock * ring_warp_bytes(p, G, max_length) <= scratch_bytes;
+    return ring_ok(p, max_length) && units_of(G) * ring_smem_per_warp(p, G, max_length) <= kMaxSmem &&
+           units_of(G) * ring_warp_bytes(p, G, max_length) <= scratch_bytes;
 }
 
 int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes) {
@@ -542,7 +702,8 @@ int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int nu
                       (uint64_t)num_pairs * G < (uint64_t)num_sms * kGoodWarps * 32))
         G *= 2;
     while (G <= 32 && !ring_fits(p, G, max_length, scratch_bytes)) G *= 2;
-    return G <= 32 ? G : 0;
+    if (G > 32 || (G == 32 && ring_smem_per_warp(p, G, max_length) > kBlockSmem)) G = 256;
+    return ring_fits(p, G, max_length, scratch_bytes) ? G : 0;
 }
 
 cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, const LimitView& L, const OutView& O,
@@ -559,36 +720,38 @@ cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, cons
     a.order = order; a.bounds = bounds; a.counters = counters; a.nbuckets = 1;
     a.bound = plan.bound; a.retry_only = plan.retry_only;
     const uint32_t len = P.max_length;
-    const size_t e_bytes = entry_bytes(len);
     r.width = (uint32_t)ring_width(plan, len);
     r.seq_words = seq_words(len);
     r.smem_warp = (uint32_t)ring_smem_per_warp(plan, G, len);
-    r.seq_rounds = seq_bytes(len, 32) <= kKeepBytes ? (uint32_t)G : 1u;
-    r.stage_shared = (size_t)plan.runs_cap * 33 * 4 <= (size_t)r.width * (32 / G) * (8 + (G == 1 ? 4 : 8));
+    r.seq_rounds = seq_bytes(len, 32) <= kKeepBytes ? (uint32_t)(32 / pairs_of(G)) : 1u;
+    r.stage_shared = (size_t)plan.runs_cap * 33 * 4 <= (size_t)r.width * pairs_of(G) * (8 + (G == 1 ? 4 : 8));
     const size_t min_warp = ring_warp_bytes(plan, G, len);
     r.round_bytes = min_warp - 32 * plan.runs_bytes;
     // value d scores back: bytes 2 (d - 1) and 2 (d - 1) + 1 of mh, the sign replicated above them
     auto sel = [](int d) { const uint32_t b = 2u * (uint32_t)(d - 1); return b | ((b + 1) << 4) | ((b + 9) << 8) | ((b + 9) << 12); };
     r.sel_x = sel(plan.x);
     r.sel_o = sel(plan.oe - plan.e);
-    void (*kernel)(RingArgs) = e_bytes == 4 ? ring_kernel_for<uint32_t>(G) : ring_kernel_for<uint64_t>(G);
-    const size_t smem = (size_t)kWarpsPerBlock * r.smem_warp;
+    void (*kernel)(RingArgs) = entry_form(len) == kWhole    ? ring_kernel_for<kWhole>(G)
+                                   : entry_form(len) == kBits16 ? ring_kernel_for<kBits16>(G)
+                                                                : ring_kernel_for<kBits32>(G);
+    const size_t units = units_of(G), smem = units * r.smem_warp;
+    const int threads = G > 32 ? G : 32 * kWarpsPerBlock;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (e != cudaSuccess) return e;
     int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, 32 * kWarpsPerBlock, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, threads, smem);
     if (e != cudaSuccess) return e;
     if (bps < 1) return cudaSuccess;
-    size_t warps = (size_t)num_sms * bps * kWarpsPerBlock;
-    warps = std::min(warps, scratch_bytes / min_warp);
-    if (!bounds) warps = std::min(warps, ((size_t)P.num_pairs * G + 31) / 32);
-    if (warps == 0) return cudaSuccess;
-    a.nwarps = (uint32_t)warps;
-    // a warp's arena: its share of the scratch, up to G worst-case rounds
-    a.warp_bytes = std::min(scratch_bytes / warps & ~(size_t)255, min_warp + (size_t)(G - 1) * r.round_bytes);
-    kernel<<<(unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock), 32 * kWarpsPerBlock, smem, st>>>(r);
+    size_t n = (size_t)num_sms * bps * units;
+    n = std::min(n, scratch_bytes / min_warp);
+    if (!bounds) n = std::min(n, ((size_t)P.num_pairs + pairs_of(G) - 1) / pairs_of(G));
+    if (n == 0) return cudaSuccess;
+    a.nwarps = (uint32_t)n;
+    // a unit's arena: its share of the scratch, up to as many worst-case rounds as it defers
+    a.warp_bytes = std::min(scratch_bytes / n & ~(size_t)255, min_warp + (32 / pairs_of(G) - 1) * r.round_bytes);
+    kernel<<<(unsigned)((n + units - 1) / units), threads, smem, st>>>(r);
     e = cudaGetLastError();
-    if (e == cudaSuccess) *warps_used = (int)warps;
+    if (e == cudaSuccess) *warps_used = (int)n;
     return e;
 }
 

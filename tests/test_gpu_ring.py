@@ -44,7 +44,7 @@ def _mixed(lengths, seed):
     return gen.from_strings(reads, targets)
 
 
-@pytest.mark.parametrize("lanes", [1, 2, 4, 8, 16, 32])
+@pytest.mark.parametrize("lanes", [1, 2, 4, 8, 16, 32, 256])
 @pytest.mark.parametrize("penalties,max_edits,band", [((0, 4, 6, 2), 6, -1), ((0, 3, 4, 1), 8, -1),
                                                       ((0, 4, 6, 2), 1, -1), ((0, 2, 3, 1), 12, 5),
                                                       ((0, 4, 4, 4), 9, 0), ((0, 4, 6, 2), 20, 15)])
@@ -64,12 +64,21 @@ def test_ring_matches_oracle(aligner, lanes, penalties, max_edits, band):
     assert_same(dev, oracle_results(p, penalties, lim, band=band), what=f"ring, {lanes} lanes")
 
 
-@pytest.mark.parametrize("length", [1000, 1022, 1023, 1500])
-def test_ring_at_the_narrow_history_limit(aligner, length):
-    """max_length up to 1,022 keeps 10-bit history fields, beyond it 16-bit ones."""
-    w = gen.Workload("ring_edge", 91, 40, length, length, 0.01, 0.01, 0.2, "wfa", (0, 4, 6, 2), 15)
+@pytest.mark.parametrize("lanes", [1, 4, 32, 256])
+@pytest.mark.parametrize("length,edits", [(1000, 15), (1022, 15), (1023, 15), (1500, 60), (16382, 20), (16383, 20)])
+def test_ring_history_forms(aligner, length, edits, lanes):
+    """max_length up to 1,022 keeps 10-bit history fields, up to 16,382 source bits in 16-bit words, beyond in 32."""
+    import paper_2208_01243_gb300 as aim
+    rate = 0.7 * edits / length
+    w = gen.Workload("ring_edge", 91, 40 if length < 2000 else 9, length, length, rate, rate, 0.2, "wfa", (0, 4, 6, 2),
+                     edits)
     p = gen.generate(w)
     keep = p.target_len <= length
     p = gen.from_strings([p.read(i) for i in np.nonzero(keep)[0]], [p.target(i) for i in np.nonzero(keep)[0]])
-    dev = device_results(p, "wfa", w.penalties, 15, max_length=length, aligner=aligner)
-    assert_same(dev, oracle_results(p, w.penalties, np.full(len(p), 120, np.int64)), what=f"ring, {length} bp")
+    aim.aim_set_wfa_group(aligner.ctx, lanes)
+    try:
+        dev = device_results(p, "wfa", w.penalties, edits, max_length=length, aligner=aligner)
+    finally:
+        aim.aim_set_wfa_group(aligner.ctx, 0)
+    assert_same(dev, oracle_results(p, w.penalties, np.full(len(p), 8 * edits, np.int64)),
+                what=f"ring, {length} bp, {lanes} lanes")
