@@ -121,6 +121,14 @@ cudaError_t launch_dp(const DpPlan& plan, const Costs& c, const PairsView& P, co
                       int64_t max_limit, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter,
                       int num_sms, cudaStream_t st, int* warps_used);
 
+// the same alignments with one pair per lane (dp_lane.cu): whether costs, band, lengths and scratch allow it and the batch
+// is large enough; the launch
+bool dp_lane_ok(bool unit, int band, const Costs& c, uint32_t max_length, int64_t max_limit, uint32_t num_pairs,
+                int num_sms, size_t scratch_bytes);
+cudaError_t launch_dp_lane(bool unit, int band, const Costs& c, const PairsView& P, const LimitView& L, const OutView& O,
+                           int64_t max_limit, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms,
+                           cudaStream_t st, int* warps_used);
+
 constexpr int kMaxBuckets = 32;
 // wavefront history: one entry per (score, diagonal) holds M~, I~, D~ and a spare slot as four int16, so an entry
 // is written with one 8-byte store

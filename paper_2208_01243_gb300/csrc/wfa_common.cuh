@@ -55,4 +55,34 @@ __device__ __forceinline__ void emit_failed(const WfaArgs& a, uint32_t pi, int s
     write_header(a.O, pi, -1, f, 0);
 }
 
+// runs in end-first order, every `stride` words
+struct RunStage {
+    uint32_t* runs;
+    uint32_t stride, cap, n, op, len;
+    __device__ __forceinline__ void flush() {
+        if (len) {
+            if (n < cap) runs[n * stride] = (len << 4) | op;
+            ++n;
+        }
+    }
+    __device__ __forceinline__ void put(uint32_t o, uint32_t l) {
+        if (o == op) { len += l; return; }
+        flush();
+        op = o; len = l;
+    }
+};
+
+// Whole warp: copies each lane's `count` runs, staged end first in slot `slot` (its i-th run at slot * between + i *
+// stride of staged), to its pair's place `at` in the CIGAR array, start first; half a warp takes one pair at a time.
+__device__ __forceinline__ void copy_runs(const OutView& O, uint32_t count, uint64_t at, const uint32_t* staged,
+                                          uint32_t between, uint32_t stride, int slot) {
+    const uint32_t wl = threadIdx.x & 31, hl = wl & 15;
+    for (int q = (int)(wl >> 4); q < 32; q += 2) {
+        const uint32_t cnt = __shfl_sync(kFull, count, q);
+        const uint64_t to = __shfl_sync(kFull, at, q);
+        const uint32_t* from = staged + (size_t)(uint32_t)__shfl_sync(kFull, slot, q) * between;
+        for (uint32_t i = hl; i < cnt; i += 16) O.cigars[to + i] = from[(size_t)(cnt - 1 - i) * stride];
+    }
+}
+
 }  // namespace aim

@@ -116,23 +116,6 @@ __device__ __forceinline__ int match_on(const uint32_t* sp, const uint32_t* st, 
     return min(run, rem);
 }
 
-// runs in end-first order, every `stride` words
-struct RunStage {
-    uint32_t* runs;
-    uint32_t stride, cap, n, op, len;
-    __device__ __forceinline__ void flush() {
-        if (len) {
-            if (n < cap) runs[n * stride] = (len << 4) | op;
-            ++n;
-        }
-    }
-    __device__ __forceinline__ void put(uint32_t o, uint32_t l) {
-        if (o == op) { len += l; return; }
-        flush();
-        op = o; len = l;
-    }
-};
-
 // A pair's ring: diagonal k at position k - koff, position 1 the window's first diagonal and `last` its last one;
 // diagonal 0 at `zero`, the end diagonal at `end`.  Row s covers lo(s) .. hi(s).
 struct Window {
@@ -365,18 +348,10 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
             write_header(a.O, pend.pi, ok ? pend.final_s * a.g : -1, flags, nruns);
         }
         __syncwarp();
-        if (a.O.cigars) {   // half a warp copies one pair's runs, start first
-            const int hl = lane & 15;
-            for (int q = (lane & 31) >> 4; q < 32; q += 2) {
-                const uint32_t cnt = __shfl_sync(kFull, copy, q);
-                const uint64_t at = __shfl_sync(kFull, off, q);
-                const int sl = __shfl_sync(kFull, slot, q);
-                const uint32_t* from = r.stage_shared ? reinterpret_cast<const uint32_t*>(sm) + sl
-                                                      : reinterpret_cast<const uint32_t*>(arena + (size_t)sl * a.runs_bytes);
-                const uint32_t step = r.stage_shared ? 33u : 1u;
-                for (uint32_t i = (uint32_t)hl; i < cnt; i += 16) a.O.cigars[at + i] = from[(cnt - 1 - i) * step];
-            }
-        }
+        if (a.O.cigars)
+            copy_runs(a.O, copy, off,
+                      r.stage_shared ? reinterpret_cast<const uint32_t*>(sm) : reinterpret_cast<const uint32_t*>(arena),
+                      r.stage_shared ? 1u : (uint32_t)(a.runs_bytes / 4), r.stage_shared ? 33u : 1u, slot);
         sync();
         pend.final_s = -1;
         round = 0;
