@@ -234,6 +234,14 @@ cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, cons
                             const uint32_t* order, const uint32_t* bounds, uint8_t* scratch, size_t scratch_bytes,
                             uint32_t* counters, int num_sms, cudaStream_t st, int* warps_used);
 
+// WFA-adaptive with its state in shared memory (wfa_adapt.cu): the lanes per pair suited to a call (0: not for it),
+// whether a launch with G lanes fits, one launch over all pairs (pairs that outgrow it get AIM_F_STEP_CAP)
+int adapt_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes);
+bool adapt_group_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_bytes);
+cudaError_t launch_wfa_adapt(const WfaPlan& plan, int G, const PairsView& P, const LimitView& L, const OutView& O,
+                             uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms, cudaStream_t st,
+                             int* warps_used);
+
 // GenASM (windowed bitap): scratch per warp for windows of W bases under the largest threshold max_limit
 size_t genasm_warp_bytes(int W, int64_t max_limit, uint32_t max_length);
 cudaError_t launch_genasm(int W, int O, const PairsView& P, const LimitView& L, const OutView& Ov, int64_t max_limit,

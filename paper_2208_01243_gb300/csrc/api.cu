@@ -171,8 +171,15 @@ int align_packed(aim_ctx* ctx, const aim::PairsView& P, int algo, const aim_pena
             g1 = fit_group(compact, g1);
             int group = fit_group(plan, ctx->wfa_group ? ctx->wfa_group : aim::wfa_default_group(plan, P.max_length));
             if (!g1 || !group) return AIM_ERR_NOMEM;
+            // the first pass: state in shared memory where costs and lengths allow it, else a compact history
+            int ga = aim::adapt_group(plan, P.max_length, P.num_pairs, ctx->num_sms, scratch_bytes);
+            if (ga && ctx->wfa_group)
+                ga = aim::adapt_group_fits(plan, ctx->wfa_group, P.max_length, scratch_bytes) ? ctx->wfa_group : 0;
             slot = time_begin(ctx, 1, st);
-            err = aim::launch_wfa(compact, g1, P, r.lim, O, scratch, scratch_bytes, counter, ctx->num_sms, st, &warps);
+            err = ga ? aim::launch_wfa_adapt(plan, ga, P, r.lim, O, scratch, scratch_bytes, counter, ctx->num_sms, st,
+                                             &warps)
+                     : aim::launch_wfa(compact, g1, P, r.lim, O, scratch, scratch_bytes, counter, ctx->num_sms, st,
+                                       &warps);
             if (err == cudaSuccess && warps > 0) {
                 aim::WfaPlan retry = plan;
                 retry.retry_only = 1;

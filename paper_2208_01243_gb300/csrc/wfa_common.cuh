@@ -55,6 +55,39 @@ __device__ __forceinline__ void emit_failed(const WfaArgs& a, uint32_t pi, int s
     write_header(a.O, pi, -1, f, 0);
 }
 
+__device__ __forceinline__ int prmt(uint32_t a, uint32_t b, uint32_t sel) {   // sign-replicating byte permute
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return (int)r;
+}
+
+// 16 bases from position pos of a sequence copy (32-bit word i of the pair at [i * P])
+template <int P>
+__device__ __forceinline__ uint32_t window16(const uint32_t* s, int pos) {
+    const uint32_t* w = s + (pos >> 4) * P;
+    return __funnelshift_l(w[P], w[0], 2 * pos);   // the shift is taken modulo 32
+}
+
+// the match run from (v, h) on, 32 bases a turn: at most rem
+template <int P>
+__device__ __forceinline__ int match_on(const uint32_t* sp, const uint32_t* st, int v, int h, int rem) {
+    int run = 0;
+    const uint32_t* p = sp + (v >> 4) * P;
+    const uint32_t* t = st + (h >> 4) * P;
+    uint32_t a = p[0], c = t[0];
+    do {
+        const uint32_t b = p[P], d = t[P];
+        const uint32_t x = __funnelshift_l(b, a, 2 * v) ^ __funnelshift_l(d, c, 2 * h);
+        if (x || run + 16 >= rem) { run += __clz((int)x) >> 1; break; }   // __clz(0) = 32
+        a = p[2 * P]; c = t[2 * P];
+        const uint32_t y = __funnelshift_l(a, b, 2 * v) ^ __funnelshift_l(c, d, 2 * h);
+        run += 16 + (__clz((int)y) >> 1);
+        if (y) break;
+        p += 2 * P; t += 2 * P;
+    } while (run < rem);
+    return min(run, rem);
+}
+
 // runs in end-first order, every `stride` words
 struct RunStage {
     uint32_t* runs;
