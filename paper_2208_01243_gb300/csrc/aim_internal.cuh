@@ -229,10 +229,20 @@ cudaError_t launch_wfa(const WfaPlan& plan, int group, const PairsView& P, const
 // over all pairs, or over the queue range bounds[0..1] of order
 bool ring_ok(const WfaPlan& p, uint32_t max_length);
 bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_bytes);
+size_t ring_warp_bytes(const WfaPlan& p, int G, uint32_t max_length);   // the least scratch of a warp (G = 256: a block)
 int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes);
 cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, const LimitView& L, const OutView& O,
                             const uint32_t* order, const uint32_t* bounds, uint8_t* scratch, size_t scratch_bytes,
                             uint32_t* counters, int num_sms, cudaStream_t st, int* warps_used);
+
+// scratch with which every unit of a full grid of launch_wfa_ring has its own
+size_t ring_full_scratch(const WfaPlan& p, int G, uint32_t max_length, int num_sms);
+// the bound pass with one pair per lane (wfa_bound.cu): whether costs and lengths allow it; over the queue range
+// bounds[0..1] of order, results in plan.bound
+bool bound_lanes_ok(const WfaPlan& p, uint32_t max_length);
+cudaError_t launch_wfa_bound(const WfaPlan& plan, const PairsView& P, const LimitView& L, const OutView& O,
+                             const uint32_t* order, const uint32_t* bounds, uint32_t* counters, int num_sms,
+                             cudaStream_t st);
 
 // WFA-adaptive with its state in shared memory (wfa_adapt.cu): the lanes per pair suited to a call (0: not for it),
 // whether a launch with G lanes fits, one launch over all pairs (pairs that outgrow it get AIM_F_STEP_CAP)

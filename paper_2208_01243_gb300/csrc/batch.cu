@@ -45,6 +45,13 @@
 // scores and CIGARs are those of the exact pass alone (the optimum and every
 // entry on an optimal path survive the clamp), so the tuner may add a bound
 // pass to any bucket it makes faster.
+// Plans of wfa_ring.cu.  Where that form takes the costs and lengths, the buckets are classes of the scaled limit S
+// instead, edges a quarter apart: a ring's size and a warp's work follow from S alone.  The bound pass, by rule rather
+// than by trial, runs over the classes above kBoundScore, the pairs are bucketed again by min(S, bound), and every class
+// has one exact launch of its own with the lanes per pair that rule suits its rings.  Planning runs the bound pass once
+// and merges classes that the batch fills too thinly.  1M pairs of 100-1,000 bp, 1-10 %: 19.7 ms, of which the bound
+// pass 2.3 (34.0 ms with the buckets above on wfa.cu's kernels, 22-26 ms with the same buckets on wfa_ring.cu's);
+// 4,000 pairs of 2-10 kbp 14.5 ms (31 ms; 18 ms; 23 ms before thin classes were merged).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -73,9 +80,22 @@ struct BucketParams {
     int8_t perm[kBuckets];          // queue order of the buckets (identity, or grouped by lanes per pair)
     int8_t gstart[kBuckets + 1];    // groups of consecutive permuted buckets sharing one lanes-per-pair value
     int ngroups;                    // 0: no groups
+    int nclasses;                   // > 0: the buckets are classes of scaled limits instead (wfa_ring.cu's plans)
+    int32_t edge[kBuckets];         // class c: limits above edge[c - 1] up to edge[c]; bucket nclasses - 1 - c
 };
 
-__device__ __forceinline__ int bucket_of(const PairsView& P, const LimitView& L, const BucketParams& bp, uint32_t i) {
+// `bound` (optional, classes only): scores that alignments of the pairs reach, which bound their limits
+__device__ __forceinline__ int bucket_of(const PairsView& P, const LimitView& L, const BucketParams& bp, uint32_t i,
+                                         const int32_t* bound) {
+    if (bp.nclasses) {
+        const int64_t lim = pair_limit(L, i);
+        int64_t S = lim < 0 ? 0 : lim / bp.g;
+        if (S > bp.smax) S = bp.smax;
+        if (bound && bound[i] >= 0 && bound[i] < S) S = bound[i];
+        int c = 0;
+        while (c + 1 < bp.nclasses && (int64_t)bp.edge[c] < S) ++c;
+        return bp.nclasses - 1 - c;
+    }
     const int64_t n = P.read_len[i], m = P.target_len[i];
     const int64_t lim = pair_limit(L, i);
     int64_t S = lim < 0 ? 0 : lim / bp.g;
@@ -96,12 +116,13 @@ __device__ __forceinline__ bool queued(const uint8_t* capped, uint32_t i) {
 }
 
 __global__ void __launch_bounds__(256) bucket_count_kernel(PairsView P, LimitView L, BucketParams bp,
-                                                           uint32_t* counts, const uint8_t* capped) {
+                                                           uint32_t* counts, const uint8_t* capped,
+                                                           const int32_t* bound) {
     __shared__ uint32_t h[kBuckets];
     if (threadIdx.x < kBuckets) h[threadIdx.x] = 0;
     __syncthreads();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < P.num_pairs; i += gridDim.x * blockDim.x)
-        if (queued(capped, i)) atomicAdd(&h[bucket_of(P, L, bp, i)], 1u);
+        if (queued(capped, i)) atomicAdd(&h[bucket_of(P, L, bp, i, bound)], 1u);
     __syncthreads();
     if (threadIdx.x < kBuckets && h[threadIdx.x]) atomicAdd(&counts[threadIdx.x], h[threadIdx.x]);
 }
@@ -130,7 +151,8 @@ __global__ void bucket_scan_kernel(const uint32_t* counts, uint32_t* bounds, uin
 
 __global__ void __launch_bounds__(256) bucket_scatter_kernel(PairsView P, LimitView L, BucketParams bp,
                                                              const uint32_t* bounds, uint32_t* fill,
-                                                             uint32_t* order, const uint8_t* capped) {
+                                                             uint32_t* order, const uint8_t* capped,
+                                                             const int32_t* bound) {
     __shared__ uint32_t h[kBuckets], base[kBuckets];
     for (uint32_t chunk = blockIdx.x * blockDim.x; chunk < P.num_pairs; chunk += gridDim.x * blockDim.x) {
         if (threadIdx.x < kBuckets) h[threadIdx.x] = 0;
@@ -139,7 +161,7 @@ __global__ void __launch_bounds__(256) bucket_scatter_kernel(PairsView P, LimitV
         int b = -1;
         uint32_t r = 0;
         if (i < P.num_pairs && queued(capped, i)) {
-            b = bucket_of(P, L, bp, i);
+            b = bucket_of(P, L, bp, i, bound);
             r = atomicAdd(&h[b], 1u);
         }
         __syncthreads();
@@ -238,6 +260,12 @@ struct aim_batch {
     int gbound[aim::kBuckets];          // lanes per pair of each group's bound pass (0: none)
     size_t gwarp_bytes[aim::kBuckets];  // scratch per warp of each group
     int64_t gdiagonals[aim::kBuckets], gscores[aim::kBuckets];   // each group's widest window and largest limit
+    // plans of wfa_ring.cu: one exact launch per class of limits, side by side on streams of their own
+    bool ring;
+    uint32_t* cclaims;
+    size_t class_at[aim::kBuckets], class_bytes[aim::kBuckets];   // each class's part of the scratch
+    cudaStream_t side[4];
+    cudaEvent_t fork, joined[4];
     uint32_t host_counts[aim::kBuckets];
     aim::BucketParams bp;
     cudaStream_t stream;
@@ -268,14 +296,195 @@ cudaError_t enqueue_prepare(aim_batch* b, cudaStream_t st) {
     e = cudaMemsetAsync(b->counts, 0, kBuckets * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)b->ctx->num_sms * 8);
-    bucket_count_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->counts, nullptr);
+    bucket_count_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->counts, nullptr, nullptr);
     bucket_scan_kernel<<<1, 32, 0, st>>>(b->counts, b->bounds, b->fill, b->claims, b->bp,
                                          b->bp.ngroups ? b->gbounds : nullptr);
-    bucket_scatter_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->bounds, b->fill, b->order, nullptr);
+    bucket_scatter_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->bounds, b->fill, b->order, nullptr,
+                                             nullptr);
     return cudaGetLastError();
 }
 
+// Plans of wfa_ring.cu.  The buckets are classes of scaled limits, each at most a quarter above the one below, so that
+// a warp's pairs have alike windows and shared memory is sized for them.  The classes from kBoundScore on run a bound
+// pass first; the pairs are then bucketed again by min(limit, bound), and every class has one exact launch with the
+// lanes per pair that its windows suit, four classes at a time on streams of their own (the tail of one class, a few
+// long pairs, runs beside the next ones).
+constexpr int64_t kBoundScore = 40;
+
+WfaPlan class_plan(const aim_batch* b, int k) {   // bucket k
+    WfaPlan p = b->plan;
+    p.smax = std::min<int64_t>(p.smax, b->bp.edge[b->bp.nclasses - 1 - k]);
+    const int64_t minc = std::min<int64_t>(p.x, p.oe);
+    p.runs_cap = (int)std::min<int64_t>(p.runs_cap, 2 * (p.smax / std::max<int64_t>(minc, 1)) + 1);
+    p.runs_bytes = align_up((size_t)p.runs_cap * sizeof(uint32_t), 16);
+    return p;
+}
+
+const TuneChoice* cached_choice(const aim_batch* b, int k) {
+    if (!b->ctx->tune_cache) return nullptr;
+    auto& c = tune_cache(b->ctx);
+    const auto it = c.find(TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, b->pen.band, k, b->plan.smax));
+    return it == c.end() ? nullptr : &it->second;
+}
+
+bool ring_bounded(const aim_batch* b) {
+    for (int k = 0; k < b->bp.nclasses; ++k)
+        if (b->bound1[k]) return true;
+    return false;
+}
+
+// the bound passes, and the counts of the classes that min(limit, bound) puts the pairs in
+cudaError_t enqueue_bounds(aim_batch* b, cudaStream_t st, bool* fits) {
+    *fits = true;
+    const int sms = b->ctx->num_sms;
+    cudaError_t e = cudaMemsetAsync(b->bound, 0xff, (size_t)b->num_pairs * sizeof(int32_t), st);   // -1: none
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->rclaims, 0, kBuckets * sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->rcounts, 0, kBuckets * sizeof(uint32_t), st);
+    for (int j = 0; j < b->bp.ngroups && e == cudaSuccess; ++j) {
+        if (!b->gbound[j]) continue;
+        WfaPlan bp = b->plan;
+        bp.bound = b->bound;
+        bp.bound_pass = 1;
+        if (b->gbound[j] == 1) {
+            e = launch_wfa_bound(bp, b->P, b->r.lim, b->O, b->order, b->gbounds + j, b->rclaims + j, sms, st);
+        } else {
+            int w = 0;
+            const size_t wb = wfa_warp_bytes(b->gbound[j], wfa_bound_pair_bytes(b->plan));
+            e = launch_wfa_buckets(bp, b->P, b->r.lim, b->O, b->order, b->gbounds + j, &b->gbound[j], 1, wb, b->scratch,
+                                   b->scratch_bytes, b->rclaims + j, sms, st, &w);
+            *fits = *fits && (e != cudaSuccess || w > 0);
+        }
+    }
+    if (e != cudaSuccess) return e;
+    const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)sms * 8);
+    bucket_count_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rcounts, nullptr, b->bound);
+    return cudaGetLastError();
+}
+
+cudaError_t enqueue_ring(aim_batch* b, cudaStream_t st, int* warps) {
+    *warps = 0;
+    const int nc = b->bp.nclasses, sms = b->ctx->num_sms;
+    const bool bounded = ring_bounded(b);
+    const uint32_t *order = b->order, *bounds = b->bounds;
+    uint32_t* claims = b->claims;
+    cudaError_t e = cudaSuccess;
+    if (bounded) {
+        bool fits = true;
+        e = enqueue_bounds(b, st, &fits);
+        if (e != cudaSuccess || !fits) return e;
+        const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)sms * 8);
+        bucket_scan_kernel<<<1, 32, 0, st>>>(b->rcounts, b->rbounds, b->rfill, b->cclaims, b->bp, nullptr);
+        bucket_scatter_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rbounds, b->rfill, b->rorder, nullptr,
+                                                      b->bound);
+        e = cudaGetLastError();
+        order = b->rorder; bounds = b->rbounds; claims = b->cclaims;
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(b->fork, st);
+    const int ns = std::min(nc, 4);
+    for (int i = 0; i < ns && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(b->side[i], b->fork, 0);
+    bool all = true;
+    for (int k = 0; k < nc && e == cudaSuccess; ++k) {
+        WfaPlan p = class_plan(b, k);
+        if (bounded) p.bound = b->bound;
+        int w = 0;
+        e = launch_wfa_ring(p, b->groups[k], b->P, b->r.lim, b->O, order, bounds + k, b->scratch + b->class_at[k],
+                            b->class_bytes[k], claims + k, sms, b->side[k % ns], &w);
+        all = all && w > 0;
+        *warps = std::max(*warps, w);
+    }
+    for (int i = 0; i < ns && e == cudaSuccess; ++i) {
+        e = cudaEventRecord(b->joined[i], b->side[i]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, b->joined[i], 0);
+    }
+    if (!all) *warps = 0;
+    return e;
+}
+
+// The classes' lanes, bound passes and parts of the scratch; false if some class fits nowhere.  A class wants a full
+// grid's scratch; when all together want more than there is each gets its share, at least eight blocks' worth.
+bool ring_layout(aim_batch* b) {
+    const int nc = b->bp.nclasses;
+    size_t want[kBuckets], least[kBuckets], total = 0, floor = 0;
+    for (int k = 0; k < kBuckets; ++k) {
+        b->groups1[k] = b->bound1[k] = 0;
+        if (k >= nc) { b->groups[k] = 32; continue; }
+        const WfaPlan p = class_plan(b, k);
+        // cached choices (an earlier plan's, or imported), else the rule of wfa_ring.cu for a batch that fills the
+        // device, and a bound pass with one pair per lane, or a warp per pair for longer reads
+        const TuneChoice* cached = cached_choice(b, k);
+        b->groups[k] = cached && ring_fits(p, std::get<0>(*cached), b->max_length, b->scratch_bytes)
+                           ? std::get<0>(*cached)
+                           : ring_group(p, b->max_length, 0x7fffffffu, b->ctx->num_sms, b->scratch_bytes);
+        const bool lanes = bound_lanes_ok(b->plan, b->max_length);
+        const int mode = b->ctx->batch_bound;
+        int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore ? 0 : lanes ? 1 : 32;
+        if (mode == 0 && cached && (std::get<2>(*cached) != 1 || lanes)) gb = std::get<2>(*cached);
+        b->bound1[k] = mode == 2 || b->max_length > kMaxWfaLength16 ? 0 : gb;
+        want[k] = b->groups[k] ? ring_full_scratch(p, b->groups[k], b->max_length, b->ctx->num_sms) : 0;
+        if (!want[k]) return false;
+        least[k] = align_up(ring_warp_bytes(p, b->groups[k], b->max_length) * (b->groups[k] > 32 ? 8 : 32), 256);
+        want[k] = std::max(align_up(want[k], 256), least[k]);
+        total += want[k];
+        floor += least[k];
+    }
+    if (floor > b->scratch_bytes) return false;
+    size_t at = 0;
+    const size_t spare = b->scratch_bytes - floor, over = total - floor;
+    for (int k = 0; k < nc; ++k) {
+        // what it wants beyond the least, or that scaled to what is there (or up: arenas hold several rounds)
+        const double share = over ? (double)(want[k] - least[k]) / (double)over : 0.0;
+        b->class_at[k] = at;
+        b->class_bytes[k] = least[k] + ((size_t)(share * (double)spare) & ~(size_t)255);
+        at += b->class_bytes[k];
+    }
+    // consecutive classes with the same bound pass are one queue range for it
+    int ng = 0;
+    for (int k = 0; k < nc; ++k)
+        if (k == 0 || b->bound1[k] != b->gbound[ng - 1]) {
+            b->bp.gstart[ng] = (int8_t)k;
+            b->gbound[ng++] = b->bound1[k];
+        }
+    b->bp.gstart[ng] = (int8_t)kBuckets;
+    b->bp.ngroups = ng;
+    return true;
+}
+
+// Classes for the plan; false if the batch is not one for wfa_ring.cu (it then keeps the buckets of wfa.cu).
+bool plan_ring(aim_batch* b) {
+    if (!ring_ok(b->plan, b->max_length) || b->ctx->batch_compact == 1) return false;
+    int nc = 0;
+    for (double edge = 24.0; nc < kBuckets; edge *= 1.25) {
+        const bool last = (int64_t)edge >= b->plan.smax || nc == kBuckets - 1;
+        b->bp.edge[nc++] = (int32_t)(last ? b->plan.smax : (int64_t)edge);
+        if (last) break;
+    }
+    b->bp.nclasses = nc;
+    if (ring_layout(b)) return true;
+    b->bp.nclasses = b->bp.ngroups = 0;
+    return false;
+}
+
+// Merges classes that the batch at hand fills with fewer pairs than its launch runs at once (a class's launch takes at
+// least as long as its longest pair): heaviest first, a class takes in the ones below it until it has that many.
+// `counts`: pairs per class under min(limit, bound).
+void ring_merge(aim_batch* b, const uint32_t* counts) {
+    int32_t edge[kBuckets];
+    int nc = 0;
+    for (int k = 0; k < b->bp.nclasses;) {   // heaviest first
+        const WfaPlan p = class_plan(b, k);
+        const size_t units = ring_full_scratch(p, b->groups[k], b->max_length, b->ctx->num_sms) /
+                             ring_warp_bytes(p, b->groups[k], b->max_length);
+        const size_t need = units * (b->groups[k] > 32 ? 1 : (size_t)(32 / b->groups[k]));
+        size_t have = 0;
+        edge[nc++] = b->bp.edge[b->bp.nclasses - 1 - k];
+        while (k < b->bp.nclasses && have < need) have += counts[k++];
+    }
+    for (int c = 0; c < nc; ++c) b->bp.edge[c] = edge[nc - 1 - c];
+    b->bp.nclasses = nc;
+}
+
 cudaError_t enqueue_align(aim_batch* b, cudaStream_t st, int* warps) {
+    if (b->ring) return enqueue_ring(b, st, warps);
     if (!b->two_pass) {
         // one launch per group of buckets sharing lanes per pair (and bound-pass lanes), each over one contiguous
         // queue range; a group with a bound pass first runs it over the same range (claim counters of their own)
@@ -322,9 +531,10 @@ cudaError_t enqueue_align(aim_batch* b, cudaStream_t st, int* warps) {
     e = cudaMemsetAsync(b->rcounts, 0, kBuckets * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)b->ctx->num_sms * 8);
-    bucket_count_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rcounts, b->O.flags);
+    bucket_count_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rcounts, b->O.flags, nullptr);
     bucket_scan_kernel<<<1, 32, 0, st>>>(b->rcounts, b->rbounds, b->rfill, b->rclaims, b->bp, nullptr);
-    bucket_scatter_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rbounds, b->rfill, b->rorder, b->O.flags);
+    bucket_scatter_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rbounds, b->rfill, b->rorder, b->O.flags,
+                                             nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     WfaPlan retry = b->plan;
@@ -448,6 +658,11 @@ void free_batch(aim_batch* b) {
     if (!b) return;
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
+    for (int i = 0; i < 4; ++i) {
+        if (b->side[i]) cudaStreamDestroy(b->side[i]);
+        if (b->joined[i]) cudaEventDestroy(b->joined[i]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     if (b->ev_start) cudaEventDestroy(b->ev_start);
     if (b->ev_stop) cudaEventDestroy(b->ev_stop);
     if (b->stream) cudaStreamDestroy(b->stream);
@@ -513,7 +728,7 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
     // owned memory: packed sequences, flags, bucket arrays, order, scratch
     const size_t seq_bytes = align_up((size_t)num_pairs * b->stride * 8, 256);
     const size_t flag_bytes = align_up(num_pairs, 256);
-    const size_t small_bytes = align_up(10 * (kBuckets + 1) * sizeof(uint32_t), 256);
+    const size_t small_bytes = align_up(11 * (kBuckets + 1) * sizeof(uint32_t), 256);
     const size_t order_bytes = align_up((size_t)num_pairs * sizeof(uint32_t), 256);
     b->scratch_bytes = ext_scratch ? ext_scratch_bytes : scratch_bytes ? scratch_bytes : ctx->ws_bytes;
     b->mem_bytes = 2 * seq_bytes + 2 * flag_bytes + small_bytes + 3 * order_bytes + (ext_scratch ? 0 : b->scratch_bytes);
@@ -529,7 +744,7 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
     b->claims = sm + 3 * (kBuckets + 1); b->trial_bounds = sm + 4 * (kBuckets + 1);
     b->rcounts = sm + 5 * (kBuckets + 1); b->rbounds = sm + 6 * (kBuckets + 1);
     b->rfill = sm + 7 * (kBuckets + 1); b->rclaims = sm + 8 * (kBuckets + 1);
-    b->gbounds = sm + 9 * (kBuckets + 1);
+    b->gbounds = sm + 9 * (kBuckets + 1); b->cclaims = sm + 10 * (kBuckets + 1);
     b->order = reinterpret_cast<uint32_t*>(p); p += order_bytes;
     b->rorder = reinterpret_cast<uint32_t*>(p); p += order_bytes;
     b->bound = reinterpret_cast<int32_t*>(p); p += order_bytes;
@@ -540,12 +755,34 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
     e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) { free_batch(b); return cuda_status(e); }
 
+    b->ring = plan_ring(b);
+
     // prepare once (synchronously) to see the bucket sizes, then tune
     e = enqueue_prepare(b, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess) e = cudaMemcpy(b->host_counts, b->counts, sizeof(b->host_counts), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) { free_batch(b); return cuda_status(e); }
-    if (autotune) {
+    if (b->ring) {
+        // classes to suit this batch: its counts after the bound passes, where there are any
+        uint32_t counts[kBuckets];
+        std::memcpy(counts, b->host_counts, sizeof(counts));
+        if (ring_bounded(b)) {
+            bool fits = true;
+            e = enqueue_bounds(b, b->stream, &fits);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+            if (e == cudaSuccess) e = cudaMemcpy(counts, b->rcounts, sizeof(counts), cudaMemcpyDeviceToHost);
+        }
+        ring_merge(b, counts);
+        if (e == cudaSuccess && !ring_layout(b)) e = cudaErrorUnknown;   // (fewer classes need no more than before)
+        if (e == cudaSuccess) e = enqueue_prepare(b, b->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+        if (e == cudaSuccess) e = cudaMemcpy(b->host_counts, b->counts, sizeof(b->host_counts), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) { free_batch(b); return cuda_status(e); }
+        for (int k = 0; autotune && k < b->bp.nclasses; ++k)
+            if (b->host_counts[k])
+                tune_cache(ctx)[TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, pen->band, k, b->plan.smax)] =
+                    TuneChoice(b->groups[k], 0, b->bound1[k]);
+    } else if (autotune) {
         rc = aim::autotune(b);
         if (rc) { free_batch(b); return rc; }
     } else {
@@ -563,11 +800,11 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
         }
     }
     // buckets empty at planning keep one pair per warp, so their worst case does not shrink the grid
-    for (int k = 0; k < kBuckets; ++k)
+    for (int k = 0; k < kBuckets && !b->ring; ++k)
         if (!b->host_counts[k]) { b->groups[k] = 32; b->groups1[k] = 0; b->bound1[k] = 0; }
     // scratch per warp of the full pass: the largest need over all buckets (a replay may see a different mix)
     size_t wb = 0;
-    for (int k = 0; k < kBuckets; ++k)
+    for (int k = 0; k < kBuckets && !b->ring; ++k)
         wb = std::max(wb, wfa_warp_bytes(b->groups[k], bucket_pair_bytes(b->plan, k, b->groups[k])));
     b->warp_bytes = wb;
     if (wb > b->scratch_bytes) { free_batch(b); return AIM_ERR_NOMEM; }
@@ -576,7 +813,19 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
     b->two_pass = false;
     for (int k = 0; k < kBuckets; ++k) b->two_pass |= b->groups1[k] != 0;
     b->warp_bytes1 = wb;
-    if (b->two_pass) {
+    if (b->ring) {
+        for (int i = 0; i < 4; ++i) {
+            if (cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking) != cudaSuccess ||
+                cudaEventCreateWithFlags(&b->joined[i], cudaEventDisableTiming) != cudaSuccess) {
+                free_batch(b);
+                return AIM_ERR_CUDA;
+            }
+        }
+        if (cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess) {
+            free_batch(b);
+            return AIM_ERR_CUDA;
+        }
+    } else if (b->two_pass) {
         size_t wb1 = 0;
         for (int k = 0; k < kBuckets; ++k) {
             if (!b->host_counts[k]) continue;
@@ -746,7 +995,7 @@ int aim_tune_import(aim_ctx* ctx, const char* text) {
         const auto lanes_ok = [](int v, bool zero) { return (zero && v == 0) || v == 1 || v == 2 || v == 4 ||
                                                             v == 8 || v == 16 || v == 32 || v == 256; };
         if (bucket < 0 || bucket >= aim::kBuckets || !lanes_ok(g, false) || !lanes_ok(g1, true) ||
-            !(gb == 0 || gb == 4 || gb == 8 || gb == 16 || gb == 32))
+            !(gb == 0 || gb == 1 || gb == 4 || gb == 8 || gb == 16 || gb == 32))
             return AIM_ERR_ARG;
         parsed.emplace_back(aim::TuneKey(x, o, e, band, bucket, (int64_t)smax), aim::TuneChoice(g, g1, gb));
         p += used;

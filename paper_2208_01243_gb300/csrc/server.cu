@@ -105,6 +105,7 @@ struct Request {
     std::vector<uint32_t> order;     // pair indices grouped into jobs (heaviest job first)
     struct Job {
         uint32_t begin, count;
+        uint32_t max_len;    // longest read or target of its pairs
         WfaPlan plan;
         int group;
         int bound_group;     // lanes per pair of a bound pass before the exact one (0: none)
@@ -312,7 +313,7 @@ int launch_request(aim_server* s, Request* r) {
         if (e != cudaSuccess) break;
         PairsView P{reinterpret_cast<const uint64_t*>(d + L.packed_r), reinterpret_cast<const uint64_t*>(d + L.packed_t),
                     nullptr, nullptr, reinterpret_cast<const uint32_t*>(d + L.rl),
-                    reinterpret_cast<const uint32_t*>(d + L.tl), d + L.bad_r, d + L.bad_t, job.count, r->max_len};
+                    reinterpret_cast<const uint32_t*>(d + L.tl), d + L.bad_r, d + L.bad_t, job.count, job.max_len};
         P.stride = L.stride;
         uint8_t* slice = s->dev_scratch + r->scratch_off + job.slice_off;
         WfaPlan exact = job.plan;
@@ -325,7 +326,10 @@ int launch_request(aim_server* s, Request* r) {
             bp.bound_pass = 1;
             int bg = job.bound_group;
             const size_t bwb = wfa_warp_bytes(bg, wfa_bound_pair_bytes(job.plan));
-            if (8 * bwb <= job.slice_bytes) {
+            if (bound_lanes_ok(job.plan, job.max_len)) {   // one pair per lane, no scratch
+                e = launch_wfa_bound(bp, P, lim, O, order + job.begin, nullptr, counter + 32, s->num_sms, js);
+                exact.bound = bp.bound;
+            } else if (8 * bwb <= job.slice_bytes) {
                 e = launch_wfa_buckets(bp, P, lim, O, order + job.begin, nullptr, &bg, 1, bwb, slice, job.slice_bytes,
                                        counter + 32, s->num_sms, js, &warps);
                 if (e == cudaSuccess && warps > 0) exact.bound = bp.bound;
@@ -558,7 +562,7 @@ int aim_server_submit(aim_server* s, const aim_request* q, uint64_t* ticket) {
             ++j;
         }
         Request::Job job;
-        job.begin = i; job.count = j - i;
+        job.begin = i; job.count = j - i; job.max_len = jl;
         job.plan = plan_wfa(s->costs, s->pen.band, jl, (int64_t)jme * ecost);
         job.group = wfa_default_group(job.plan, jl);
         job.warp_bytes = wfa_warp_bytes(job.group, wfa_pair_bytes(job.plan, job.group));
@@ -570,7 +574,8 @@ int aim_server_submit(aim_server* s, const aim_request* q, uint64_t* ticket) {
         // diagonals), where the batched form's tuner keeps one: 4 lanes per pair before groups of up to 32 lanes,
         // 16 before whole blocks.  Results are the exact pass's either way.
         const int key = keyed[i].first, kc = 7 - key / 4, wc = 3 - key % 4;
-        job.bound_group = kc >= 5 && wc == 3 && r->max_len <= kMaxWfaLength16 ? (job.group > 32 ? 16 : 4) : 0;
+        // (one pair per lane where wfa_bound.cu takes the job)
+        job.bound_group = kc >= 5 && wc == 3 && jl <= kMaxWfaLength16 ? (job.group > 32 ? 16 : 4) : 0;
         // warps wanted: every pair in flight at once (a 256-lane group uses 8 warps), within the device's capacity
         const size_t want = job.group > 32 ? (size_t)job.count * (job.group / 32)
                                            : (job.count + (32 / job.group) - 1) / (size_t)(32 / job.group);

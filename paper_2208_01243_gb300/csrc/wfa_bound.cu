@@ -1,0 +1,218 @@
+// Bound pass with one pair per lane: a pruned forward pass whose end score bounds a pair's optimum from above (see
+// wfa.cu), for reads short enough that a warp's 32 pairs keep their sequences in shared memory.
+//
+// The pass follows the best alignment with a window of nine diagonals kept whole in registers, in wfa_ring.cu's form
+// (M~ of the last four scores, J and K per diagonal; E == 1, X and O up to 4): no range, record or reduction, and
+// neighbours are the lane's own registers.  After a score the window moves one diagonal towards the entry closest to
+// the end, by max(n - v, m - h), once that entry is two diagonals off its centre.  What leaves the window is lost and
+// what enters it starts invalid, so every value is an offset that some alignment of that cost reaches, and the score
+// at which the closest entry has nothing left is the cost of an alignment.  A pair whose window loses the end by its
+// limit gets no bound (-1), and its exact pass runs under the limit alone.
+// Pairs end at scores far apart, so idle lanes take new pairs while the others carry on (kRefill).  1M pairs of
+// 100-1,000 bp, 1-10 %: 3.8 ms in step with the slowest lane (16 of 32 lanes at work), 2.3 ms with refills; wfa.cu's
+// groups of four lanes took about 11 ms over the same pairs.
+#include <algorithm>
+#include <cstdint>
+
+#include "wfa_common.cuh"
+
+namespace aim {
+namespace {
+
+constexpr int kBoundWarps = 2;    // per block
+constexpr int kWin = 9, kMid = kWin / 2;
+constexpr int kRefill = 8;        // idle lanes that call for a refill
+
+struct BoundArgs {
+    WfaArgs w;
+    uint32_t seq_words;
+    uint32_t smem_warp;
+    uint32_t sel_x, sel_o;
+};
+
+extern __shared__ __align__(16) uint8_t s_bound[];
+
+__global__ void __launch_bounds__(32 * kBoundWarps) wfa_bound_kernel(BoundArgs r) {
+    const WfaArgs& a = r.w;
+    const int lane = (int)(threadIdx.x & 31);
+    const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (gwarp >= a.nwarps) return;
+    uint32_t* sp = reinterpret_cast<uint32_t*>(s_bound + (size_t)(threadIdx.x >> 5) * r.smem_warp) + 32 + lane;
+    uint32_t* st = sp + r.seq_words * 32;
+    const int O = a.OE - 1;
+    const uint32_t begin = a.bounds ? a.bounds[0] : 0;
+    const uint32_t end = a.bounds ? a.bounds[1] : a.P.num_pairs;
+    uint32_t ml[kWin], mu[kWin], jk[kWin];   // M~ of scores s-1, s-2 and s-3, s-4; J, K
+#pragma unroll
+    for (int i = 0; i < kWin; ++i) ml[i] = mu[i] = jk[i] = ~0u;
+    uint32_t pi = 0, cells = 0, windows = 0;
+    int n = 0, m = 0, S = 0, klo = 0, khi = 0, s = 0;
+    int mid = 0;        // the window's middle diagonal
+    bool run = false;   // this lane's pair is under way
+    bool more = true;   // the queue may hold pairs
+    unsigned long long st_cells = 0, st_windows = 0;
+
+    for (;;) {
+        // new pairs for the idle lanes once there are eight of them: pairs end at very different scores, and a refill
+        // costs the warp as much for one lane as for many
+        const uint32_t idle = __ballot_sync(kFull, !run);
+        if (more && __popc(idle) >= kRefill) {
+            uint32_t pos = 0;
+            if (lane == 0) pos = atomicAdd(a.counters, (uint32_t)__popc(idle));
+            pos = __shfl_sync(kFull, pos, 0);
+            more = begin < end && pos + (uint32_t)__popc(idle) < end - begin;
+            const uint32_t q = pos + (uint32_t)__popc(idle & ((1u << lane) - 1u));
+            bool fresh = !run && begin < end && q < end - begin;
+            if (fresh) {
+                pi = a.order ? a.order[begin + q] : begin + q;
+                n = (int)a.P.read_len[pi];
+                m = (int)a.P.target_len[pi];
+                const int kend = m - n;
+                const int64_t lim = pair_limit(a.L, pi);
+                const int64_t S64 = lim / a.g;
+                S = (int)(S64 > a.smax ? a.smax : S64);
+                klo = a.band >= 0 ? max(-n, -a.band) : -n;
+                khi = a.band >= 0 ? min(m, a.band) : m;
+                // (the exact pass reports the others)
+                fresh = !pair_bad(a.P, pi) && (uint32_t)n <= a.P.max_length && (uint32_t)m <= a.P.max_length && lim != -2 &&
+                        kend >= klo && kend <= khi && (kend == 0 || abs(kend) + O <= S);
+                if (!fresh) a.bound[pi] = -1;
+            }
+            if (fresh) {
+                const uint64_t* Pw = read_words(a.P, pi);
+                const uint64_t* Tw = target_words(a.P, pi);
+#pragma unroll 4
+                for (int w = 0; w < (n + 31) >> 5; ++w) {
+                    const uint64_t x = __ldg(Pw + w);
+                    sp[2 * w * 32] = (uint32_t)(x >> 32); sp[(2 * w + 1) * 32] = (uint32_t)x;
+                }
+#pragma unroll 4
+                for (int w = 0; w < (m + 31) >> 5; ++w) {
+                    const uint64_t x = __ldg(Tw + w);
+                    st[2 * w * 32] = (uint32_t)(x >> 32); st[(2 * w + 1) * 32] = (uint32_t)x;
+                }
+                const int m0 = match_on<32>(sp, st, 0, 0, min(n, m));
+#pragma unroll
+                for (int i = 0; i < kWin; ++i) ml[i] = mu[i] = jk[i] = ~0u;
+                ml[kMid] = (uint32_t)m0 | 0xffff0000u;
+                mid = 0;
+                s = 0;
+                ++cells; ++windows;
+                run = true;
+                if (n == m && m0 == m) { a.bound[pi] = 0; run = false; }
+            }
+            __syncwarp();
+        }
+        if (!__any_sync(kFull, run)) {
+            if (more) continue;
+            break;
+        }
+        // one score of every pair under way
+        int move = 0;
+        if (run) {
+            ++s;
+            if (s > S) { a.bound[pi] = -1; run = false; }
+        }
+        if (run) {
+            uint32_t before = ~0u;   // J, K of the diagonal below, from score s-1
+            int best = 1 << 30;      // (distance to the end) * 16 + place
+#pragma unroll
+            for (int i = 0; i < kWin; ++i) {
+                const int k = mid - kMid + i;
+                const uint32_t left = before, right = i + 1 < kWin ? jk[i + 1] : ~0u;
+                before = jk[i];
+                const bool in = k >= klo && k <= khi;
+                const int hmax = in ? min(m, n + k) : -1, room = max(hmax, 0);
+                const int mo = prmt(ml[i], mu[i], r.sel_o);
+                int mis = prmt(ml[i], mu[i], r.sel_x);
+                int ins = prmt(right, 0u, 0x9910u), del = prmt(left, 0u, 0xbb32u);
+                mis = (unsigned)mis < (unsigned)room ? mis + 1 : -1;
+                del = (unsigned)del < (unsigned)room ? del + 1 : -1;
+                ins = ins <= hmax ? ins : -1;
+                int mv = max(mis, max(ins, del));
+                if (mv >= 0) {
+                    const int rem = hmax - mv;
+                    const uint32_t x = window16<32>(sp, mv - k) ^ window16<32>(st, mv);
+                    int len = min(__clz((int)x) >> 1, rem);
+                    ++windows;
+                    if (x == 0 && rem > 16) {
+                        len = 16 + match_on<32>(sp, st, mv - k + 16, mv + 16, rem - 16);
+                        windows += (uint32_t)len >> 5;
+                    }
+                    mv += len;
+                    best = min(best, (max(n + k, m) - mv) * 16 + i);
+                }
+                mu[i] = (uint32_t)prmt(ml[i], mu[i], 0x5432u);
+                ml[i] = (uint32_t)prmt((uint32_t)mv, ml[i], 0x5410u);
+                jk[i] = (uint32_t)prmt((uint32_t)max(mo, ins), (uint32_t)max(mo, del), 0x5410u);
+            }
+            cells += kWin;
+            if (best < 16) { a.bound[pi] = s; run = false; }   // nothing left on either sequence
+            else if (best < (1 << 30)) move = (best & 15) >= kMid + 2 ? 1 : (best & 15) <= kMid - 2 ? -1 : 0;
+        }
+        if (__any_sync(kFull, move != 0)) {
+            mid += move;
+            uint32_t l = ~0u, u = ~0u, j = ~0u;   // the place below, before it moved
+#pragma unroll
+            for (int i = 0; i < kWin; ++i) {
+                const uint32_t nl = i + 1 < kWin ? ml[i + 1] : ~0u, nu = i + 1 < kWin ? mu[i + 1] : ~0u,
+                               nj = i + 1 < kWin ? jk[i + 1] : ~0u;
+                const uint32_t cl = ml[i], cu = mu[i], cj = jk[i];
+                ml[i] = move > 0 ? nl : move < 0 ? l : cl;
+                mu[i] = move > 0 ? nu : move < 0 ? u : cu;
+                jk[i] = move > 0 ? nj : move < 0 ? j : cj;
+                l = cl; u = cu; j = cj;
+            }
+        }
+        if (cells >= 1u << 30) { st_cells += cells; st_windows += windows; cells = windows = 0; }
+    }
+    st_cells += cells;
+    st_windows += windows;
+    warp_stat_add(a.O.stats, 0, st_cells, (uint32_t)lane);
+    warp_stat_add(a.O.stats, 1, st_windows, (uint32_t)lane);
+}
+
+uint32_t bound_seq_words(uint32_t max_length) { return 2 * ((max_length + 31) / 32) + 2; }
+// (a word of room before the copies: nothing reads there, an index below them would)
+size_t bound_smem(uint32_t max_length) { return 128 + (size_t)bound_seq_words(max_length) * 256; }
+
+constexpr size_t kLaneBoundSmem = 40u << 10;   // shared memory per warp: 5 warps on an SM
+
+}  // namespace
+
+bool bound_lanes_ok(const WfaPlan& p, uint32_t max_length) {
+    const int O = p.oe - p.e;
+    return p.e == 1 && O >= 1 && O <= 4 && p.x <= 4 && max_length <= kMaxWfaLength16 && p.smax < (1 << 26) &&
+           bound_smem(max_length) <= kLaneBoundSmem;
+}
+
+cudaError_t launch_wfa_bound(const WfaPlan& plan, const PairsView& P, const LimitView& L, const OutView& O,
+                             const uint32_t* order, const uint32_t* bounds, uint32_t* counters, int num_sms,
+                             cudaStream_t st) {
+    if (P.num_pairs == 0) return cudaSuccess;
+    BoundArgs r{};
+    WfaArgs& a = r.w;
+    a.X = plan.x; a.OE = plan.oe; a.E = plan.e; a.g = plan.g; a.smax = plan.smax; a.band = plan.band;
+    a.P = P; a.L = L; a.O = O;
+    a.order = order; a.bounds = bounds; a.counters = counters; a.nbuckets = 1;
+    a.bound = plan.bound;
+    r.seq_words = bound_seq_words(P.max_length);
+    r.smem_warp = (uint32_t)bound_smem(P.max_length);
+    auto sel = [](int d) { const uint32_t b = 2u * (uint32_t)(d - 1); return b | ((b + 1) << 4) | ((b + 9) << 8) | ((b + 9) << 12); };
+    r.sel_x = sel(plan.x);
+    r.sel_o = sel(plan.oe - plan.e);
+    const size_t smem = (size_t)kBoundWarps * r.smem_warp;
+    cudaError_t e = cudaFuncSetAttribute(wfa_bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kBoundWarps * kLaneBoundSmem));
+    if (e != cudaSuccess) return e;
+    int bps = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, wfa_bound_kernel, 32 * kBoundWarps, smem);
+    if (e != cudaSuccess) return e;
+    size_t warps = (size_t)num_sms * std::max(bps, 1) * kBoundWarps;
+    warps = std::min(warps, ((size_t)P.num_pairs + 31) / 32);
+    a.nwarps = (uint32_t)warps;
+    wfa_bound_kernel<<<(unsigned)((warps + kBoundWarps - 1) / kBoundWarps), 32 * kBoundWarps, smem, st>>>(r);
+    return cudaGetLastError();
+}
+
+}  // namespace aim

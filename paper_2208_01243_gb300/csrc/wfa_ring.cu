@@ -182,8 +182,21 @@ __device__ uint32_t ring_traceback(const WfaArgs& a, const uint8_t* rounds, cons
         const int at = H::m(opening);
         return at >= 0 && at + more <= hmax ? at + more : -1;
     };
+    // matching bases back from (v, h), as far as one window shows
+    auto match_back = [&](int v, int h) -> int {
+        if (seqs_kept) {   // 16 bases back; before the start the window's earlier bases are not looked at
+            const int back = min(min(v, h), 16);
+            const uint32_t x = window16<P>(sp, max(v - 16, 0)) >> (v < 16 ? 2 * (16 - v) & 31 : 0);
+            const uint32_t y = window16<P>(st, max(h - 16, 0)) >> (h < 16 ? 2 * (16 - h) & 31 : 0);
+            const uint32_t d = x ^ y;
+            return min(d ? (__ffs((int)d) - 1) >> 1 : 16, back);
+        }
+        const int back = min(min(v, h), 32);
+        const uint64_t d = back ? window_ending(Pg, nwP, v - 1) ^ window_ending(Tg, nwT, h - 1) : 1ull;
+        return min(d ? (__ffsll((long long)d) - 1) >> 1 : 32, back);
+    };
     int v = n, h = m, cM = q.final_s, cI = q.final_s, cD = q.final_s;
-    while (v > 0 || h > 0) {
+    while ((v > 0 || h > 0) && ok) {
         const int j = h - v - q.koff;
         const auto eX = entry(cM - X, j), eM = entry(cM, j);
         typename H::T eI, eD, oI, oD;
@@ -193,51 +206,48 @@ __device__ uint32_t ring_traceback(const WfaArgs& a, const uint8_t* rounds, cons
             eI = entry(cI - 1, j + 1); oI = entry(cI - OE, j + 1);
             eD = entry(cD - 1, j - 1); oD = entry(cD - OE, j - 1);
         }
-        const int avail = min(v, h);
-        int same;   // matching bases back from (v, h), as far as the window shows
-        if (seqs_kept) {   // 16 bases back; before the start the window's earlier bases are not looked at
-            const int back = min(avail, 16);
-            const uint32_t x = window16<P>(sp, max(v - 16, 0)) >> (v < 16 ? 2 * (16 - v) & 31 : 0);
-            const uint32_t y = window16<P>(st, max(h - 16, 0)) >> (h < 16 ? 2 * (16 - h) & 31 : 0);
-            const uint32_t d = x ^ y;
-            same = min(d ? (__ffs((int)d) - 1) >> 1 : 16, back);
-        } else {
-            const int back = min(avail, 32);
-            const uint64_t d = back ? window_ending(Pg, nwP, v - 1) ^ window_ending(Tg, nwT, h - 1) : 1ull;
-            same = min(d ? (__ffsll((long long)d) - 1) >> 1 : 32, back);
-        }
-        const bool diag = avail > 0, match = same > 0;
-        if (diag && !match && H::m(eX) >= h - 1) {
-            cM = cI = cD = cM - X; --v; --h;
-            wr.put(kOpMismatch, 1);
-            continue;
-        }
+        int same = match_back(v, h);
+        const int mX = H::m(eX), mM = H::m(eM);
         int vI, vD;
         if constexpr (FMT == kWhole) { vI = H::i(eI); vD = H::d(eD); }
         else { vI = ins_of(cI, j, eI, oI); vD = del_of(cD, j, eD, oD); }
-        if (v > 0 && vI >= h) {
-            const int c = cI;
-            cM = cD = c - OE; cI = c - 1; --v;
-            wr.put(kOpIns, 1);
-        } else if (h > 0 && vD >= h) {
-            const int c = cD;
-            cM = cI = c - OE; cD = c - 1; --h;
-            wr.put(kOpDel, 1);
-        } else if (match && H::m(eM) >= h - 1) {
-            // a longer run is taken window by window: I~ and D~ of this score stop it at the same offset
-            if constexpr (FMT == kWhole) { vI = H::i(eM); vD = H::d(eM); }
-            else {
-                if (cI != cM) vI = ins_of(cM, j, entry(cM - 1, j + 1), entry(cM - OE, j + 1));
-                if (cD != cM) vD = del_of(cM, j, entry(cM - 1, j - 1), entry(cM - OE, j - 1));
+        // A run of matches leaves the diagonal and the score, and so the entries, as they are: the edit before it is
+        // decided from the same loads.
+        for (;;) {
+            const bool diag = v > 0 && h > 0, match = same > 0;
+            if (diag && !match && mX >= h - 1) {
+                cM = cI = cD = cM - X; --v; --h;
+                wr.put(kOpMismatch, 1);
+                break;
             }
+            if (v > 0 && vI >= h) {
+                const int c = cI;
+                cM = cD = c - OE; cI = c - 1; --v;
+                wr.put(kOpIns, 1);
+                break;
+            }
+            if (h > 0 && vD >= h) {
+                const int c = cD;
+                cM = cI = c - OE; cD = c - 1; --h;
+                wr.put(kOpDel, 1);
+                break;
+            }
+            if (!match || mM < h - 1) { ok = false; break; }
+            if (cI != cM || cD != cM) {   // I~ and D~ of M~'s own score from here on
+                if constexpr (FMT == kWhole) { vI = H::i(eM); vD = H::d(eM); }
+                else {
+                    if (cI != cM) vI = ins_of(cM, j, entry(cM - 1, j + 1), entry(cM - OE, j + 1));
+                    if (cD != cM) vD = del_of(cM, j, entry(cM - 1, j - 1), entry(cM - OE, j - 1));
+                }
+                cI = cD = cM;
+            }
+            // to where a gap may end or the window does: a longer run is taken window by window
             const int run = min(same, h - max(vI, vD));
             if (run < 1) { ok = false; break; }
             v -= run; h -= run;
-            cI = cD = cM;
             wr.put(kOpMatch, (uint32_t)run);
-        } else {
-            ok = false;
-            break;
+            if (v == 0 && h == 0) break;
+            same = match_back(v, h);
         }
     }
     wr.flush();
@@ -648,6 +658,34 @@ int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int nu
     return ring_fits(p, G, max_length, scratch_bytes) ? G : 0;
 }
 
+namespace {
+
+using RingKernel = void (*)(RingArgs);
+RingKernel ring_kernel(int G, uint32_t max_length) {
+    const int form = entry_form(max_length);
+    return form == kWhole ? ring_kernel_for<kWhole>(G) : form == kBits16 ? ring_kernel_for<kBits16>(G) : ring_kernel_for<kBits32>(G);
+}
+
+// units of a grid that fills the device (0: none fits)
+cudaError_t ring_grid(const WfaPlan& p, int G, uint32_t max_length, int num_sms, size_t* n) {
+    const RingKernel kernel = ring_kernel(G, max_length);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    if (e != cudaSuccess) return e;
+    int bps = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, G > 32 ? G : 32 * kWarpsPerBlock,
+                                                      units_of(G) * ring_smem_per_warp(p, G, max_length));
+    *n = (size_t)num_sms * (size_t)std::max(bps, 0) * units_of(G);
+    return e;
+}
+
+}  // namespace
+
+size_t ring_full_scratch(const WfaPlan& p, int G, uint32_t max_length, int num_sms) {
+    size_t n = 0;
+    if (ring_grid(p, G, max_length, num_sms, &n) != cudaSuccess) return 0;
+    return n * ring_warp_bytes(p, G, max_length);
+}
+
 cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, const LimitView& L, const OutView& O,
                             const uint32_t* order, const uint32_t* bounds, uint8_t* scratch, size_t scratch_bytes,
                             uint32_t* counters, int num_sms, cudaStream_t st, int* warps_used) {
@@ -673,25 +711,18 @@ cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, cons
     auto sel = [](int d) { const uint32_t b = 2u * (uint32_t)(d - 1); return b | ((b + 1) << 4) | ((b + 9) << 8) | ((b + 9) << 12); };
     r.sel_x = sel(plan.x);
     r.sel_o = sel(plan.oe - plan.e);
-    void (*kernel)(RingArgs) = entry_form(len) == kWhole    ? ring_kernel_for<kWhole>(G)
-                                   : entry_form(len) == kBits16 ? ring_kernel_for<kBits16>(G)
-                                                                : ring_kernel_for<kBits32>(G);
     const size_t units = units_of(G), smem = units * r.smem_warp;
     const int threads = G > 32 ? G : 32 * kWarpsPerBlock;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-    if (e != cudaSuccess) return e;
-    int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, threads, smem);
-    if (e != cudaSuccess) return e;
-    if (bps < 1) return cudaSuccess;
-    size_t n = (size_t)num_sms * bps * units;
+    size_t n = 0;
+    cudaError_t e = ring_grid(plan, G, len, num_sms, &n);
+    if (e != cudaSuccess || n == 0) return e;
     n = std::min(n, scratch_bytes / min_warp);
     if (!bounds) n = std::min(n, ((size_t)P.num_pairs + pairs_of(G) - 1) / pairs_of(G));
     if (n == 0) return cudaSuccess;
     a.nwarps = (uint32_t)n;
     // a unit's arena: its share of the scratch, up to as many worst-case rounds as it defers
     a.warp_bytes = std::min(scratch_bytes / n & ~(size_t)255, min_warp + (32 / pairs_of(G) - 1) * r.round_bytes);
-    kernel<<<(unsigned)((n + units - 1) / units), threads, smem, st>>>(r);
+    ring_kernel(G, len)<<<(unsigned)((n + units - 1) / units), threads, smem, st>>>(r);
     e = cudaGetLastError();
     if (e == cudaSuccess) *warps_used = (int)n;
     return e;
