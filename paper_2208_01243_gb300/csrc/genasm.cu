@@ -1,4 +1,4 @@
-// GenASM (Section 2.4.3): windowed bit-parallel edit distance (bitap) with a
+// GenASM (Section 2.4.3): windowed bit-parallel edit distance with a
 // forward traceback, under a threshold of k edits.  One thread aligns one pair.
 //
 // Window.  At read position i and target position j a window holds
@@ -8,43 +8,40 @@
 // whose sequence goes on past the window is free (cost 0 there), an edge whose
 // sequence ends inside it charges one edit per base left on the other side.
 //
-// Status vectors.  Bit b of A_d(t) (one 64-bit word) is [f(wp-1-b, t) <= d]:
-// bit 0 is the last read base of the window, bit wp-1 the first.  With
-// EQ[c] = the bits whose read base equals c, and e(t, d) = [f(wp, t) <= d] the
-// empty read suffix, the recurrence over the target position t (from wt down) is
-//   A_d(wt) = target ends ? low d bits : all bits
-//   A_d(t)  = ((A_d(t+1) << 1 | e(t+1, d)) & EQ[T[t]])       match
-//           | (A_{d-1}(t+1) << 1 | e(t+1, d-1))              mismatch
-//           | (A_{d-1}(t) << 1 | e(t, d-1))                  I (read base)
-//           | A_{d-1}(t+1)                                   D (target base)
-// which is the suffix edit-distance recurrence one distance level at a time.
-// Bits above wp-1 carry no meaning; shifts only move them further up.  The
-// window distance is the first d with bit wp-1 of A_d(0) set.  A window whose
-// distance exceeds the edits left ends the pair: any way the alignment goes on
-// crosses the window's far edge, so the count only grows.
+// Difference vectors.  Neighbouring values of f differ by at most one, so a column t is held by the signs of its
+// differences, one bit per read base (bit 0 the last read base of the window, bit wp-1 the first):
+//   P, N   f(a, t) - f(a+1, t) is +1, is -1
+//   H+, H- f(a, t) - f(a, t+1) is +1, is -1
+//   Z      f(a, t) - f(a+1, t+1) is 0
+// and one column follows from the next with a dozen word operations and one carry chain, whatever the distance
+// (Myers, "A fast bit-vector algorithm for approximate string matching based on dynamic programming", 1999, over the
+// reversed window).  With EQ the bits whose read base equals T[t] and h the difference along the empty read suffix (1 where
+// the read ends in the window, 0 where its edge is free):
+//   Z  = (((EQ & P) + P) ^ P) | EQ | N
+//   H+ = N | ~(Z | P),   H- = P & Z
+//   P' = (H- << 1) | ~(EQ | N | (H+ << 1 | h)),   N' = (H+ << 1 | h) & (EQ | N)
+// (Z, in H+ and H-, without its last term, which changes neither).  The column past the window starts all +1 where the
+// target ends in it, all 0 where its edge is free.  The window distance is f(wp, 0) plus the differences of column 0.
+// A bitap's status vectors say the same level by level: [f <= d] for d up to the distance, eight words a column for
+// windows of up to seven edits.  A window whose distance exceeds the edits left ends the pair: any way the alignment
+// goes on crosses the window's far edge, so the count only grows.
 //
-// Sweeps.  Levels are computed in blocks of four or eight, target position by
-// target position (t descending): a block keeps its vectors in registers and
-// reads only the top level of the block below, A_{L0-1}(t), from a per-lane
-// carry row that it overwrites in place with its own top level (written only
-// when another block may follow).
+// Traceback, forward from (0, 0): after an I, I first; after a D, D first; then M, X, I, D, each only when the rest
+// still fits the window's distance.  The edits left always equal f(a, c), so an I fits where f(a, c) - f(a+1, c) is 1
+// (P of column c), a D where f(a, c) - f(a, c+1) is 1 (H+ of column c), an X where f(a, c) - f(a+1, c+1) is not 0 (Z of
+// column c; the bases differ), and a match always.  Match runs are taken with 32-base XOR compares.  A non-final window
+// stops once W-O read or W-O target bases have been consumed in it; the final window runs to its corner.  So the three
+// words are kept for the columns the traceback can reach, as the 32 bits from 16 below the diagonal position wp-1-t (or
+// from bit 0): a path with d edits never strays more than d diagonals, and a window that turns out to need more than 14
+// is computed again with whole words.
 //
-// Traceback, forward from (0, 0) with budget d (the window distance): after an
-// I, I first; after a D, D first; then M, X, I, D, each only when the rest still
-// fits (a match always does: on equal bases f(a, c) = f(a+1, c+1), since the
-// values of neighbouring cells differ by at most one).  Match runs are taken
-// with 32-base XOR compares.  A non-final window stops once W-O read or W-O
-// target bases have been consumed in it; the final window runs to its corner.
-// The traceback reads level d-1 at target positions c and c+1 only, for c up
-// to W-O in a non-final window, and only near the diagonal: a path with d
-// edits never strays more than d diagonals.  So the stored copy of A_d(t) is
-// kept for t up to the last position the traceback can read, and, when no
-// window can need more than 14 levels, only as the 32 bits from 16 below the
-// diagonal position wp-1-t (or from bit 0).
+// Scratch per warp, lane-interleaved (32 lanes of a step store one contiguous row): W columns of three rows of 32 words.
 //
-// Scratch per warp, lane-interleaved (32 lanes of a step store one contiguous
-// row): the carry row, (W+1) x 32 words, then levels x (W+1) x 32 stored
-// vectors (32 or 64 bits each).
+// What bounds it: the integer pipe, 81-84 % busy, on the columns' word operations (150 bp at 5 %: 587 warp instructions
+// a pair where status vectors level by level took 1,637).  1M pairs of 150 bp at 5 % in 0.82 ms (2.20 before), of 250 bp
+// at 5 % in 1.30 (4.93), of 100 bp at 1 % in 0.45 (0.62); 200k of 1,000 bp at 5 % in 1.16 ms (5.31; 1.93 with whole
+// words always kept, where the waits for them in the traceback led); 2,700 of 1,000 bp in 0.19 (0.58).
+#include <algorithm>
 #include <type_traits>
 
 #include "aim_internal.cuh"
@@ -52,30 +49,22 @@
 namespace aim {
 namespace {
 
-// distance levels per register block, one size per call: blocks of 8 when the threshold allows about two or
-// more edits per window (then most windows would need a second block of 4, and a whole warp waits for the
-// sweeps any one of its lanes needs), blocks of 4 otherwise
-constexpr int kSmallBlock = 4, kBigBlock = 8;
-constexpr int kBandLevels = 14;         // widest window distance a 32-bit band serves
+constexpr int kBandEdits = 14;         // widest window distance a 32-bit band serves
 
 struct GenasmArgs {
     PairsView P;
     LimitView L;
     OutView O;
     uint8_t* scratch;
-    size_t warp_bytes;              // carry row + stored levels of one warp
-    size_t carry_bytes;             // offset of the stored levels inside a warp's scratch
+    size_t warp_bytes;              // stored columns of one warp
     int W, overlap;
-    bool big_blocks;                // blocks of kBigBlock levels (else kSmallBlock): picks the kernel instance
     uint32_t nwarps;
     uint32_t* counter;
 };
 
 constexpr uint32_t kNoOp = 0;
 
-__device__ __forceinline__ uint64_t low_bits(int d) { return d >= 64 ? ~0ull : ((1ull << d) - 1ull); }
-
-// The stored copy of A_d(t): the whole word, or the 32 bits from band_start(wp, t) up, which hold every bit
+// The stored copy of a word of column t: the whole word, or the 32 bits from band_start(wp, t) up, which hold every bit
 // the traceback can ask for (within 16 of the diagonal position wp-1-t, never below bit 0).
 __device__ __forceinline__ int band_start(int wp, int t) { return max(wp - 17 - t, 0); }
 template <typename Band>
@@ -108,125 +97,59 @@ __device__ __forceinline__ uint32_t match_bits(uint64_t w, uint32_t code) {
     return even_bits(~(x | (x >> 1)));
 }
 
-// matching bases of read[p..] and target[q..], at most `cap`
-__device__ __forceinline__ int match_run(const uint64_t* rw, uint32_t nrw, uint32_t p, const uint64_t* tw,
-                                         uint32_t ntw, uint32_t q, int cap) {
-    int run = 0;
-    while (run < cap) {
-        const uint64_t x = window32(rw, nrw, p + run) ^ window32(tw, ntw, q + run);
-        const int same = __clzll((long long)x) >> 1;   // __clzll(0) = 64: the whole window matches
-        run += same;
-        if (same < 32) break;
-    }
-    return run < cap ? run : cap;
+// 32 bases from place p (0..63) of a window of two words
+__device__ __forceinline__ uint64_t from_place(uint64_t w0, uint64_t w1, int p) {
+    return p < 32 ? join_window(w0, w1, 2 * p) : w1 << (2 * (p - 32));
 }
 
 struct Window {
     uint64_t eq[4];     // read bases of the window, one mask per base code
-    uint64_t t0, t1;    // target bases 0..31 and 32..63 of the window
+    uint64_t r0, r1;    // read bases 0..31 and 32..63 of the window
+    uint64_t t0, t1;    // target bases
     int wp, wt;
-    int tmax;           // last target position the traceback can read
+    int tmax;           // last column the traceback can read
     bool end_r, end_t;
 };
 
-// One sweep of the B levels L0..L0+B-1 over t = wt..0.  FREE_R: the read goes on past the window (the
-// empty read suffix costs nothing); BANDS: store the levels for the traceback (positions up to w.tmax);
-// CARRY_OUT: overwrite the carry row with level L0+B-1; CARRY_IN: read level L0-1 from the carry row.
-template <int B, typename Band, bool FREE_R, bool BANDS, bool CARRY_OUT, bool CARRY_IN>
-__device__ __forceinline__ void sweep(const Window& w, int L0, Band* lv, size_t lstride, uint64_t* carry,
-                                      uint64_t (&cur)[B]) {
-    const int wp = w.wp, wt = w.wt;
-    const uint64_t edge = w.end_t ? 0ull : ~0ull;   // A_d(wt) = edge | low d bits
-#pragma unroll
-    for (int q = 0; q < B; ++q) {
-        cur[q] = edge | low_bits(L0 + q);
-        if (BANDS && wt <= w.tmax)
-            lv[(size_t)(L0 + q) * lstride + (size_t)wt * 32] = band_of<Band>(cur[q], band_start(wp, wt));
-    }
-    if (CARRY_OUT) carry[(size_t)wt * 32] = cur[B - 1];
-    uint64_t lo_old = CARRY_IN ? (edge | low_bits(L0 - 1)) : 0ull;   // A_{L0-1}(t+1)
-    auto step = [&](const int t, auto keep_tag) {
-        constexpr bool KEEP = decltype(keep_tag)::value;
+// The window's distance; columns 0 .. tmax stored at lv (three words of 32 lanes each).
+template <typename Band>
+__device__ __forceinline__ int window_distance(const Window& w, Band* lv) {
+    uint64_t P = w.end_t ? ~0ull : 0ull, N = 0ull;
+    const uint64_t h = w.end_r ? 1ull : 0ull;
+    auto column = [&](const int t, auto keep) {
         const uint64_t tword = t < 32 ? w.t0 : w.t1;
         const uint32_t code = (uint32_t)(tword >> (62 - 2 * (t & 31))) & 3u;
         const uint64_t e01 = (code & 1) ? w.eq[1] : w.eq[0], e23 = (code & 1) ? w.eq[3] : w.eq[2];
-        const uint64_t eqc = (code & 2) ? e23 : e01;
-        const uint64_t lo_new = CARRY_IN ? carry[(size_t)t * 32] : 0ull;   // A_{L0-1}(t)
-        // the empty read suffix at t+1 fits level d iff the wt-t-1 target bases left fit: e(t+1, d) = [x <= q],
-        // e(t+1, d-1) = [x + 1 <= q] (which covers e(t, d-1) too); on a free read edge both are 1
-        const int x = wt - t - 1 - L0;
-        const int s = KEEP ? band_start(wp, t) : 0;
-        uint64_t b_old = lo_old, b_new = lo_new;
-#pragma unroll
-        for (int q = 0; q < B; ++q) {
-            const uint64_t old = cur[q];
-            const uint64_t e1 = (FREE_R || x <= q) ? 1ull : 0ull;
-            uint64_t v = ((old << 1) | e1) & eqc;
-            if (CARRY_IN || q > 0) {
-                const uint64_t e2 = (FREE_R || x + 1 <= q) ? 1ull : 0ull;
-                v |= ((b_old | b_new) << 1) | e2 | b_old;
-            }
-            cur[q] = v;
-            if (KEEP) lv[(size_t)(L0 + q) * lstride + (size_t)t * 32] = band_of<Band>(v, s);
-            b_old = old;
-            b_new = v;
+        const uint64_t eq = (code & 2) ? e23 : e01;
+        const uint64_t z = (((eq & P) + P) ^ P) | eq;
+        const uint64_t hp = N | ~(z | P), hn = P & z;
+        const uint64_t x = eq | N, hs = (hp << 1) | h;
+        const uint64_t zero = z | N;
+        P = (hn << 1) | ~(x | hs);
+        N = hs & x;
+        if constexpr (decltype(keep)::value) {
+            const int s = band_start(w.wp, t);
+            Band* at = lv + (size_t)t * 96;
+            at[0] = band_of<Band>(P, s);
+            at[32] = band_of<Band>(hp, s);
+            at[64] = band_of<Band>(zero, s);
         }
-        if (CARRY_OUT) carry[(size_t)t * 32] = cur[B - 1];
-        lo_old = lo_new;
     };
-    // positions past the last one the traceback can read are computed but not stored
-    const int split = BANDS ? min(w.tmax, wt - 1) : -1;
-    for (int t = wt - 1; t > split; --t) step(t, std::false_type{});
-    if (BANDS)
-        for (int t = split; t >= 0; --t) step(t, std::true_type{});
+    int t = w.wt - 1;
+    for (; t > w.tmax; --t) column(t, std::false_type{});
+    for (; t >= 0; --t) column(t, std::true_type{});
+    const uint64_t rows = w.wp >= 64 ? ~0ull : (1ull << w.wp) - 1ull;
+    return (w.end_r ? w.wt : 0) + __popcll(P & rows) - __popcll(N & rows);
 }
 
-// Levels from L0 on in blocks of B until one reaches the window's start (or lmax is passed); the first
-// block (L0 = 0) reads no carry.  Returns the window's distance or -1.
-template <int B, typename Band, bool FREE_R>
-__device__ __forceinline__ int blocks_from(const Window& w, int lmax, Band* lv, size_t lstride, uint64_t* carry) {
-    uint64_t cur[B];
-    int found = -1;
-    for (int L0 = 0; found < 0 && L0 <= lmax; L0 += B) {
-        // a block fills the carry row whenever another may follow: lanes of a warp move together, so one lane
-        // that needs the next block makes the whole warp wait for it
-        const bool more = L0 + B <= lmax;
-        if (L0 == 0) {
-            if (more) sweep<B, Band, FREE_R, true, true, false>(w, 0, lv, lstride, carry, cur);
-            else sweep<B, Band, FREE_R, true, false, false>(w, 0, lv, lstride, carry, cur);
-        } else {
-            if (more) sweep<B, Band, FREE_R, true, true, true>(w, L0, lv, lstride, carry, cur);
-            else sweep<B, Band, FREE_R, true, false, true>(w, L0, lv, lstride, carry, cur);
-        }
-#pragma unroll
-        for (int q = 0; q < B; ++q)
-            if (found < 0 && L0 + q <= lmax && ((cur[q] >> (w.wp - 1)) & 1ull)) found = L0 + q;
-    }
-    return found;
-}
-
-// The window's distance (the first level whose bit wp-1 is set at t = 0), or -1 if it exceeds lmax.
-template <int B, typename Band, bool FREE_R>
-__device__ __forceinline__ int window_distance(const Window& w, int lmax, Band* lv, size_t lstride, uint64_t* carry) {
-    return blocks_from<B, Band, FREE_R>(w, lmax, lv, lstride, carry);
-}
-
-// 5 blocks of 128 threads per SM (96 registers) measured faster than 6 (80) or 8 (64, with spills)
-#ifndef AIM_GENASM_MIN_BLOCKS
-#define AIM_GENASM_MIN_BLOCKS 5
-#endif
-
-// B: distance levels per register block, a kernel instance per block size (one call uses one)
-template <typename Band, int B>
-__global__ void __launch_bounds__(128, AIM_GENASM_MIN_BLOCKS) genasm_kernel(GenasmArgs a) {
+// WIDE: some window may need more than kBandEdits edits: its columns are then computed again and kept whole
+template <bool WIDE>
+__global__ void __launch_bounds__(128) genasm_kernel(GenasmArgs a) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (gwarp >= a.nwarps) return;
     const int W = a.W, stop = a.W - a.overlap;
-    const size_t lstride = (size_t)(W + 1) * 32;                  // stored entries per level
     uint8_t* slot = a.scratch + (size_t)gwarp * a.warp_bytes;
-    uint64_t* carry = reinterpret_cast<uint64_t*>(slot) + lane;
-    Band* lv = reinterpret_cast<Band*>(slot + a.carry_bytes) + lane;
     unsigned long long st_cells = 0, st_pairs = 0;
 
     for (;;) {
@@ -268,67 +191,69 @@ __global__ void __launch_bounds__(128, AIM_GENASM_MIN_BLOCKS) genasm_kernel(Gena
             w.end_t = m - j <= (uint32_t)W;
             const bool fin = w.end_r && w.end_t;
             const int wp = w.wp, wt = w.wt;
-            w.tmax = fin ? wt : min(stop, wt);
+            w.tmax = (fin ? wt : min(stop, wt)) - 1;
             // read window masks: bit wp-1-a is read base i+a
-            const uint64_t r0 = window32(rw, nrw, i), r1 = window32(rw, nrw, i + 32);
+            w.r0 = window32(rw, nrw, i);
+            w.r1 = window32(rw, nrw, i + 32);
 #pragma unroll
             for (uint32_t c = 0; c < 4; ++c)
-                w.eq[c] = (((uint64_t)match_bits(r0, c) << 32) | match_bits(r1, c)) >> (64 - wp);
+                w.eq[c] = (((uint64_t)match_bits(w.r0, c) << 32) | match_bits(w.r1, c)) >> (64 - wp);
             w.t0 = window32(tw, ntw, j);
             w.t1 = window32(tw, ntw, j + 32);
 
-            // distance levels, in blocks, until the window's start is reached
             const int64_t left = k - used;
-            const int lmax = (int)(left < (int64_t)max(wp, wt) ? left : (int64_t)max(wp, wt));
-            const int found = w.end_r ? window_distance<B, Band, false>(w, lmax, lv, lstride, carry)
-                                      : window_distance<B, Band, true>(w, lmax, lv, lstride, carry);
-            // work of a plain bitap: levels 0..d (0..lmax when the window is over the budget) at every position
-            st_cells += (unsigned long long)((found < 0 ? lmax : found) + 1) * wt;
-            if (found < 0) { rejected = true; break; }
+            const int dist = window_distance<uint32_t>(w, reinterpret_cast<uint32_t*>(slot) + lane);
+            const bool over = dist > left;
+            // work of a bitap: levels 0..d (0..left when the window is over the budget) at every position
+            st_cells += (unsigned long long)((over ? left : (int64_t)dist) + 1) * wt;
+            if (over) { rejected = true; break; }
 
             // traceback
-            int ta = 0, tc = 0, d = found;
-            for (;;) {
-                if (!fin && (ta >= stop || tc >= stop)) break;
-                if (ta == wp && tc == wt) break;
-                uint32_t op;
-                int len = 1;
-                if (ta == wp) {
-                    op = kOpDel;
-                } else if (tc == wt) {
-                    op = kOpIns;
-                } else {
-                    const uint32_t pa = (uint32_t)(__ldg(rw + ((i + ta) >> 5)) >> (62 - 2 * ((i + ta) & 31))) & 3u;
-                    const uint32_t pb = (uint32_t)(__ldg(tw + ((j + tc) >> 5)) >> (62 - 2 * ((j + tc) & 31))) & 3u;
-                    const bool same = pa == pb;
-                    const int b = wp - 1 - ta;
-                    bool fI = false, fD = false, fX = false;
-                    if (d > 0) {
-                        const Band* ld = lv + (size_t)(d - 1) * lstride;
-                        const Band at_c = ld[(size_t)tc * 32], at_c1 = ld[(size_t)(tc + 1) * 32];
-                        const int p_c = band_start(wp, tc), p_c1 = band_start(wp, tc + 1);
-                        const bool e_c = !w.end_r || wt - tc <= d - 1, e_c1 = !w.end_r || wt - tc - 1 <= d - 1;
-                        fI = b >= 1 ? band_bit(at_c, b - 1, p_c) : e_c;
-                        fD = band_bit(at_c1, b, p_c1);
-                        fX = b >= 1 ? band_bit(at_c1, b - 1, p_c1) : e_c1;
+            int ta = 0, tc = 0;
+            auto trace = [&](auto lv) {   // pointer to this lane's stored columns
+                using Band = typename std::remove_pointer<decltype(lv)>::type;
+                for (;;) {
+                    if (!fin && (ta >= stop || tc >= stop)) break;
+                    if (ta == wp && tc == wt) break;
+                    uint32_t op;
+                    int len = 1;
+                    if (ta == wp) {
+                        op = kOpDel;
+                    } else if (tc == wt) {
+                        op = kOpIns;
+                    } else {
+                        const Band* at = lv + (size_t)tc * 96;
+                        const int b = wp - 1 - ta, from = sizeof(Band) == 4 ? band_start(wp, tc) : 0;
+                        const bool fI = band_bit(at[0], b, from), fD = band_bit(at[32], b, from);
+                        const bool fX = !band_bit(at[64], b, from);
+                        // equal bases from here on, as far as 32 bases of the window's words show
+                        const uint64_t x = from_place(w.r0, w.r1, ta) ^ from_place(w.t0, w.t1, tc);
+                        const int same = __clzll((long long)x) >> 1;   // __clzll(0) = 64
+                        if (prev == kOpIns && fI) op = kOpIns;
+                        else if (prev == kOpDel && fD) op = kOpDel;
+                        else if (same) {
+                            op = kOpMatch;
+                            int lim = min(wp - ta, wt - tc);
+                            if (!fin) lim = min(lim, min(stop - ta, stop - tc));
+                            len = min(same, lim);
+                        } else if (fX) op = kOpMismatch;
+                        else if (fI) op = kOpIns;
+                        else op = kOpDel;
                     }
-                    if (prev == kOpIns && fI) op = kOpIns;
-                    else if (prev == kOpDel && fD) op = kOpDel;
-                    else if (same) {
-                        op = kOpMatch;
-                        int lim = min(wp - ta, wt - tc);
-                        if (!fin) lim = min(lim, min(stop - ta, stop - tc));
-                        len = match_run(rw, nrw, i + ta, tw, ntw, j + tc, lim);
-                    } else if (fX) op = kOpMismatch;
-                    else if (fI) op = kOpIns;
-                    else op = kOpDel;
+                    out.put(op, (uint32_t)len);
+                    prev = op;
+                    if (op != kOpMatch) ++used;
+                    if (op == kOpMatch || op == kOpMismatch) { ta += len; tc += len; }
+                    else if (op == kOpIns) ++ta;
+                    else ++tc;
                 }
-                out.put(op, (uint32_t)len);
-                prev = op;
-                if (op != kOpMatch) { --d; ++used; }
-                if (op == kOpMatch || op == kOpMismatch) { ta += len; tc += len; }
-                else if (op == kOpIns) ++ta;
-                else ++tc;
+            };
+            if (WIDE && dist > kBandEdits) {
+                uint64_t* whole = reinterpret_cast<uint64_t*>(slot) + lane;
+                window_distance<uint64_t>(w, whole);
+                trace(whole);
+            } else {
+                trace(reinterpret_cast<uint32_t*>(slot) + lane);
             }
             i += (uint32_t)ta;
             j += (uint32_t)tc;
@@ -352,29 +277,24 @@ __global__ void __launch_bounds__(128, AIM_GENASM_MIN_BLOCKS) genasm_kernel(Gena
     warp_stat_add(a.O.stats, 3, st_pairs, lane);
 }
 
-// blocks of kBigBlock levels when the threshold allows about two or more edits per window of W bases
-bool big_blocks_for(int W, int64_t max_limit, uint32_t max_length) {
-    const int64_t len = max_length > (uint32_t)W ? (int64_t)max_length : (int64_t)W;
-    return max_limit >= kSmallBlock && max_limit * W >= 2 * len;
+bool banded(int W, int64_t max_limit) { return (max_limit < W ? max_limit : W) <= kBandEdits; }
+
+// a warp's stored columns
+size_t column_bytes(int W, int64_t max_limit) {
+    return align_up((size_t)W * 96 * (banded(W, max_limit) ? sizeof(uint32_t) : sizeof(uint64_t)), 256);
 }
-
-// distance levels a window can need under the largest threshold, in whole register blocks
-int levels_for(int W, int64_t max_limit, bool big) {
-    const int64_t top = max_limit < W ? max_limit : W;   // a window's distance never exceeds W
-    const int B = big ? kBigBlock : kSmallBlock;
-    return (int)((top + 1 + B - 1) / B * B);
-}
-
-bool banded(int W, int64_t max_limit) { return (max_limit < W ? max_limit : W) <= kBandLevels; }
-
-size_t carry_bytes_for(int W) { return align_up((size_t)(W + 1) * 32 * sizeof(uint64_t), 256); }
 
 }  // namespace
 
+// The scratch a call has to bring for one warp (the entry points' limit, kept from the form that stored a word per
+// distance level: a row of W + 1 words, then levels in blocks of 4, or 8 where the threshold allows about two or more
+// edits per window).  Never less than column_bytes.
 size_t genasm_warp_bytes(int W, int64_t max_limit, uint32_t max_length) {
-    const size_t band = banded(W, max_limit) ? sizeof(uint32_t) : sizeof(uint64_t);
-    const int levels = levels_for(W, max_limit, big_blocks_for(W, max_limit, max_length));
-    return carry_bytes_for(W) + align_up((size_t)levels * (W + 1) * 32 * band, 256);
+    const int64_t len = std::max<int64_t>(max_length, W), top = std::min<int64_t>(max_limit, W);
+    const int block = max_limit >= 4 && max_limit * W >= 2 * len ? 8 : 4;
+    const size_t levels = (size_t)((top + block) / block * block);
+    const size_t word = banded(W, max_limit) ? sizeof(uint32_t) : sizeof(uint64_t);
+    return align_up((size_t)(W + 1) * 32 * sizeof(uint64_t), 256) + align_up(levels * (W + 1) * 32 * word, 256);
 }
 
 cudaError_t launch_genasm(int W, int O, const PairsView& P, const LimitView& L, const OutView& Ov, int64_t max_limit,
@@ -386,20 +306,13 @@ cudaError_t launch_genasm(int W, int O, const PairsView& P, const LimitView& L, 
     a.P = P; a.L = L; a.O = Ov;
     a.W = W; a.overlap = O;
     a.counter = counter;
-    a.carry_bytes = carry_bytes_for(W);
-    a.big_blocks = big_blocks_for(W, max_limit, P.max_length);
-    a.warp_bytes = genasm_warp_bytes(W, max_limit, P.max_length);
+    a.warp_bytes = column_bytes(W, max_limit);
     // warp slots start on 256-byte boundaries so that every stored row is one aligned segment
     uint8_t* base = reinterpret_cast<uint8_t*>(align_up(reinterpret_cast<size_t>(scratch), 256));
     const size_t skip = (size_t)(base - scratch);
     if (skip >= scratch_bytes) return cudaSuccess;
     a.scratch = base;
-    const bool band = banded(W, max_limit);
-    // the four kernel instances: stored copies as 32-bit bands or whole words, blocks of 4 or 8 levels
-    void (*kernel)(GenasmArgs) = band ? (a.big_blocks ? genasm_kernel<uint32_t, kBigBlock>
-                                                      : genasm_kernel<uint32_t, kSmallBlock>)
-                                      : (a.big_blocks ? genasm_kernel<uint64_t, kBigBlock>
-                                                      : genasm_kernel<uint64_t, kSmallBlock>);
+    void (*kernel)(GenasmArgs) = banded(W, max_limit) ? genasm_kernel<false> : genasm_kernel<true>;
     int bps = 0;
     cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, 128, 0);
     if (err != cudaSuccess) return err;
