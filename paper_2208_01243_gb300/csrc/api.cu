@@ -190,20 +190,22 @@ int align_packed(aim_ctx* ctx, const aim::PairsView& P, int algo, const aim_pena
                                           &w2);
                 if (err == cudaSuccess && w2 == 0) warps = 0;
             }
-        } else if (const int ring = !aim::ring_ok(plan, P.max_length) ? 0
-                                    : !ctx->wfa_group ? aim::ring_group(plan, P.max_length, P.num_pairs, ctx->num_sms,
-                                                                        scratch_bytes)
-                                    : aim::ring_fits(plan, ctx->wfa_group, P.max_length, scratch_bytes) ? ctx->wfa_group
-                                                                                                         : 0) {
-            slot = time_begin(ctx, 1, st);
-            err = aim::launch_wfa_ring(plan, ring, P, r.lim, O, nullptr, nullptr, scratch, scratch_bytes, counter,
-                                       ctx->num_sms, st, &warps);
         } else {
+            // (whatever kernel runs, the workspace has to hold the general one's scratch)
             const int group = fit_group(plan, ctx->wfa_group ? ctx->wfa_group
                                                              : aim::wfa_default_group(plan, P.max_length));
             if (!group) return AIM_ERR_NOMEM;
+            int ring = 0;
+            if (aim::ring_ok(plan, P.max_length)) {
+                ring = ctx->wfa_group ? ctx->wfa_group
+                                      : aim::ring_group(plan, P.max_length, P.num_pairs, ctx->num_sms, scratch_bytes);
+                if (ctx->wfa_group && !aim::ring_fits(plan, ring, P.max_length, scratch_bytes)) ring = 0;
+            }
             slot = time_begin(ctx, 1, st);
-            err = aim::launch_wfa(plan, group, P, r.lim, O, scratch, scratch_bytes, counter, ctx->num_sms, st, &warps);
+            err = ring ? aim::launch_wfa_ring(plan, ring, P, r.lim, O, nullptr, nullptr, scratch, scratch_bytes,
+                                              counter, ctx->num_sms, st, &warps)
+                       : aim::launch_wfa(plan, group, P, r.lim, O, scratch, scratch_bytes, counter, ctx->num_sms, st,
+                                         &warps);
         }
     } else {
         const bool unit = algo == AIM_ALGO_EDIT_NW;
@@ -219,7 +221,7 @@ int align_packed(aim_ctx* ctx, const aim::PairsView& P, int algo, const aim_pena
         const aim::DpPlan plan = aim::plan_dp(unit, (int)b, P.max_length, r.max_limit);
         const bool lanes = aim::dp_lane_ok(unit, (int)b, r.costs, P.max_length, r.max_limit, P.num_pairs,
                                            ctx->num_sms, scratch_bytes);
-        if (!lanes && plan.slot_bytes > scratch_bytes) return AIM_ERR_NOMEM;
+        if (plan.slot_bytes > scratch_bytes) return AIM_ERR_NOMEM;
         slot = time_begin(ctx, 1, st);
         if (lanes)
             err = aim::launch_dp_lane(unit, (int)b, r.costs, P, r.lim, O, r.max_limit, scratch, scratch_bytes, counter,

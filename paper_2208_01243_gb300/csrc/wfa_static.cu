@@ -111,16 +111,18 @@ extern "C" int aim_wfa_align_static(const uint64_t* packed_reads, const uint64_t
 
     const aim::WfaPlan plan = aim::plan_wfa(costs, pen->band, max_length, max_limit);
     const size_t capacity = kStaticScratchBytes - kStaticHeaderBytes;
+    int group = aim::wfa_default_group(plan, max_length);
+    while (group <= 32 && 8 * aim::wfa_warp_bytes(group, aim::wfa_pair_bytes(plan, group)) > capacity)
+        group = group == 32 ? 256 : group * 2;
+    if (8 * aim::wfa_warp_bytes(group, aim::wfa_pair_bytes(plan, group)) > capacity)
+        return AIM_ERR_NOMEM;   // one pair is too big
+
     uint8_t* base = nullptr;
     int sms = 0;
     const int rc = scratch_for_current_device((cudaStream_t)stream, &base, &sms);
     if (rc) return rc;
     const int ring = aim::ring_ok(plan, max_length) ? aim::ring_group(plan, max_length, num_pairs, sms, capacity) : 0;
-    int group = ring ? ring : aim::wfa_default_group(plan, max_length);
-    while (!ring && group <= 32 && 8 * aim::wfa_warp_bytes(group, aim::wfa_pair_bytes(plan, group)) > capacity)
-        group = group == 32 ? 256 : group * 2;
-    if (!ring && 8 * aim::wfa_warp_bytes(group, aim::wfa_pair_bytes(plan, group)) > capacity)
-        return AIM_ERR_NOMEM;   // one pair is too big
+    if (ring) group = ring;
 
     cudaStream_t st = (cudaStream_t)stream;
     uint32_t* counter = reinterpret_cast<uint32_t*>(base);
