@@ -268,8 +268,8 @@ AIM_API int aim_set_wfa_adaptive(aim_ctx *ctx, int min_length, int max_distance)
  * >= 0, else max_edits or the per-pair array), and a band is not supported
  * (pen->band >= 0 gives AIM_ERR_UNSUPPORTED).  Any max_length is accepted.
  *
- * The pair is aligned in windows of `window` bases (1..64: one 64-bit word per
- * bitap status vector; default 64) that overlap by `overlap` bases (0..window-1,
+ * The pair is aligned in windows of `window` bases (1..64: one bit of a word per
+ * read base; default 64) that overlap by `overlap` bases (0..window-1,
  * default 24).  A window's distance is its edit distance to the window's far
  * edge, where an edge is free if its sequence goes on past the window (the
  * last window, holding both ends, is a global alignment).  A forward traceback
@@ -282,8 +282,9 @@ AIM_API int aim_set_wfa_adaptive(aim_ctx *ctx, int min_length, int max_distance)
  * iff it exceeds k.  Inside one window this is the exact edit distance; across
  * windows the score can exceed it.
  *
- * Work counter [4] (aim_stats_read) counts the 64-bit status vectors computed
- * (one distance level at one target position of one window).
+ * Work counter [4] (aim_stats_read) counts the bitap's status vectors: distance
+ * + 1 levels at each target position of a window (the kernel computes a fixed
+ * number of words per position that say the same).
  */
 AIM_API int aim_set_genasm_window(aim_ctx *ctx, int window, int overlap);
 
@@ -291,15 +292,22 @@ AIM_API int aim_set_genasm_window(aim_ctx *ctx, int window, int overlap);
  * Batched form (wavefront algorithm): pairs of uneven length and error rate
  * in persistent launches over length-bucketed queues.  The batch is planned
  * once and then replayed:
- *   - packing, length/threshold bucketing of the pairs (on the device: a
- *     histogram, a scan and a scatter into an order array, heaviest work class
- *     first, buckets sharing a lanes-per-pair value kept contiguous) and one
- *     persistent alignment launch per lanes-per-pair value, each draining its
- *     queue range in that order, are recorded as one CUDA graph;
- *   - with `autotune`, the lanes per pair of every non-empty bucket are chosen by
- *     timed trial launches on a device-filling sample of its pairs (each choice cached in
- *     the context per costs, band and bucket); otherwise from the bucket's
- *     width class or an earlier cached choice.
+ *   - packing, bucketing of the pairs (on the device: a histogram, a scan and a
+ *     scatter into an order array, heaviest bucket first) and the persistent
+ *     alignment launches that drain the queues are recorded as one CUDA graph;
+ *   - where a pair's running wavefronts fit shared memory (the common case: costs
+ *     whose scaled mismatch and gap steps are at most 4, gap extension the
+ *     scaled unit, and thresholds whose wavefronts are narrow enough), buckets
+ *     are classes of the largest scaled score a pair may reach, pairs are
+ *     bucketed again by min(limit, bound) after a bound pass (below), and each
+ *     class is one launch, on streams of the plan's own; thin classes are merged
+ *     at planning.  Lanes per pair and bound passes follow from the class, or
+ *     from an earlier cached choice; `autotune` caches them and runs no trials;
+ *   - otherwise buckets are work and width classes, and with `autotune` the lanes
+ *     per pair of every non-empty one are chosen by timed trial launches on a
+ *     device-filling sample of its pairs (each choice cached in the context per
+ *     costs, band and bucket), else from the bucket's width class or an earlier
+ *     cached choice; buckets sharing a lanes-per-pair value share a launch.
  * Arguments are those of aim_align_batch_ascii (the same buffers are bound to
  * the plan: every aim_batch_run aligns their current contents, which may
  * change between runs as long as the shapes and bounds still hold).
@@ -335,8 +343,9 @@ AIM_API int aim_batch_info(aim_batch *batch, int *groups /* host[32] */, uint32_
  * algorithm).  aim_batch_passes reports, per bucket, the first-pass lanes (0:
  * one pass only) and the full-pass lanes; it returns the number of buckets with
  * a compact first pass.  aim_set_batch_compact sets how later plans of the
- * context choose: 0 (default) by timed trials when autotuning, 1 always where
- * the scratch allows, 2 never.
+ * context choose: 0 (default) by timed trials when autotuning (plans whose
+ * wavefronts run in shared memory need no compact pass and use none), 1 always
+ * where the scratch allows, 2 never.
  */
 AIM_API int aim_batch_passes(aim_batch *batch, int *first_pass /* host[32] */, int *full_pass /* host[32] */);
 AIM_API int aim_set_batch_compact(aim_ctx *ctx, int mode);
@@ -352,10 +361,12 @@ AIM_API int aim_set_batch_compact(aim_ctx *ctx, int mode);
  * runs with min(limit, bound) as the pair's limit, and its clamp keeps only
  * a diamond around the optimal paths.  Scores, flags and CIGARs are those of
  * the exact pass alone.  aim_batch_bound_passes reports, per bucket, the
- * bound pass's lanes per pair (0: none) and returns the number of buckets
- * with one.  aim_set_batch_bound sets how later plans of the context choose:
- * 0 (default) by timed trials when autotuning, 1 always (reads up to 32,000
- * bp), 2 never.  Plans with a compact first pass run no bound pass.  Work
+ * bound pass's lanes per pair (0: none; 1: the form with its few
+ * diagonals in registers, a lane or a warp per pair) and returns the number of buckets with one.  aim_set_batch_bound sets how later plans of the context choose:
+ * 0 (default) by timed trials when autotuning, or, with wavefronts in shared
+ * memory, for every class that may reach a scaled score of 48 (but a batch
+ * that makes one small class); 1 always (reads
+ * up to 32,000 bp), 2 never.  Plans with a compact first pass run no bound pass.  Work
  * counters [0] and [1] include the bound pass's entries and windows.
  */
 AIM_API int aim_batch_bound_passes(aim_batch *batch, int *bound_pass /* host[32] */);
@@ -390,8 +401,7 @@ AIM_API int aim_batch_destroy(aim_batch *batch);
  * one launch per job side by side, copy out), so its jobs and the requests
  * that arrive while others run overlap on the device.  Jobs of the heaviest
  * work classes (work class >= 5, wavefronts over 256 diagonals; reads up to
- * 32,000 bp) run a bound pass first, as the batched form's tuner chooses for
- * such buckets.  Results are those of
+ * 32,000 bp) run a bound pass first.  Results are those of
  * aim_align_batch_ascii for the same pairs, independent of what else runs.
  * aim_server_create allocates the arenas and starts the worker thread.
  */
@@ -453,7 +463,7 @@ AIM_API int aim_set_wfa_group(aim_ctx *ctx, int lanes);
  *   [1] 32-base windows compared by the WFA extend
  *   [2] DP cells computed (in-band cells actually swept, up to early exit)
  *   [3] pairs aligned (every pair a kernel finished, any flag)
- *   [4] GenASM status vectors computed (one distance level at one target position of one window)
+ *   [4] GenASM status vectors (distance + 1 levels at each target position of a window)
  * aim_stats_reset is asynchronous on `stream`; aim_stats_read synchronises
  * the device and copies the five counters to host memory `out`.
  */

@@ -237,9 +237,9 @@ cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, cons
 
 // scratch with which every unit of a full grid of launch_wfa_ring has its own
 size_t ring_full_scratch(const WfaPlan& p, int G, uint32_t max_length, int num_sms);
-// the bound pass with one pair per lane (wfa_bound.cu): whether costs and lengths allow it; over the queue range
-// bounds[0..1] of order, results in plan.bound
-bool bound_lanes_ok(const WfaPlan& p, uint32_t max_length);
+// the bound passes of wfa_bound.cu: whether costs and lengths allow them; over the queue range bounds[0..1] of order,
+// results in plan.bound
+bool bound_ok(const WfaPlan& p, uint32_t max_length);
 cudaError_t launch_wfa_bound(const WfaPlan& plan, const PairsView& P, const LimitView& L, const OutView& O,
                              const uint32_t* order, const uint32_t* bounds, uint32_t* counters, int num_sms,
                              cudaStream_t st);

@@ -49,9 +49,11 @@
 // instead, edges a quarter apart: a ring's size and a warp's work follow from S alone.  The bound pass, by rule rather
 // than by trial, runs over the classes above kBoundScore, the pairs are bucketed again by min(S, bound), and every class
 // has one exact launch of its own with the lanes per pair that rule suits its rings.  Planning runs the bound pass once
-// and merges classes that the batch fills too thinly.  1M pairs of 100-1,000 bp, 1-10 %: 19.7 ms, of which the bound
+// and merges classes that the batch fills too thinly; a class of few pairs takes more lanes for each, and a batch that
+// makes one small class goes without the bound pass.  1M pairs of 100-1,000 bp, 1-10 %: 19.1 ms, of which the bound
 // pass 2.3 (34.0 ms with the buckets above on wfa.cu's kernels, 22-26 ms with the same buckets on wfa_ring.cu's);
-// 4,000 pairs of 2-10 kbp 14.5 ms (31 ms; 18 ms; 23 ms before thin classes were merged).
+// 4,000 pairs of 2-10 kbp 12.7 ms (31 ms; 18 ms; 23 ms before thin classes were merged); 1,000 pairs of 138-408 bp
+// 137 us (335 us; 312 us with the bound pass), 16,000 431 us (475 us; 548 us with a full batch's lanes).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -262,6 +264,9 @@ struct aim_batch {
     int64_t gdiagonals[aim::kBuckets], gscores[aim::kBuckets];   // each group's widest window and largest limit
     // plans of wfa_ring.cu: one exact launch per class of limits, side by side on streams of their own
     bool ring;
+    bool few;                               // pairs for too few rounds of the launches for a bound pass to pay
+    bool tuning;                            // autotune: cached choices are not taken
+    uint32_t class_pairs[aim::kBuckets];    // pairs of each class seen at planning (before: as many as fill any launch)
     uint32_t* cclaims;
     size_t class_at[aim::kBuckets], class_bytes[aim::kBuckets];   // each class's part of the scratch
     cudaStream_t side[4];
@@ -309,7 +314,7 @@ cudaError_t enqueue_prepare(aim_batch* b, cudaStream_t st) {
 // pass first; the pairs are then bucketed again by min(limit, bound), and every class has one exact launch with the
 // lanes per pair that its windows suit, four classes at a time on streams of their own (the tail of one class, a few
 // long pairs, runs beside the next ones).
-constexpr int64_t kBoundScore = 40;
+constexpr int64_t kBoundScore = 48;   // (at 44, 500k pairs of 139 bp from host buffers took 2.17 ms with it, 2.06 without)
 
 WfaPlan class_plan(const aim_batch* b, int k) {   // bucket k
     WfaPlan p = b->plan;
@@ -355,7 +360,7 @@ cudaError_t enqueue_bounds(aim_batch* b, cudaStream_t st, bool* fits) {
             *fits = *fits && (e != cudaSuccess || w > 0);
         }
     }
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || b->bp.nclasses == 1) return e;   // one class takes them all
     const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)sms * 8);
     bucket_count_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rcounts, nullptr, b->bound);
     return cudaGetLastError();
@@ -372,12 +377,14 @@ cudaError_t enqueue_ring(aim_batch* b, cudaStream_t st, int* warps) {
         bool fits = true;
         e = enqueue_bounds(b, st, &fits);
         if (e != cudaSuccess || !fits) return e;
-        const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)sms * 8);
-        bucket_scan_kernel<<<1, 32, 0, st>>>(b->rcounts, b->rbounds, b->rfill, b->cclaims, b->bp, nullptr);
-        bucket_scatter_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rbounds, b->rfill, b->rorder, nullptr,
-                                                      b->bound);
-        e = cudaGetLastError();
-        order = b->rorder; bounds = b->rbounds; claims = b->cclaims;
+        if (nc > 1) {
+            const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)sms * 8);
+            bucket_scan_kernel<<<1, 32, 0, st>>>(b->rcounts, b->rbounds, b->rfill, b->cclaims, b->bp, nullptr);
+            bucket_scatter_kernel<<<blocks, 256, 0, st>>>(b->P, b->r.lim, b->bp, b->rbounds, b->rfill, b->rorder,
+                                                          nullptr, b->bound);
+            e = cudaGetLastError();
+            order = b->rorder; bounds = b->rbounds; claims = b->cclaims;
+        }
     }
     if (e == cudaSuccess) e = cudaEventRecord(b->fork, st);
     const int ns = std::min(nc, 4);
@@ -411,14 +418,14 @@ bool ring_layout(aim_batch* b) {
         const WfaPlan p = class_plan(b, k);
         // cached choices (an earlier plan's, or imported), else the rule of wfa_ring.cu for a batch that fills the
         // device, and a bound pass with one pair per lane, or a warp per pair for longer reads
-        const TuneChoice* cached = cached_choice(b, k);
+        const TuneChoice* cached = b->tuning ? nullptr : cached_choice(b, k);
         b->groups[k] = cached && ring_fits(p, std::get<0>(*cached), b->max_length, b->scratch_bytes)
                            ? std::get<0>(*cached)
-                           : ring_group(p, b->max_length, 0x7fffffffu, b->ctx->num_sms, b->scratch_bytes);
-        const bool lanes = bound_lanes_ok(b->plan, b->max_length);
+                           : ring_group(p, b->max_length, b->class_pairs[k], b->ctx->num_sms, b->scratch_bytes);
+        const bool regs = bound_ok(b->plan, b->max_length);
         const int mode = b->ctx->batch_bound;
-        int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore ? 0 : lanes ? 1 : 32;
-        if (mode == 0 && cached && (std::get<2>(*cached) != 1 || lanes)) gb = std::get<2>(*cached);
+        int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore || b->few ? 0 : regs ? 1 : 32;
+        if (mode == 0 && cached && (std::get<2>(*cached) != 1 || regs)) gb = std::get<2>(*cached);
         b->bound1[k] = mode == 2 || b->max_length > kMaxWfaLength16 ? 0 : gb;
         want[k] = b->groups[k] ? ring_full_scratch(p, b->groups[k], b->max_length, b->ctx->num_sms) : 0;
         if (!want[k]) return false;
@@ -466,21 +473,33 @@ bool plan_ring(aim_batch* b) {
 
 // Merges classes that the batch at hand fills with fewer pairs than its launch runs at once (a class's launch takes at
 // least as long as its longest pair): heaviest first, a class takes in the ones below it until it has that many.
-// `counts`: pairs per class under min(limit, bound).
-void ring_merge(aim_batch* b, const uint32_t* counts) {
+// Classes without pairs stay apart from a full one below them, which then keeps the lanes that suit it.
+// `counts`: pairs per class under min(limit, bound).  Returns whether the batch is one class's and too small for a bound
+// pass: below four rounds of its launch the exact pass gains less from narrower wavefronts than the pass takes.
+// (Limit 11 edits on 139 bp: 60k pairs 523 us without it, 575 with; 16k pairs of 138-408 bp 405 and 435, 1k 137 and 171;
+// two classes: 60k pairs of 138-408 bp 1,021 and 862, 1.6k of 1-10 kbp 8.6 ms and 7.4 ms.)
+bool ring_merge(aim_batch* b, const uint32_t* counts) {
     int32_t edge[kBuckets];
-    int nc = 0;
+    int nc = 0, filled = 0;
+    bool small = true;
     for (int k = 0; k < b->bp.nclasses;) {   // heaviest first
         const WfaPlan p = class_plan(b, k);
         const size_t units = ring_full_scratch(p, b->groups[k], b->max_length, b->ctx->num_sms) /
                              ring_warp_bytes(p, b->groups[k], b->max_length);
-        const size_t need = units * (b->groups[k] > 32 ? 1 : (size_t)(32 / b->groups[k]));
+        const size_t need = std::max<size_t>(units * (b->groups[k] > 32 ? 1 : 32 / b->groups[k]), 1);
         size_t have = 0;
-        edge[nc++] = b->bp.edge[b->bp.nclasses - 1 - k];
-        while (k < b->bp.nclasses && have < need) have += counts[k++];
+        edge[nc] = b->bp.edge[b->bp.nclasses - 1 - k];
+        for (const int first = k; k < b->bp.nclasses && have < need; ++k) {
+            if (have == 0 && k > first && counts[k] >= need) break;
+            have += counts[k];
+        }
+        filled += have > 0;
+        small = small && have < 4 * need;
+        b->class_pairs[nc++] = (uint32_t)have;
     }
     for (int c = 0; c < nc; ++c) b->bp.edge[c] = edge[nc - 1 - c];
     b->bp.nclasses = nc;
+    return filled <= 1 && small;
 }
 
 cudaError_t enqueue_align(aim_batch* b, cudaStream_t st, int* warps) {
@@ -755,7 +774,16 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
     e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) { free_batch(b); return cuda_status(e); }
 
+    b->tuning = autotune != 0;
+    for (int k = 0; k < kBuckets; ++k) b->class_pairs[k] = 0x7fffffffu;
     b->ring = plan_ring(b);
+    // the scratch has to hold the general kernels' worst case at one pair per warp or per block, whichever kernels run:
+    // how much a plan asks for does not hang on its costs or lengths
+    if (b->ring && 8 * std::min(wfa_warp_bytes(32, bucket_pair_bytes(b->plan, 0, 32)),
+                                wfa_warp_bytes(256, bucket_pair_bytes(b->plan, 0, 256))) > b->scratch_bytes) {
+        free_batch(b);
+        return AIM_ERR_NOMEM;
+    }
 
     // prepare once (synchronously) to see the bucket sizes, then tune
     e = enqueue_prepare(b, b->stream);
@@ -766,14 +794,23 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
         // classes to suit this batch: its counts after the bound passes, where there are any
         uint32_t counts[kBuckets];
         std::memcpy(counts, b->host_counts, sizeof(counts));
-        if (ring_bounded(b)) {
+        if (ring_bounded(b) && b->bp.nclasses > 1) {
             bool fits = true;
             e = enqueue_bounds(b, b->stream, &fits);
             if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
             if (e == cudaSuccess) e = cudaMemcpy(counts, b->rcounts, sizeof(counts), cudaMemcpyDeviceToHost);
         }
-        ring_merge(b, counts);
-        if (e == cudaSuccess && !ring_layout(b)) e = cudaErrorUnknown;   // (fewer classes need no more than before)
+        if (ring_merge(b, counts) && ctx->batch_bound == 0) {
+            b->few = true;
+            b->bp.nclasses = 1;
+            b->bp.edge[0] = b->plan.smax;
+            b->class_pairs[0] = num_pairs;
+        }
+        if (e == cudaSuccess && !ring_layout(b)) {
+            // (with the lanes of full classes, fewer classes need no more than before)
+            for (int k = 0; k < kBuckets; ++k) b->class_pairs[k] = 0x7fffffffu;
+            if (!ring_layout(b)) e = cudaErrorUnknown;
+        }
         if (e == cudaSuccess) e = enqueue_prepare(b, b->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
         if (e == cudaSuccess) e = cudaMemcpy(b->host_counts, b->counts, sizeof(b->host_counts), cudaMemcpyDeviceToHost);

@@ -319,14 +319,14 @@ int launch_request(aim_server* s, Request* r) {
         WfaPlan exact = job.plan;
         int warps = 0;
         if (job.bound_group) {
-            // a bound pass in the job's scratch slice first (the exact pass then reuses the slice); if not one
-            // block of it fits, the exact pass runs alone
+            // a bound pass first: without scratch, or, for costs that wfa_bound.cu does not take, in the job's slice
+            // (the exact pass then reuses it; if not one block of it fits, the exact pass runs alone)
             WfaPlan bp = job.plan;
             bp.bound = reinterpret_cast<int32_t*>(d + L.bound);
             bp.bound_pass = 1;
             int bg = job.bound_group;
             const size_t bwb = wfa_warp_bytes(bg, wfa_bound_pair_bytes(job.plan));
-            if (bound_lanes_ok(job.plan, job.max_len)) {   // one pair per lane, no scratch
+            if (bound_ok(job.plan, job.max_len)) {   // no scratch
                 e = launch_wfa_bound(bp, P, lim, O, order + job.begin, nullptr, counter + 32, s->num_sms, js);
                 exact.bound = bp.bound;
             } else if (8 * bwb <= job.slice_bytes) {
@@ -574,7 +574,6 @@ int aim_server_submit(aim_server* s, const aim_request* q, uint64_t* ticket) {
         // diagonals), where the batched form's tuner keeps one: 4 lanes per pair before groups of up to 32 lanes,
         // 16 before whole blocks.  Results are the exact pass's either way.
         const int key = keyed[i].first, kc = 7 - key / 4, wc = 3 - key % 4;
-        // (one pair per lane where wfa_bound.cu takes the job)
         job.bound_group = kc >= 5 && wc == 3 && jl <= kMaxWfaLength16 ? (job.group > 32 ? 16 : 4) : 0;
         // warps wanted: every pair in flight at once (a 256-lane group uses 8 warps), within the device's capacity
         const size_t want = job.group > 32 ? (size_t)job.count * (job.group / 32)

@@ -1296,6 +1296,11 @@ cudaError_t launch_wfa_buckets(const WfaPlan& plan, const PairsView& P, const Li
     *warps_used = 0;
     if (P.num_pairs == 0) return cudaSuccess;
     if (nbuckets < 1 || nbuckets > kMaxBuckets) return cudaErrorInvalidValue;
+    // one queue of a bound pass: the forms with the window in registers, where the costs allow them
+    if (nbuckets == 1 && plan.bound_pass && plan.bound && plan.adapt_min_len < 0 && bound_ok(plan, P.max_length)) {
+        *warps_used = 1;
+        return launch_wfa_bound(plan, P, L, O, order, bounds, counters, num_sms, st);
+    }
     // one queue of an exact pass: the form with its state in shared memory, where the costs and widths allow it
     if (nbuckets == 1 && !plan.bound_pass) {
         const int G = groups[0] > 32 ? 256 : groups[0];
