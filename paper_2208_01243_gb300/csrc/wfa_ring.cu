@@ -50,7 +50,6 @@ struct RingArgs {
     uint32_t seq_rounds;     // rounds whose copies are kept: G, or 1 and the traceback reads the packed sequences
     uint32_t smem_warp;      // bytes of shared memory per warp
     uint32_t stage_shared;   // runs are staged in shared memory
-    size_t round_bytes;      // history of one round, worst case
     uint32_t sel_x, sel_o;   // byte permute selectors of M~[s-X], M~[s-O] in mh
 };
 
@@ -348,7 +347,6 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
             pos = __shfl_sync(kFull, pos, 0);
         }
         if (pos >= end - begin || end <= begin) break;
-        if (round == kRounds || rounds_bytes - used < r.round_bytes) finish();
 
         // ---- the round's pairs
         const uint32_t q = begin + pos + (uint32_t)g;
@@ -391,6 +389,15 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
         const int wide = P == 1 ? win.last : __reduce_max_sync(kFull, win.last);   // 0: no pair to run
         // entry (s, t-th of its row) of the history at [s * stride + t * P]
         const uint32_t stride = ((uint32_t)wide * P + 31u) & ~31u;
+        // what rows 0 .. S take, from the pairs' own limits and windows: the arena holds more rounds than of the worst case
+        size_t need = 0;
+        if constexpr (kDense) {
+            if (run) need = (size_t)RowMap<P, true>(win, O, 0).start(S + 1) * sizeof(E);
+        } else {
+            const int rows = P == 1 ? S : __reduce_max_sync(kFull, run ? S : 0);
+            if (wide) need = (size_t)(rows + 1) * stride * sizeof(E);
+        }
+        if (round == kRounds || rounds_bytes - used < need) finish();
         int final_s = -1, s = 0;
         uint32_t entries = 0;   // of the round's history
         if (wide) {
@@ -706,7 +713,6 @@ cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, cons
     r.seq_rounds = seq_bytes(len, 32) <= kKeepBytes ? (uint32_t)(32 / pairs_of(G)) : 1u;
     r.stage_shared = (size_t)plan.runs_cap * 33 * 4 <= (size_t)r.width * pairs_of(G) * (8 + (G == 1 ? 4 : 8));
     const size_t min_warp = ring_warp_bytes(plan, G, len);
-    r.round_bytes = min_warp - 32 * plan.runs_bytes;
     // value d scores back: bytes 2 (d - 1) and 2 (d - 1) + 1 of mh, the sign replicated above them
     auto sel = [](int d) { const uint32_t b = 2u * (uint32_t)(d - 1); return b | ((b + 1) << 4) | ((b + 9) << 8) | ((b + 9) << 12); };
     r.sel_x = sel(plan.x);
@@ -721,7 +727,8 @@ cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, cons
     if (n == 0) return cudaSuccess;
     a.nwarps = (uint32_t)n;
     // a unit's arena: its share of the scratch, up to as many worst-case rounds as it defers
-    a.warp_bytes = std::min(scratch_bytes / n & ~(size_t)255, min_warp + (32 / pairs_of(G) - 1) * r.round_bytes);
+    a.warp_bytes = std::min(scratch_bytes / n & ~(size_t)255,
+                            min_warp + (32 / pairs_of(G) - 1) * (min_warp - 32 * plan.runs_bytes));
     ring_kernel(G, len)<<<(unsigned)((n + units - 1) / units), threads, smem, st>>>(r);
     e = cudaGetLastError();
     if (e == cudaSuccess) *warps_used = (int)n;
