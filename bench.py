@@ -374,10 +374,12 @@ def run_ours(args, w, algo):
             aim.aim_batch_run(plan)
         # kernels per replay: 2 pack and 3 bucketing launches, then one alignment launch per group of buckets sharing
         # lanes per pair and bound-pass lanes, plus one bound-pass launch per group that has one; a compact first pass
-        # instead adds the second pass's count/scan/scatter and its alignment launches
+        # instead adds the second pass's count/scan/scatter and its alignment launches; a plan whose bound pass runs in
+        # registers (1) has one such launch, buckets its pairs again (3) and has at least one launch per filled class
         first_eff = [f or g for f, g in zip(first_pass, full_pass)]
         keys = set(zip(full_pass, bound_pass))
         launches_per_step = 5 + (len(set(first_eff)) + 3 + len(set(full_pass)) if n_compact
+                                 else 4 + sum(1 for c in counts if c) if 1 in bound_pass
                                  else len(keys) + sum(1 for _, b in keys if b))
     else:
         def step(src=None):
@@ -559,13 +561,13 @@ def run_ours(args, w, algo):
     launches = max(align_n, 1)
     if algo in ("wfa", "wfa_adaptive"):
         ops = stats["wf_entries"] * OPS_WF_ENTRY + stats["extend_windows"] * OPS_EXT_WINDOW
-        kernel = "wfa_kernel"
+        kernel = "wfa_ring_kernel" if algo == "wfa" else "wfa_adapt_kernel"
     elif algo == "genasm":
         ops = stats["bitap_words"] * OPS_BITAP_WORD
         kernel = "genasm_kernel"
     else:
         ops = stats["dp_cells"] * (OPS_UNIT_CELL if algo == "edit" else OPS_GOTOH_CELL)
-        kernel = "dp_kernel"
+        kernel = "dp_lane_kernel"
     ops_per_launch = ops / launches
     kern_s = align_ms / launches / 1e3
     achieved = ops_per_launch / kern_s / 1e12
