@@ -575,7 +575,8 @@ void (*ring_kernel_for(int G))(RingArgs) {
 
 // Lanes per pair: the fewest whose warps fit an SM at least 16 at a time (14 KB of shared memory each), since one lane
 // per pair wastes no lane on a row's end and shares a row's fixed work between the most pairs; more when the batch
-// would otherwise give the device less than 8 warps per SM, where the pair's own serial chain is what counts.
+// would otherwise give the device less than 8 warps per SM, where the pair's own serial chain is what counts, up to the
+// lanes that the widest row gives work to (1,270 pairs, 2 edits: 18.0 us with 8 lanes, 18.1 with 32).
 // Measured, ms at 1 / 2 / 4 / 8 / 16 lanes: 1M x 150 bp, 6 edits (12 KB at 1 lane) 1.15 / 1.24 / 1.50 / 1.99 / 2.89;
 // 1M x 250 bp, 25 edits, band 25 (12 KB at 4) 13.4 / 10.7 / 9.8 / 10.4 / 12.8; 300k x 300 bp, 30 edits (11 KB at 8)
 // 12.6 / 12.2 / 5.7 / 4.6 / 4.9; 10k x 150 bp 0.080 / 0.067 / 0.060 / 0.064 / 0.073; 61 x 150 bp 0.072 / 0.056 /
@@ -658,7 +659,8 @@ bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_byte
 int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes) {
     int G = 1;
     while (G < 32 && (ring_smem_per_warp(p, G, max_length) > kGoodSmem ||
-                      (uint64_t)num_pairs * G < (uint64_t)num_sms * kGoodWarps * 32))
+                      ((uint64_t)num_pairs * G < (uint64_t)num_sms * kGoodWarps * 32 &&
+                       G < ring_width(p, max_length) - 2)))
         G *= 2;
     while (G <= 32 && !ring_fits(p, G, max_length, scratch_bytes)) G *= 2;
     if (G > 32 || (G == 32 && ring_smem_per_warp(p, G, max_length) > kBlockSmem)) G = 256;
@@ -676,11 +678,13 @@ RingKernel ring_kernel(int G, uint32_t max_length) {
 // units of a grid that fills the device (0: none fits)
 cudaError_t ring_grid(const WfaPlan& p, int G, uint32_t max_length, int num_sms, size_t* n) {
     const RingKernel kernel = ring_kernel(G, max_length);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    const size_t smem = units_of(G) * ring_smem_per_warp(p, G, max_length);
+    cudaError_t e = cudaSuccess;
+    if (smem > (48u << 10))   // what a launch may use unasked; small calls are short enough for the call to count
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (e != cudaSuccess) return e;
     int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, G > 32 ? G : 32 * kWarpsPerBlock,
-                                                      units_of(G) * ring_smem_per_warp(p, G, max_length));
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, G > 32 ? G : 32 * kWarpsPerBlock, smem);
     *n = (size_t)num_sms * (size_t)std::max(bps, 0) * units_of(G);
     return e;
 }
