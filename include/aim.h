@@ -361,12 +361,13 @@ AIM_API int aim_set_batch_compact(aim_ctx *ctx, int mode);
  * runs with min(limit, bound) as the pair's limit, and its clamp keeps only
  * a diamond around the optimal paths.  Scores, flags and CIGARs are those of
  * the exact pass alone.  aim_batch_bound_passes reports, per bucket, the
- * bound pass's lanes per pair (0: none; 1: the form with its few
- * diagonals in registers, a lane or a warp per pair) and returns the number of buckets with one.  aim_set_batch_bound sets how later plans of the context choose:
- * 0 (default) by timed trials when autotuning, or, with wavefronts in shared
- * memory, for every class that may reach a scaled score of 48 (but a batch
- * that makes one small class); 1 always (reads
- * up to 32,000 bp), 2 never.  Plans with a compact first pass run no bound pass.  Work
+ * bound pass's lanes per pair (0: none; 1: the form with its few diagonals in
+ * registers, a lane or a warp per pair) and returns the number of buckets with
+ * one.  aim_set_batch_bound sets how later plans of the context choose: 0
+ * (default) by timed trials when autotuning, or, with wavefronts in shared
+ * memory, for every class that may reach a scaled score of 48 (but not for a
+ * batch that makes one small class); 1 always (reads up to 32,000 bp), 2
+ * never.  Plans with a compact first pass run no bound pass.  Work
  * counters [0] and [1] include the bound pass's entries and windows.
  */
 AIM_API int aim_batch_bound_passes(aim_batch *batch, int *bound_pass /* host[32] */);
