@@ -585,6 +585,7 @@ constexpr size_t kGoodSmem = 14u << 10;
 constexpr int kGoodWarps = 8;
 constexpr size_t kBlockSmem = 20u << 10;   // a whole block per pair where a warp's state takes more
 constexpr size_t kMaxSmem = 226u << 10;   // dynamic shared memory a block may use (227 KB, less its static few bytes)
+constexpr size_t kPlainSmem = 47u << 10;  // ... and without asking for it (48 KB, less the same)
 
 int entry_form(uint32_t max_length) {
     return max_length <= kNarrowLength ? kWhole : max_length <= kMaxWfaLength16c ? kBits16 : kBits32;
@@ -680,7 +681,7 @@ cudaError_t ring_grid(const WfaPlan& p, int G, uint32_t max_length, int num_sms,
     const RingKernel kernel = ring_kernel(G, max_length);
     const size_t smem = units_of(G) * ring_smem_per_warp(p, G, max_length);
     cudaError_t e = cudaSuccess;
-    if (smem > (48u << 10))   // what a launch may use unasked; small calls are short enough for the call to count
+    if (smem > kPlainSmem)   // small calls are short enough for the call to count
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (e != cudaSuccess) return e;
     int bps = 0;

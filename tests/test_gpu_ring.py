@@ -1,6 +1,10 @@
 """The shared-memory wavefront form (wfa_ring.cu) against the oracle, for every number of lanes per pair: at lengths
 around a packed word and around the 10-bit history's limit, at thresholds of one gap up to wide windows, with a band,
 with thresholds that differ from pair to pair, and over end diagonals far from 0."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -82,3 +86,25 @@ def test_ring_history_forms(aligner, length, edits, lanes):
         aim.aim_set_wfa_group(aligner.ctx, 0)
     assert_same(dev, oracle_results(p, w.penalties, np.full(len(p), 8 * edits, np.int64)),
                 what=f"ring, {length} bp, {lanes} lanes")
+
+
+@pytest.mark.parametrize("length,edits", [(9952, 690), (9921, 689), (9920, 690), (9953, 690), (2000, 752)])
+def test_ring_shared_memory_around_48_kb(length, edits):
+    """16 (W + ceil(length / 32) + 1) bytes of dynamic shared memory for a block per pair, W = 4 edits: 48 KB to the byte
+    (beside which the kernel has a few static ones), a step below and a step above.  A process of its own for each: an
+    earlier launch of the same kernel would already have asked for more."""
+    code = f"""
+import numpy as np
+import __graft_entry__
+__graft_entry__.build()
+import gen
+from devutil import assert_same, device_results, oracle_results
+w = gen.Workload("ring_48k", 5, 3, {length} - 40, {length} - 40, 0.002, 0.002, 0.0, "wfa", (0, 4, 6, 2), 30)
+p = gen.generate(w)
+dev = device_results(p, "wfa", w.penalties, {edits}, max_length={length}, workspace=1 << 30)
+assert_same(dev, oracle_results(p, w.penalties, np.full(len(p), 8 * {edits}, np.int64)), what="48 KB")
+"""
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([here, os.path.dirname(here)]))
+    r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
