@@ -301,8 +301,8 @@ AIM_API int aim_set_genasm_window(aim_ctx *ctx, int window, int overlap);
  *     are classes of the largest scaled score a pair may reach, pairs are
  *     bucketed again by min(limit, bound) after a bound pass (below), and each
  *     class is one launch, on streams of the plan's own; thin classes are merged
- *     at planning.  Lanes per pair and bound passes follow from the class, or
- *     from an earlier cached choice; `autotune` caches them and runs no trials;
+ *     at planning.  Lanes per pair and bound passes follow from the class and
+ *     its pairs; `autotune` runs no trials and only records them (below);
  *   - otherwise buckets are work and width classes, and with `autotune` the lanes
  *     per pair of every non-empty one are chosen by timed trial launches on a
  *     device-filling sample of its pairs (each choice cached in the context per
@@ -377,7 +377,10 @@ AIM_API int aim_set_batch_bound(aim_ctx *ctx, int mode);
  * did.  The context caches, per (costs, band, bucket, largest scaled score),
  * the lanes per pair, the compact first-pass lanes (0: none) and the
  * bound-pass lanes (0: none) its plans chose; plans made with autotune 0 take
- * cached choices where present.  aim_tune_export writes the cache as text,
+ * cached choices where present.  Plans with wavefronts in shared memory choose
+ * by a rule, which plans the same batch the same way in any process: their
+ * choices are cached for the record, bucket 32 and up naming the class of
+ * limits, and are not taken.  aim_tune_export writes the cache as text,
  * one line "x o e band bucket smax lanes compact bound" per entry, into buf
  * (host, cap bytes, always NUL-terminated when cap > 0) and returns the
  * text's length without the NUL (a larger value than cap - 1 means buf was

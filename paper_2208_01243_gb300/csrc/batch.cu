@@ -265,7 +265,6 @@ struct aim_batch {
     // plans of wfa_ring.cu: one exact launch per class of limits, side by side on streams of their own
     bool ring;
     bool few;                               // pairs for too few rounds of the launches for a bound pass to pay
-    bool tuning;                            // autotune: cached choices are not taken
     uint32_t class_pairs[aim::kBuckets];    // pairs of each class seen at planning (before: as many as fill any launch)
     uint32_t* cclaims;
     size_t class_at[aim::kBuckets], class_bytes[aim::kBuckets];   // each class's part of the scratch
@@ -325,11 +324,16 @@ WfaPlan class_plan(const aim_batch* b, int k) {   // bucket k
     return p;
 }
 
-const TuneChoice* cached_choice(const aim_batch* b, int k) {
-    if (!b->ctx->tune_cache) return nullptr;
-    auto& c = tune_cache(b->ctx);
-    const auto it = c.find(TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, b->pen.band, k, b->plan.smax));
-    return it == c.end() ? nullptr : &it->second;
+// The classes' upper edges before any are merged: kFirstEdge, a quarter more each, and the plan's own largest limit last.
+constexpr double kFirstEdge = 24.0, kEdgeStep = 1.25;
+
+// Bucket k's number in the cache of choices: kBuckets and up, by its upper edge's place among those edges, which does not
+// change with the batch (k does: planning merges classes).
+int class_id(const aim_batch* b, int k) {
+    const int64_t edge = b->bp.edge[b->bp.nclasses - 1 - k];
+    int i = 0;
+    for (double e = kFirstEdge; i + 1 < kBuckets && (int64_t)e < edge; e *= kEdgeStep) ++i;
+    return kBuckets + i;
 }
 
 bool ring_bounded(const aim_batch* b) {
@@ -416,16 +420,12 @@ bool ring_layout(aim_batch* b) {
         b->groups1[k] = b->bound1[k] = 0;
         if (k >= nc) { b->groups[k] = 32; continue; }
         const WfaPlan p = class_plan(b, k);
-        // cached choices (an earlier plan's, or imported), else the rule of wfa_ring.cu for a batch that fills the
-        // device, and a bound pass with one pair per lane, or a warp per pair for longer reads
-        const TuneChoice* cached = b->tuning ? nullptr : cached_choice(b, k);
-        b->groups[k] = cached && ring_fits(p, std::get<0>(*cached), b->max_length, b->scratch_bytes)
-                           ? std::get<0>(*cached)
-                           : ring_group(p, b->max_length, b->class_pairs[k], b->ctx->num_sms, b->scratch_bytes);
+        // lanes by the rule of wfa_ring.cu for the class's pairs, and a bound pass with one pair per lane, or a warp per
+        // pair for longer reads.  The rule looks at this batch, so cached choices, made for another, are not taken.
+        b->groups[k] = ring_group(p, b->max_length, b->class_pairs[k], b->ctx->num_sms, b->scratch_bytes);
         const bool regs = bound_ok(b->plan, b->max_length);
         const int mode = b->ctx->batch_bound;
-        int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore || b->few ? 0 : regs ? 1 : 32;
-        if (mode == 0 && cached && (std::get<2>(*cached) != 1 || regs)) gb = std::get<2>(*cached);
+        const int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore || b->few ? 0 : regs ? 1 : 32;
         b->bound1[k] = mode == 2 || b->max_length > kMaxWfaLength16 ? 0 : gb;
         want[k] = b->groups[k] ? ring_full_scratch(p, b->groups[k], b->max_length, b->ctx->num_sms) : 0;
         if (!want[k]) return false;
@@ -460,7 +460,7 @@ bool ring_layout(aim_batch* b) {
 bool plan_ring(aim_batch* b) {
     if (!ring_ok(b->plan, b->max_length) || b->ctx->batch_compact == 1) return false;
     int nc = 0;
-    for (double edge = 24.0; nc < kBuckets; edge *= 1.25) {
+    for (double edge = kFirstEdge; nc < kBuckets; edge *= kEdgeStep) {
         const bool last = (int64_t)edge >= b->plan.smax || nc == kBuckets - 1;
         b->bp.edge[nc++] = (int32_t)(last ? b->plan.smax : (int64_t)edge);
         if (last) break;
@@ -774,7 +774,6 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
     e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) { free_batch(b); return cuda_status(e); }
 
-    b->tuning = autotune != 0;
     for (int k = 0; k < kBuckets; ++k) b->class_pairs[k] = 0x7fffffffu;
     b->ring = plan_ring(b);
     // the scratch has to hold the general kernels' worst case at one pair per warp or per block, whichever kernels run:
@@ -817,8 +816,8 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
         if (e != cudaSuccess) { free_batch(b); return cuda_status(e); }
         for (int k = 0; autotune && k < b->bp.nclasses; ++k)
             if (b->host_counts[k])
-                tune_cache(ctx)[TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, pen->band, k, b->plan.smax)] =
-                    TuneChoice(b->groups[k], 0, b->bound1[k]);
+                tune_cache(ctx)[TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, pen->band, class_id(b, k),
+                                        b->plan.smax)] = TuneChoice(b->groups[k], 0, b->bound1[k]);
     } else if (autotune) {
         rc = aim::autotune(b);
         if (rc) { free_batch(b); return rc; }
@@ -1031,7 +1030,8 @@ int aim_tune_import(aim_ctx* ctx, const char* text) {
             return AIM_ERR_ARG;
         const auto lanes_ok = [](int v, bool zero) { return (zero && v == 0) || v == 1 || v == 2 || v == 4 ||
                                                             v == 8 || v == 16 || v == 32 || v == 256; };
-        if (bucket < 0 || bucket >= aim::kBuckets || !lanes_ok(g, false) || !lanes_ok(g1, true) ||
+        if (bucket < 0 || bucket >= 2 * aim::kBuckets ||   // (from kBuckets on: class_id)
+            !lanes_ok(g, false) || !lanes_ok(g1, true) ||
             !(gb == 0 || gb == 1 || gb == 4 || gb == 8 || gb == 16 || gb == 32))
             return AIM_ERR_ARG;
         parsed.emplace_back(aim::TuneKey(x, o, e, band, bucket, (int64_t)smax), aim::TuneChoice(g, g1, gb));

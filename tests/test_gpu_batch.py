@@ -205,3 +205,45 @@ def test_batched_replay_sees_new_contents(gen_lib):
     aim.aim_batch_destroy(plan); al.close()
     assert np.array_equal(a, device_results(p1, "wfa", AFF, 6)[0])
     assert np.array_equal(b, device_results(p2, "wfa", AFF, 6)[0])
+
+
+def _plan_of(al, p, me, autotune, ml=None, pen=(4, 6, 2)):
+    """A plan over the pairs: (lanes, first-pass lanes, bound-pass lanes) per bucket and the pairs' scores and flags."""
+    import torch
+    import paper_2208_01243_gb300 as aim
+    reads, targets, ro, to, rl, tl, pp = aim.upload(p.reads, p.targets, p.read_off, p.target_off, p.read_len,
+                                                    p.target_len, me.astype(np.int32))
+    out = al.outputs(len(p))
+    ml = int(ml or max(p.read_len.max(), p.target_len.max()))
+    plan = aim.aim_batch_plan(al.ctx, reads, targets, ro, to, rl, tl, ml, aim.penalties(*pen), int(me.max()), pp,
+                              out["scores"], None, None, out["cigar_lens"], out["flags"], autotune=autotune)
+    aim.aim_batch_run(plan); torch.cuda.synchronize()
+    first, full, _ = aim.aim_batch_passes(plan)
+    res = ((full, first, aim.aim_batch_bound_passes(plan)[0]),
+           (out["scores"].cpu().numpy().copy(), out["flags"].cpu().numpy().copy()))
+    aim.aim_batch_destroy(plan)
+    return res
+
+
+def test_choices_of_one_batch_do_not_reach_another(gen_lib):
+    """A context that tuned a small batch, and one that imported its choices, plan a large batch of the same costs and
+    thresholds as a fresh context does."""
+    import paper_2208_01243_gb300 as aim
+    p, me = _mixed(20_000, 0)
+    small = gen.concat([gen.from_strings([p.read(i)], [p.target(i)]) for i in range(60)])
+    few = me[:60].copy(); few[0] = me.max()
+    al = aim.Aligner(0, 1 << 30)
+    fresh, want = _plan_of(al, p, me, autotune=False)
+    al.close()
+    al = aim.Aligner(0, 1 << 30)
+    tuned, _ = _plan_of(al, small, few, autotune=True)
+    assert tuned[0] != fresh[0]                      # the small batch takes other lanes
+    text = aim.aim_tune_export(al.ctx)
+    assert text
+    again, got = _plan_of(al, p, me, autotune=False)
+    al.close()
+    assert again == fresh and all(np.array_equal(a, b) for a, b in zip(got, want))
+    al = aim.Aligner(0, 1 << 30)
+    aim.aim_tune_import(al.ctx, text)
+    assert _plan_of(al, p, me, autotune=False)[0] == fresh
+    al.close()
