@@ -742,6 +742,15 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
             auto& c = tune_cache(ctx);
             auto it = c.find(TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, pen->band, k, b->plan.smax));
             if (it != c.end()) std::tie(b->groups[k], b->groups1[k], b->bound1[k]) = it->second;
+            // the key has no lengths: a choice for shorter reads gives way where these need 32-bit offsets, which
+            // groups of at least 32 lanes hold and bound passes don't
+            if (max_length > kMaxWfaLength16) {
+                b->groups[k] = std::max(b->groups[k], 32);
+                if (b->groups1[k] < 32) b->groups1[k] = 0;
+                b->bound1[k] = 0;
+            }
+            // (1, the form in registers, may have been imported for costs it does not take)
+            if (b->bound1[k] == 1 && !bound_ok(b->plan, max_length)) b->bound1[k] = kBoundDefaultGroup;
         }
     }
     // owned memory: packed sequences, flags, bucket arrays, order, scratch

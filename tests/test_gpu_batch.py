@@ -247,3 +247,30 @@ def test_choices_of_one_batch_do_not_reach_another(gen_lib):
     aim.aim_tune_import(al.ctx, text)
     assert _plan_of(al, p, me, autotune=False)[0] == fresh
     al.close()
+
+
+def test_cached_choices_for_longer_reads(oracle_lib, gen_lib):
+    """Choices tuned on short reads, or imported, for costs of the general kernels (a gap opening of 6 scaled units): a plan
+    whose reads may pass 32,000 bp keeps to groups of 32 lanes and up without a bound pass, and bound lanes of 1 become 4
+    where the form in registers does not take the costs."""
+    import paper_2208_01243_gb300 as aim
+    pen = (0, 4, 6, 1)
+    w = gen.Workload("tuned", 12, 600, 100, 260, 0.0, 0.06, 0.1, "wfa", pen, 12)
+    p = gen.generate(w)
+    me = np.full(len(p), 12, np.int32)
+    lim = np.full(len(p), 12 * 7, np.int64)
+    want = oracle_results(p, pen, lim)
+    al = aim.Aligner(0, 1 << 30)
+    (full, first, bound), res = _plan_of(al, p, me, autotune=True, pen=pen[1:])
+    text = aim.aim_tune_export(al.ctx)
+    lines = [[int(v) for v in line.split()] for line in text.splitlines()]
+    assert lines
+    for change in (lambda v: v, lambda v: v[:6] + [4, 4, 1], lambda v: v[:6] + [8, 0, 1]):
+        aim.aim_tune_import(al.ctx, "".join(" ".join(map(str, change(v))) + "\n" for v in lines))
+        (full, first, bound), res = _plan_of(al, p, me, autotune=False, ml=33_000, pen=pen[1:])
+        assert min(full) >= 32 and set(first) <= {0, 32, 256} and not any(bound)
+        assert np.array_equal(res[0], want[0]) and np.array_equal(res[1], want[1])
+    (full, first, bound), res = _plan_of(al, p, me, autotune=False, pen=pen[1:])
+    assert 4 in bound and set(bound) <= {0, 4} and 8 in full
+    assert np.array_equal(res[0], want[0]) and np.array_equal(res[1], want[1])
+    al.close()
