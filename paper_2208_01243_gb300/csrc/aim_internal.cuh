@@ -213,13 +213,18 @@ struct WfaArgs {
     int16_t group[kMaxBuckets]; // lanes per pair of each bucket (1..32, or 256: a whole block)
 };
 
-// bucketed queues (longest-first order given by the caller): one launch per distinct group size among the
-// buckets, each draining the buckets of its size; warps_used: the largest grid (0: nothing fitted)
+// bucketed queues (longest-first order given by the caller) on wfa.cu's kernels: one launch per distinct group size among
+// the buckets, each draining the buckets of its size; warps_used: the largest grid (0: nothing fitted)
 cudaError_t launch_wfa_buckets(const WfaPlan& plan, const PairsView& P, const LimitView& L, const OutView& O,
                                const uint32_t* order, const uint32_t* bounds, const int* groups, int nbuckets,
                                size_t warp_bytes, uint8_t* scratch, size_t scratch_bytes, uint32_t* counters,
                                int num_sms, cudaStream_t st, int* warps_used);
-// one launch over all pairs in index order with `group` lanes per pair
+// one queue (order positions bounds[0..1], or all pairs) by the form that takes it: wfa_bound.cu for a bound pass and
+// wfa_ring.cu for an exact one where costs, lengths and scratch allow, else launch_wfa_buckets
+cudaError_t launch_wfa_queue(const WfaPlan& plan, int group, const PairsView& P, const LimitView& L, const OutView& O,
+                             const uint32_t* order, const uint32_t* bounds, size_t warp_bytes, uint8_t* scratch,
+                             size_t scratch_bytes, uint32_t* counter, int num_sms, cudaStream_t st, int* warps_used);
+// one launch_wfa_queue over all pairs in index order with `group` lanes per pair
 cudaError_t launch_wfa(const WfaPlan& plan, int group, const PairsView& P, const LimitView& L, const OutView& O,
                        uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms, cudaStream_t st,
                        int* warps_used);

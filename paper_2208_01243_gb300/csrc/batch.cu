@@ -524,16 +524,16 @@ cudaError_t enqueue_align(aim_batch* b, cudaStream_t st, int* warps) {
                 bp.bound = b->bound;
                 bp.bound_pass = 1;
                 const size_t wb = wfa_warp_bytes(b->gbound[j], wfa_bound_pair_bytes(b->plan));
-                const cudaError_t e = launch_wfa_buckets(bp, b->P, b->r.lim, b->O, b->order, b->gbounds + j,
-                                                         &b->gbound[j], 1, wb, b->scratch, b->scratch_bytes,
-                                                         b->rclaims + j, b->ctx->num_sms, st, &w);
+                const cudaError_t e = launch_wfa_queue(bp, b->gbound[j], b->P, b->r.lim, b->O, b->order,
+                                                       b->gbounds + j, wb, b->scratch, b->scratch_bytes,
+                                                       b->rclaims + j, b->ctx->num_sms, st, &w);
                 if (e != cudaSuccess) return e;
                 if (w == 0) { *warps = 0; return cudaSuccess; }
                 exact.bound = b->bound;
             }
-            const cudaError_t e = launch_wfa_buckets(exact, b->P, b->r.lim, b->O, b->order, b->gbounds + j,
-                                                     &b->ggroup[j], 1, b->gwarp_bytes[j], b->scratch,
-                                                     b->scratch_bytes, b->claims + j, b->ctx->num_sms, st, &w);
+            const cudaError_t e = launch_wfa_queue(exact, b->ggroup[j], b->P, b->r.lim, b->O, b->order,
+                                                   b->gbounds + j, b->gwarp_bytes[j], b->scratch, b->scratch_bytes,
+                                                   b->claims + j, b->ctx->num_sms, st, &w);
             if (e != cudaSuccess) return e;
             if (w == 0) { *warps = 0; return cudaSuccess; }
             *warps = std::max(*warps, w);
@@ -565,8 +565,9 @@ cudaError_t enqueue_align(aim_batch* b, cudaStream_t st, int* warps) {
     return e;
 }
 
-// one timed trial launch over order positions tb[0]..tb[1] with G lanes per pair and warp_bytes of scratch
-cudaError_t trial(aim_batch* b, const WfaPlan& plan, const uint32_t tb[2], int G, size_t wb, cudaEvent_t t0,
+// one timed trial launch over order positions tb[0]..tb[1] with G lanes per pair and wb bytes of scratch a warp, by the
+// form that a one-pass plan runs, or on wfa.cu's kernels, as both passes of a two-pass plan do
+cudaError_t trial(aim_batch* b, const WfaPlan& plan, const uint32_t tb[2], int G, size_t wb, bool two_pass, cudaEvent_t t0,
                   cudaEvent_t t1, float* ms) {
     cudaStream_t st = b->stream;
     cudaError_t e = cudaMemcpyAsync(b->trial_bounds, tb, 2 * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
@@ -574,8 +575,10 @@ cudaError_t trial(aim_batch* b, const WfaPlan& plan, const uint32_t tb[2], int G
     if (e == cudaSuccess) e = cudaEventRecord(t0, st);
     int w = 0;
     if (e == cudaSuccess)
-        e = launch_wfa_buckets(plan, b->P, b->r.lim, b->O, b->order, b->trial_bounds, &G, 1, wb, b->scratch,
-                               b->scratch_bytes, b->claims, b->ctx->num_sms, st, &w);
+        e = two_pass ? launch_wfa_buckets(plan, b->P, b->r.lim, b->O, b->order, b->trial_bounds, &G, 1, wb, b->scratch,
+                                          b->scratch_bytes, b->claims, b->ctx->num_sms, st, &w)
+                     : launch_wfa_queue(plan, G, b->P, b->r.lim, b->O, b->order, b->trial_bounds, wb, b->scratch,
+                                        b->scratch_bytes, b->claims, b->ctx->num_sms, st, &w);
     if (e == cudaSuccess) e = cudaEventRecord(t1, st);
     if (e == cudaSuccess) e = cudaEventSynchronize(t1);
     if (e == cudaSuccess) e = cudaEventElapsedTime(ms, t0, t1);
@@ -594,14 +597,16 @@ bool compact_allowed(const aim_batch* b, int k, int G1, int g_full) {
            wfa_warp_bytes(g_full, full) <= b->scratch_bytes;
 }
 
-int autotune(aim_batch* b) {
-    cudaEvent_t t0, t1;
-    if (cudaEventCreate(&t0) != cudaSuccess || cudaEventCreate(&t1) != cudaSuccess) return AIM_ERR_CUDA;
-    uint32_t bounds[kBuckets + 1];
-    cudaError_t e = cudaMemcpy(bounds, b->bounds, sizeof(bounds), cudaMemcpyDeviceToHost);
+// The fastest choices of every bucket with pairs: for a plan of one pass, each bucket by the form that takes it, or, with
+// two_pass, for a plan that may give buckets a compact first pass and then runs wfa.cu's kernels throughout.  total: the
+// choices' time over all pairs.
+cudaError_t tune_buckets(aim_batch* b, const uint32_t* bounds, bool two_pass, cudaEvent_t t0, cudaEvent_t t1,
+                         TuneChoice* choices, double* total) {
     const size_t min_warps = (size_t)b->ctx->num_sms * 8;
     WfaPlan retry = b->plan;
     retry.retry_only = 1;
+    cudaError_t e = cudaSuccess;
+    *total = 0.0;
     for (int k = 0; k < kBuckets && e == cudaSuccess; ++k) {
         const uint32_t count = b->host_counts[k];
         if (!count) continue;
@@ -611,7 +616,7 @@ int autotune(aim_batch* b) {
         const uint32_t tb[2] = {bounds[k], bounds[k] + sample};
         float best = 1e30f;
         int best_g = b->groups[k];
-        const WfaPlan exact = bucket_plan(b->plan, k);
+        const WfaPlan exact = two_pass ? b->plan : bucket_plan(b->plan, k);
         // lanes per pair worth trying for this width class: at most ~64 diagonals per lane and score step
         const int wc = kWidthClasses - 1 - k % kWidthClasses;
         const int gmin = wc == 0 ? 1 : wc == 1 ? 2 : wc == 2 ? 4 : 8;
@@ -621,12 +626,12 @@ int autotune(aim_batch* b) {
             const size_t wb = wfa_warp_bytes(G, bucket_pair_bytes(b->plan, k, G));
             if (wb * min_warps > b->scratch_bytes) continue;
             float ms = 0.f;
-            for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) e = trial(b, exact, tb, G, wb, t0, t1, &ms);
+            for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) e = trial(b, exact, tb, G, wb, two_pass, t0, t1, &ms);
             if (e == cudaSuccess && ms < best) { best = ms; best_g = G; }
         }
         // compact first pass with fewer lanes, then the full-scratch pass over the pairs that outgrew it
         int best_g1 = 0;
-        if (b->ctx->batch_compact != 2) {
+        if (two_pass) {
             const size_t wb_full = wfa_warp_bytes(best_g, bucket_pair_bytes(b->plan, k, best_g));
             for (int G1 : {4, 8, 16, 32}) {
                 if (!compact_allowed(b, k, G1, best_g)) continue;
@@ -634,13 +639,13 @@ int autotune(aim_batch* b) {
                 if (b->ctx->batch_compact == 1) { best_g1 = G1; break; }   // forced: the fewest lanes that fit
                 float ms1 = 0.f, ms2 = 0.f;
                 for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
-                    e = trial(b, b->plan, tb, G1, wb, t0, t1, &ms1);
-                    if (e == cudaSuccess) e = trial(b, retry, tb, best_g, wb_full, t0, t1, &ms2);
+                    e = trial(b, b->plan, tb, G1, wb, true, t0, t1, &ms1);
+                    if (e == cudaSuccess) e = trial(b, retry, tb, best_g, wb_full, true, t0, t1, &ms2);
                 }
                 if (e == cudaSuccess && ms1 + ms2 < best) { best = ms1 + ms2; best_g1 = G1; }
             }
         }
-        // a bound pass, then the exact pass clamped at each pair's bound (only where no compact pass was chosen)
+        // a bound pass, then the exact pass clamped at each pair's bound (plans of one pass only)
         int best_gb = 0;
         if (best_g1 == 0 && b->ctx->batch_bound != 2 && b->max_length <= kMaxWfaLength16) {
             WfaPlan bp = b->plan, ep = exact;
@@ -648,25 +653,56 @@ int autotune(aim_batch* b) {
             bp.bound_pass = 1;
             const size_t wb_full = wfa_warp_bytes(best_g, bucket_pair_bytes(b->plan, k, best_g));
             const size_t bpb = wfa_bound_pair_bytes(b->plan);
+            const bool regs = bound_ok(b->plan, b->max_length);   // one form, in registers and without scratch
             if (b->ctx->batch_bound == 1) {
                 best_gb = kBoundDefaultGroup;   // forced: the default lanes, no trials
             } else {
-                for (int Gb : {4, 8, 16, 32}) {
-                    if (wfa_warp_bytes(Gb, bpb) * min_warps > b->scratch_bytes) continue;
+                for (int Gb : {1, 4, 8, 16, 32}) {
+                    if (regs != (Gb == 1)) continue;
+                    if (!regs && wfa_warp_bytes(Gb, bpb) * min_warps > b->scratch_bytes) continue;
                     float ms1 = 0.f, ms2 = 0.f;
                     for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
-                        e = trial(b, bp, tb, Gb, wfa_warp_bytes(Gb, bpb), t0, t1, &ms1);
-                        if (e == cudaSuccess) e = trial(b, ep, tb, best_g, wb_full, t0, t1, &ms2);
+                        e = trial(b, bp, tb, Gb, wfa_warp_bytes(Gb, bpb), false, t0, t1, &ms1);
+                        if (e == cudaSuccess) e = trial(b, ep, tb, best_g, wb_full, two_pass, t0, t1, &ms2);
                     }
                     if (e == cudaSuccess && ms1 + ms2 < kBoundGain * best) { best = ms1 + ms2; best_gb = Gb; }
                 }
             }
         }
-        b->groups[k] = best_g;
-        b->groups1[k] = best_g1;
-        b->bound1[k] = best_gb;
-        tune_cache(b->ctx)[TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, b->pen.band, k, b->plan.smax)] =
-            TuneChoice(best_g, best_g1, best_gb);
+        choices[k] = TuneChoice(best_g, best_g1, best_gb);
+        *total += (double)best * count / sample;
+    }
+    return e;
+}
+
+int autotune(aim_batch* b) {
+    cudaEvent_t t0, t1;
+    if (cudaEventCreate(&t0) != cudaSuccess || cudaEventCreate(&t1) != cudaSuccess) return AIM_ERR_CUDA;
+    uint32_t bounds[kBuckets + 1];
+    cudaError_t e = cudaMemcpy(bounds, b->bounds, sizeof(bounds), cudaMemcpyDeviceToHost);
+    // Costs that wfa_ring.cu never takes run the same kernels either way: one round of trials, compact passes among them.
+    // For the others (their scratch was too small for classes, or compact passes are forced) the buckets that fit run
+    // there if no bucket has a compact pass: a round for each kind of plan, and the faster one.
+    const int mode = b->ctx->batch_compact;
+    const bool ring = ring_ok(b->plan, b->max_length);
+    TuneChoice one[kBuckets], two[kBuckets];
+    double t_one = 1e30, t_two = 1e30;
+    if (e == cudaSuccess && (mode == 2 || (mode == 0 && ring))) e = tune_buckets(b, bounds, false, t0, t1, one, &t_one);
+    bool compact = false;
+    if (e == cudaSuccess && mode != 2) {
+        bool allowed = !ring || mode == 1;   // else only if some bucket could have a compact pass at all
+        for (int k = 0; k < kBuckets && !allowed; ++k)
+            for (int G1 : {4, 8, 16, 32}) allowed |= b->host_counts[k] && compact_allowed(b, k, G1, 256);
+        if (allowed) e = tune_buckets(b, bounds, true, t0, t1, two, &t_two);
+        for (int k = 0; allowed && k < kBuckets; ++k) compact |= b->host_counts[k] && std::get<1>(two[k]);
+        // (forced, and no bucket allows one)
+        if (e == cudaSuccess && mode == 1 && ring && !compact) e = tune_buckets(b, bounds, false, t0, t1, one, &t_one);
+    }
+    const TuneChoice* use = t_one > 1e29 || (compact && t_two < t_one) ? two : one;
+    for (int k = 0; k < kBuckets && e == cudaSuccess; ++k) {
+        if (!b->host_counts[k]) continue;
+        std::tie(b->groups[k], b->groups1[k], b->bound1[k]) = use[k];
+        tune_cache(b->ctx)[TuneKey(b->r.costs.x, b->r.costs.o, b->r.costs.e, b->pen.band, k, b->plan.smax)] = use[k];
     }
     cudaEventDestroy(t0);
     cudaEventDestroy(t1);

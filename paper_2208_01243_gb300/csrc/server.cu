@@ -324,20 +324,17 @@ int launch_request(aim_server* s, Request* r) {
             WfaPlan bp = job.plan;
             bp.bound = reinterpret_cast<int32_t*>(d + L.bound);
             bp.bound_pass = 1;
-            int bg = job.bound_group;
+            const int bg = job.bound_group;
             const size_t bwb = wfa_warp_bytes(bg, wfa_bound_pair_bytes(job.plan));
-            if (bound_ok(job.plan, job.max_len)) {   // no scratch
-                e = launch_wfa_bound(bp, P, lim, O, order + job.begin, nullptr, counter + 32, s->num_sms, js);
-                exact.bound = bp.bound;
-            } else if (8 * bwb <= job.slice_bytes) {
-                e = launch_wfa_buckets(bp, P, lim, O, order + job.begin, nullptr, &bg, 1, bwb, slice, job.slice_bytes,
-                                       counter + 32, s->num_sms, js, &warps);
+            if (bound_ok(job.plan, job.max_len) || 8 * bwb <= job.slice_bytes) {
+                e = launch_wfa_queue(bp, bg, P, lim, O, order + job.begin, nullptr, bwb, slice, job.slice_bytes,
+                                     counter + 32, s->num_sms, js, &warps);
                 if (e == cudaSuccess && warps > 0) exact.bound = bp.bound;
             }
             if (e != cudaSuccess) break;
         }
-        e = launch_wfa_buckets(exact, P, lim, O, order + job.begin, nullptr, &job.group, 1, job.warp_bytes, slice,
-                               job.slice_bytes, counter, s->num_sms, js, &warps);
+        e = launch_wfa_queue(exact, job.group, P, lim, O, order + job.begin, nullptr, job.warp_bytes, slice,
+                             job.slice_bytes, counter, s->num_sms, js, &warps);
         if (e == cudaSuccess && warps == 0) e = cudaErrorMemoryAllocation;
         if (e == cudaSuccess) e = cudaEventRecord(r->events[1 + j], js);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, r->events[1 + j], 0);

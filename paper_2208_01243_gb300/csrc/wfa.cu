@@ -1296,18 +1296,6 @@ cudaError_t launch_wfa_buckets(const WfaPlan& plan, const PairsView& P, const Li
     *warps_used = 0;
     if (P.num_pairs == 0) return cudaSuccess;
     if (nbuckets < 1 || nbuckets > kMaxBuckets) return cudaErrorInvalidValue;
-    // one queue of a bound pass: the forms with the window in registers, where the costs allow them
-    if (nbuckets == 1 && plan.bound_pass && plan.bound && plan.adapt_min_len < 0 && bound_ok(plan, P.max_length)) {
-        *warps_used = 1;
-        return launch_wfa_bound(plan, P, L, O, order, bounds, counters, num_sms, st);
-    }
-    // one queue of an exact pass: the form with its state in shared memory, where the costs and widths allow it
-    if (nbuckets == 1 && !plan.bound_pass) {
-        const int G = groups[0] > 32 ? 256 : groups[0];
-        if (ring_fits(plan, G, P.max_length, scratch_bytes))
-            return launch_wfa_ring(plan, G, P, L, O, order, bounds, scratch, scratch_bytes, counters, num_sms, st,
-                                   warps_used);
-    }
     WfaArgs a;
     a.X = plan.x; a.OE = plan.oe; a.E = plan.e; a.g = plan.g; a.smax = plan.smax; a.band = plan.band;
     a.P = P; a.L = L; a.O = O;
@@ -1403,12 +1391,26 @@ size_t wfa_warp_bytes(int group, size_t pair_bytes) {
     return (size_t)(32 / group) * pair_bytes;
 }
 
+cudaError_t launch_wfa_queue(const WfaPlan& plan, int group, const PairsView& P, const LimitView& L, const OutView& O,
+                             const uint32_t* order, const uint32_t* bounds, size_t warp_bytes, uint8_t* scratch,
+                             size_t scratch_bytes, uint32_t* counter, int num_sms, cudaStream_t st, int* warps_used) {
+    if (plan.bound_pass && bound_ok(plan, P.max_length)) {
+        *warps_used = P.num_pairs != 0;
+        return launch_wfa_bound(plan, P, L, O, order, bounds, counter, num_sms, st);
+    }
+    if (!plan.bound_pass && ring_fits(plan, group, P.max_length, scratch_bytes))
+        return launch_wfa_ring(plan, group, P, L, O, order, bounds, scratch, scratch_bytes, counter, num_sms, st,
+                               warps_used);
+    return launch_wfa_buckets(plan, P, L, O, order, bounds, &group, 1, warp_bytes, scratch, scratch_bytes, counter,
+                              num_sms, st, warps_used);
+}
+
 cudaError_t launch_wfa(const WfaPlan& plan, int group, const PairsView& P, const LimitView& L, const OutView& O,
                        uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms, cudaStream_t st,
                        int* warps_used) {
     const size_t warp_bytes = wfa_warp_bytes(group, wfa_pair_bytes(plan, group));
-    return launch_wfa_buckets(plan, P, L, O, nullptr, nullptr, &group, 1, warp_bytes, scratch, scratch_bytes,
-                              counter, num_sms, st, warps_used);
+    return launch_wfa_queue(plan, group, P, L, O, nullptr, nullptr, warp_bytes, scratch, scratch_bytes, counter, num_sms,
+                            st, warps_used);
 }
 
 }  // namespace aim

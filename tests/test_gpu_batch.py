@@ -274,3 +274,21 @@ def test_cached_choices_for_longer_reads(oracle_lib, gen_lib):
     assert 4 in bound and set(bound) <= {0, 4} and 8 in full
     assert np.array_equal(res[0], want[0]) and np.array_equal(res[1], want[1])
     al.close()
+
+
+@pytest.mark.parametrize("scratch_mb,compact", [(48, 0), (48, 1), (160, 0), (160, 2)])
+def test_plans_short_of_scratch(oracle_lib, gen_lib, scratch_mb, compact):
+    """Scratch too small for classes of limits: buckets tuned by trials, each on the kernels that then run it.  The bound
+    pass of these costs has one form, reported as 1 lane; results are the plain form's."""
+    p = gen.generate(gen.Workload("scratch", 31, 500, 300, 2600, 0.01, 0.15, 0.1, "wfa", AFF, None, max_edits_frac=0.2))
+    me = gen.per_pair_max_edits(gen.Workload("scratch", 31, 500, 300, 2600, 0.01, 0.15, 0.1, "wfa", AFF, None,
+                                             max_edits_frac=0.2), p)
+    bounds, passes = [], []
+    outs, groups, counts = _batched(p, me, True, scratch=scratch_mb << 20, compact=compact, passes=passes, bounds=bounds)
+    assert [k for k in range(32) if counts[k]] == [0, 4, 8]   # work and width classes
+    assert set(bounds[0][0]) <= {0, 1}
+    assert bounds[0][1] or (scratch_mb, compact) != (48, 0)   # (it saves far more than the few per cent it has to)
+    plain = device_results(p, "wfa", AFF, int(me.max()), per_pair=me)
+    for o in outs:
+        assert np.array_equal(o[0], plain[0]) and np.array_equal(o[1], plain[1])
+        assert all(np.array_equal(x, y) for x, y in zip(o[2], plain[2]))
