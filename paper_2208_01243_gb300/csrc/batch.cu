@@ -342,9 +342,9 @@ bool ring_bounded(const aim_batch* b) {
     return false;
 }
 
-// the bound passes, and the counts of the classes that min(limit, bound) puts the pairs in
-cudaError_t enqueue_bounds(aim_batch* b, cudaStream_t st, bool* fits) {
-    *fits = true;
+// the bound passes (these costs take wfa_bound.cu's, whatever lanes are asked for), and the counts of the classes that
+// min(limit, bound) puts the pairs in
+cudaError_t enqueue_bounds(aim_batch* b, cudaStream_t st) {
     const int sms = b->ctx->num_sms;
     cudaError_t e = cudaMemsetAsync(b->bound, 0xff, (size_t)b->num_pairs * sizeof(int32_t), st);   // -1: none
     if (e == cudaSuccess) e = cudaMemsetAsync(b->rclaims, 0, kBuckets * sizeof(uint32_t), st);
@@ -354,15 +354,7 @@ cudaError_t enqueue_bounds(aim_batch* b, cudaStream_t st, bool* fits) {
         WfaPlan bp = b->plan;
         bp.bound = b->bound;
         bp.bound_pass = 1;
-        if (b->gbound[j] == 1) {
-            e = launch_wfa_bound(bp, b->P, b->r.lim, b->O, b->order, b->gbounds + j, b->rclaims + j, sms, st);
-        } else {
-            int w = 0;
-            const size_t wb = wfa_warp_bytes(b->gbound[j], wfa_bound_pair_bytes(b->plan));
-            e = launch_wfa_buckets(bp, b->P, b->r.lim, b->O, b->order, b->gbounds + j, &b->gbound[j], 1, wb, b->scratch,
-                                   b->scratch_bytes, b->rclaims + j, sms, st, &w);
-            *fits = *fits && (e != cudaSuccess || w > 0);
-        }
+        e = launch_wfa_bound(bp, b->P, b->r.lim, b->O, b->order, b->gbounds + j, b->rclaims + j, sms, st);
     }
     if (e != cudaSuccess || b->bp.nclasses == 1) return e;   // one class takes them all
     const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)sms * 8);
@@ -378,9 +370,8 @@ cudaError_t enqueue_ring(aim_batch* b, cudaStream_t st, int* warps) {
     uint32_t* claims = b->claims;
     cudaError_t e = cudaSuccess;
     if (bounded) {
-        bool fits = true;
-        e = enqueue_bounds(b, st, &fits);
-        if (e != cudaSuccess || !fits) return e;
+        e = enqueue_bounds(b, st);
+        if (e != cudaSuccess) return e;
         if (nc > 1) {
             const unsigned blocks = (unsigned)std::min<uint64_t>((b->num_pairs + 255) / 256, (uint64_t)sms * 8);
             bucket_scan_kernel<<<1, 32, 0, st>>>(b->rcounts, b->rbounds, b->rfill, b->cclaims, b->bp, nullptr);
@@ -423,10 +414,9 @@ bool ring_layout(aim_batch* b) {
         // lanes by the rule of wfa_ring.cu for the class's pairs, and a bound pass with one pair per lane, or a warp per
         // pair for longer reads.  The rule looks at this batch, so cached choices, made for another, are not taken.
         b->groups[k] = ring_group(p, b->max_length, b->class_pairs[k], b->ctx->num_sms, b->scratch_bytes);
-        const bool regs = bound_ok(b->plan, b->max_length);
         const int mode = b->ctx->batch_bound;
-        const int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore || b->few ? 0 : regs ? 1 : 32;
-        b->bound1[k] = mode == 2 || b->max_length > kMaxWfaLength16 ? 0 : gb;
+        const int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore || b->few ? 0 : 1;
+        b->bound1[k] = mode == 2 ? 0 : gb;
         want[k] = b->groups[k] ? ring_full_scratch(p, b->groups[k], b->max_length, b->ctx->num_sms) : 0;
         if (!want[k]) return false;
         least[k] = align_up(ring_warp_bytes(p, b->groups[k], b->max_length) * (b->groups[k] > 32 ? 8 : 32), 256);
@@ -839,8 +829,7 @@ int batch_plan_impl(aim_ctx* ctx, const uint8_t* reads, const uint8_t* targets, 
         uint32_t counts[kBuckets];
         std::memcpy(counts, b->host_counts, sizeof(counts));
         if (ring_bounded(b) && b->bp.nclasses > 1) {
-            bool fits = true;
-            e = enqueue_bounds(b, b->stream, &fits);
+            e = enqueue_bounds(b, b->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
             if (e == cudaSuccess) e = cudaMemcpy(counts, b->rcounts, sizeof(counts), cudaMemcpyDeviceToHost);
         }

@@ -176,20 +176,17 @@ __global__ void __launch_bounds__(32 * kBoundWarps) wfa_bound_kernel(BoundArgs r
     warp_stat_add(a.O.stats, 1, st_windows, (uint32_t)lane);
 }
 
-// The same with L lanes per pair, one diagonal of the window in each: neighbours come by shuffles, and a score costs a
-// pair L lanes' instructions but one entry's latency.  The window moves every kLook scores, to have the
-// entry closest to the end in its middle.
+// The same with a warp per pair, one diagonal of the window in each lane: neighbours come by shuffles, and a score costs
+// a pair 32 lanes' instructions but one entry's latency.  The window moves every kLook scores, to have the entry closest
+// to the end in its middle.
 constexpr int kLook = 4;
 
-template <int L>
 __global__ void __launch_bounds__(32 * kBoundWarps) wfa_bound_group_kernel(BoundArgs r) {
     const WfaArgs& a = r.w;
-    const int lane = (int)(threadIdx.x & 31), g = lane / L, gl = lane % L;
+    const int lane = (int)(threadIdx.x & 31);
     const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (gwarp >= a.nwarps) return;
-    const uint32_t mine = (L == 32 ? kFull : (1u << (L & 31)) - 1u) << (g * L);   // the pair's lanes
-    uint32_t* sp = reinterpret_cast<uint32_t*>(s_bound + (size_t)(threadIdx.x >> 5) * r.smem_warp) +
-                   (size_t)g * 2 * r.seq_words;
+    uint32_t* sp = reinterpret_cast<uint32_t*>(s_bound + (size_t)(threadIdx.x >> 5) * r.smem_warp);
     uint32_t* st = sp + r.seq_words;
     const int O = a.OE - 1;
     const uint32_t begin = a.bounds ? a.bounds[0] : 0;
@@ -198,19 +195,17 @@ __global__ void __launch_bounds__(32 * kBoundWarps) wfa_bound_group_kernel(Bound
     uint32_t pi = 0, cells = 0, windows = 0;
     int n = 0, m = 0, S = 0, klo = 0, khi = 0, s = 0;
     int k = 0;          // this lane's diagonal
-    bool run = false;   // this lane's pair is under way
+    bool run = false;   // the warp's pair is under way
     bool more = true;   // the queue may hold pairs
     unsigned long long st_cells = 0, st_windows = 0;
 
     for (;;) {
-        const uint32_t idle = __ballot_sync(kFull, !run);
-        if (more && idle) {
-            uint32_t pos = 0;
-            if (lane == 0) pos = atomicAdd(a.counters, (uint32_t)(__popc(idle) / L));
-            pos = __shfl_sync(kFull, pos, 0);
-            more = begin < end && pos + (uint32_t)(__popc(idle) / L) < end - begin;
-            const uint32_t q = pos + (uint32_t)(__popc(idle & ((1u << (g * L)) - 1u)) / L);
-            bool fresh = !run && begin < end && q < end - begin;
+        if (!run) {
+            uint32_t q = 0;
+            if (lane == 0) q = atomicAdd(a.counters, 1u);
+            q = __shfl_sync(kFull, q, 0);
+            more = begin < end && q + 1 < end - begin;
+            bool fresh = begin < end && q < end - begin;
             if (fresh) {
                 pi = a.order ? a.order[begin + q] : begin + q;
                 n = (int)a.P.read_len[pi];
@@ -224,16 +219,17 @@ __global__ void __launch_bounds__(32 * kBoundWarps) wfa_bound_group_kernel(Bound
                 // (the exact pass reports the others)
                 fresh = !pair_bad(a.P, pi) && (uint32_t)n <= a.P.max_length && (uint32_t)m <= a.P.max_length && lim != -2 &&
                         kend >= klo && kend <= khi && (kend == 0 || abs(kend) + O <= S);
-                if (!fresh && gl == 0) a.bound[pi] = -1;
+                if (!fresh && lane == 0) a.bound[pi] = -1;
             }
+            __syncwarp();   // the last pair's copies have been read
             if (fresh) {
                 const uint64_t* Pw = read_words(a.P, pi);
                 const uint64_t* Tw = target_words(a.P, pi);
-                for (int w = gl; w < (n + 31) >> 5; w += L) {
+                for (int w = lane; w < (n + 31) >> 5; w += 32) {
                     const uint64_t x = __ldg(Pw + w);
                     sp[2 * w] = (uint32_t)(x >> 32); sp[2 * w + 1] = (uint32_t)x;
                 }
-                for (int w = gl; w < (m + 31) >> 5; w += L) {
+                for (int w = lane; w < (m + 31) >> 5; w += 32) {
                     const uint64_t x = __ldg(Tw + w);
                     st[2 * w] = (uint32_t)(x >> 32); st[2 * w + 1] = (uint32_t)x;
                 }
@@ -242,34 +238,32 @@ __global__ void __launch_bounds__(32 * kBoundWarps) wfa_bound_group_kernel(Bound
             if (fresh) {
                 const int m0 = match_on<1>(sp, st, 0, 0, min(n, m));
                 ml = mu = jk = ~0u;
-                k = gl - L / 2;
+                k = lane - 16;
                 if (k == 0) ml = (uint32_t)m0 | 0xffff0000u;
                 s = 0;
                 ++cells; ++windows;
                 run = true;
                 if (n == m && m0 == m) {
-                    if (gl == 0) a.bound[pi] = 0;
+                    if (lane == 0) a.bound[pi] = 0;
                     run = false;
                 }
             }
         }
-        if (!__any_sync(kFull, run)) {
+        if (!run) {
             if (more) continue;
             break;
         }
-        if (run) {
-            ++s;
-            if (s > S) {
-                if (gl == 0) a.bound[pi] = -1;
-                run = false;
-            }
+        if (++s > S) {
+            if (lane == 0) a.bound[pi] = -1;
+            run = false;
+            continue;
         }
-        uint32_t left = __shfl_up_sync(kFull, jk, 1, L), right = __shfl_down_sync(kFull, jk, 1, L);
-        if (gl == 0) left = ~0u;
-        if (gl == L - 1) right = ~0u;
+        uint32_t left = __shfl_up_sync(kFull, jk, 1), right = __shfl_down_sync(kFull, jk, 1);
+        if (lane == 0) left = ~0u;
+        if (lane == 31) right = ~0u;
         bool hit = false;
         int dist = 1 << 30;
-        if (run) {
+        {
             const bool in = k >= klo && k <= khi;
             const int hmax = in ? min(m, n + k) : -1, room = max(hmax, 0);
             const int mo = prmt(ml, mu, r.sel_o);
@@ -297,19 +291,15 @@ __global__ void __launch_bounds__(32 * kBoundWarps) wfa_bound_group_kernel(Bound
             jk = (uint32_t)prmt((uint32_t)max(mo, ins), (uint32_t)max(mo, del), 0x5410u);
             ++cells;
         }
-        if (__ballot_sync(kFull, hit) & mine) {
+        if (__any_sync(kFull, hit)) {
             if (hit) a.bound[pi] = s;
             run = false;
-        }
-        if (__any_sync(kFull, run && s % kLook == 0)) {
-            const bool look = run && s % kLook == 0;
-            int best = look && dist < (1 << 30) ? dist * 32 + gl : INT32_MAX;   // (distances are at most 32,000)
-#pragma unroll
-            for (int o = 1; o < L; o <<= 1) best = min(best, __shfl_xor_sync(kFull, best, o));
-            const int move = best == INT32_MAX ? 0 : (best & 31) - L / 2;
-            const int from = gl + move;
-            const bool have = from >= 0 && from < L;
-            const int src = g * L + (have ? from : gl);
+        } else if (s % kLook == 0) {
+            const int best = __reduce_min_sync(kFull, dist < (1 << 30) ? dist * 32 + lane : INT32_MAX);   // (dist <= 32,000)
+            const int move = best == INT32_MAX ? 0 : (best & 31) - 16;
+            const int from = lane + move;
+            const bool have = from >= 0 && from < 32;
+            const int src = have ? from : lane;
             const uint32_t l = __shfl_sync(kFull, ml, src), u = __shfl_sync(kFull, mu, src), j = __shfl_sync(kFull, jk, src);
             ml = have ? l : ~0u;
             mu = have ? u : ~0u;
@@ -328,7 +318,6 @@ uint32_t bound_seq_words(uint32_t max_length) { return 2 * ((max_length + 31) / 
 // (a word of room before the copies: nothing reads there, an index below them would)
 size_t bound_smem(uint32_t max_length) { return 128 + (size_t)bound_seq_words(max_length) * 256; }
 
-constexpr int kGroupLanes = 32;
 // pairs per SM from which a lane per pair is the faster form: five warps, what 1,000 bp reads leave room for
 constexpr uint32_t kLanePairs = 160;
 constexpr size_t kLaneBoundSmem = 40u << 10;   // shared memory per warp: 5 warps on an SM
@@ -355,9 +344,9 @@ cudaError_t launch_wfa_bound(const WfaPlan& plan, const PairsView& P, const Limi
     auto sel = [](int d) { const uint32_t b = 2u * (uint32_t)(d - 1); return b | ((b + 1) << 4) | ((b + 9) << 8) | ((b + 9) << 12); };
     r.sel_x = sel(plan.x);
     r.sel_o = sel(plan.oe - plan.e);
-    const int per_warp = lanes ? 32 : 32 / kGroupLanes;
+    const int per_warp = lanes ? 32 : 1;
     r.smem_warp = (uint32_t)(lanes ? bound_smem(P.max_length) : (size_t)r.seq_words * 8 * per_warp);
-    void (*kernel)(BoundArgs) = lanes ? wfa_bound_kernel : wfa_bound_group_kernel<kGroupLanes>;
+    void (*kernel)(BoundArgs) = lanes ? wfa_bound_kernel : wfa_bound_group_kernel;
     const size_t smem = (size_t)kBoundWarps * r.smem_warp;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(kBoundWarps * kLaneBoundSmem));

@@ -352,12 +352,8 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
         const uint32_t q = begin + pos + (uint32_t)g;
         int status = kIdle, n = 0, m = 0, S = 0, kend = 0;
         uint32_t pi = 0;
-        bool skip = q >= end;
-        if (!skip) {
+        if (q < end) {
             pi = a.order ? a.order[q] : q;
-            skip = a.retry_only && a.O.flags[pi] != AIM_F_STEP_CAP;
-        }
-        if (!skip) {
             n = (int)a.P.read_len[pi];
             m = (int)a.P.target_len[pi];
             kend = m - n;
@@ -710,7 +706,7 @@ cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, cons
     a.scratch = scratch;
     a.runs_bytes = plan.runs_bytes; a.runs_cap = (uint32_t)plan.runs_cap;
     a.order = order; a.bounds = bounds; a.counters = counters; a.nbuckets = 1;
-    a.bound = plan.bound; a.retry_only = plan.retry_only;
+    a.bound = plan.bound;
     const uint32_t len = P.max_length;
     r.width = (uint32_t)ring_width(plan, len);
     r.seq_words = seq_words(len);
