@@ -34,6 +34,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "ring_rows.h"
 #include "wfa_common.cuh"
 
 namespace aim {
@@ -82,14 +83,6 @@ struct Entry<kWhole> {
     static __device__ __forceinline__ bool from_del(T) { return false; }
 };
 
-// A pair's ring: diagonal k at position k - koff, position 1 the window's first diagonal and `last` its last one;
-// diagonal 0 at `zero`, the end diagonal at `end`.  Row s covers lo(s) .. hi(s).
-struct Window {
-    int koff, last, zero, end, S;
-    __device__ __forceinline__ int lo(int s, int O) const { return max(max(zero - max(s - O, 0), end - (S - s)), 1); }
-    __device__ __forceinline__ int hi(int s, int O) const { return min(min(zero + max(s - O, 0), end + (S - s)), last); }
-};
-
 // What the traceback of a lane's pair needs.
 struct Pending {
     uint32_t pi;
@@ -99,38 +92,17 @@ struct Pending {
     int round;
 };
 
-// Where entry (c, j) of a finished pair lies: row c at c * stride, or, with kDense, rows end to end, row c at the sum
-// of hi(i) - lo(i) + 1 over i < c.  lo(i) is zero - min(g, zero - 1), g = max(i - O, 0), up to row turn_lo and the
-// line end - S + i from there on (the first does not grow with i, the second does); hi(i) likewise.
+// Where entry (c, j) of a finished pair lies: row c at c * stride, or, with kDense, rows end to end.
 template <int P, bool kDense>
 struct RowMap {
     Window w;
     int O;
     uint32_t stride;
-    int turn_lo, turn_hi, sum_lo, sum_hi;   // kDense: the sums of lo, hi up to those rows
-    // sum of min(t, a) over t = 1 .. u
-    static __device__ __forceinline__ int ramp(int u, int a) {
-        u = max(u, 0);
-        const int q = min(u, a);
-        return q * (q + 1) / 2 + (u - q) * a;
-    }
-    __device__ __forceinline__ int early_lo(int c) const { return c * w.zero - ramp(c - 1 - O, w.zero - 1); }
-    __device__ __forceinline__ int early_hi(int c) const { return c * w.zero + ramp(c - 1 - O, w.last - w.zero); }
-    __device__ __forceinline__ RowMap(const Window& win, int o, uint32_t st) : w(win), O(o), stride(st) {
-        if constexpr (kDense) {
-            const int S = w.S, z = w.zero, e = w.end;
-            turn_lo = max(min(z + S - e, (z + O + S - e) >> 1), 1 - e + S);
-            turn_hi = max(min(e + S - z, (e + S - z + O) >> 1), e + S - w.last);
-            sum_lo = early_lo(turn_lo + 1);
-            sum_hi = early_hi(turn_hi + 1);
-        }
-    }
+    DenseRows dense;
+    __device__ __forceinline__ RowMap(const Window& win, int o, uint32_t st) : w(win), O(o), stride(st), dense(win, o) {}
     __device__ __forceinline__ uint32_t start(int c) const {
-        if constexpr (!kDense) return (uint32_t)c * stride;
-        const int dl = c - 1 - turn_lo, dh = c - 1 - turn_hi;
-        const int lo = dl <= 0 ? early_lo(c) : sum_lo + dl * (w.end - w.S) + (int)((uint32_t)((c + turn_lo) * dl) >> 1);
-        const int hi = dh <= 0 ? early_hi(c) : sum_hi + dh * (w.end + w.S) - (int)((uint32_t)((c + turn_hi) * dh) >> 1);
-        return (uint32_t)(hi - lo + c);
+        if constexpr (kDense) return dense.start(c);
+        return (uint32_t)c * stride;
     }
     template <typename H>
     __device__ __forceinline__ typename H::T get(const typename H::T* hist, int c, int j) const {
@@ -376,24 +348,30 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
         bool run = status == kRun;
         Window win{0, 0, 0, 0, S};
         if (run) {
-            // the window: 2 O + k + (k - kend) <= S beyond both 0 and kend, and likewise on the other side
-            int right = min(max(max(0, kend), (S - 2 * O + kend) >> 1), m);
-            int left = min(max(max(0, -kend), (S - 2 * O - kend) >> 1), n);
-            if (a.band >= 0) { right = min(right, a.band); left = min(left, a.band); }
-            win = Window{-left - 1, left + right + 1, left + 1, kend + left + 1, S};
+            win = window_of(n, m, S, O, a.band);
         }
-        const int wide = P == 1 ? win.last : __reduce_max_sync(kFull, win.last);   // 0: no pair to run
+        int wide = P == 1 ? win.last : __reduce_max_sync(kFull, win.last);   // 0: no pair to run
         // entry (s, t-th of its row) of the history at [s * stride + t * P]
         const uint32_t stride = ((uint32_t)wide * P + 31u) & ~31u;
         // what rows 0 .. S take, from the pairs' own limits and windows: the arena holds more rounds than of the worst case
         size_t need = 0;
         if constexpr (kDense) {
-            if (run) need = (size_t)RowMap<P, true>(win, O, 0).start(S + 1) * sizeof(E);
+            if (run) need = (size_t)DenseRows(win, O).start(S + 1) * sizeof(E);
         } else {
             const int rows = P == 1 ? S : __reduce_max_sync(kFull, run ? S : 0);
             if (wide) need = (size_t)(rows + 1) * stride * sizeof(E);
         }
-        if (round == kRounds || rounds_bytes - used < need) finish();
+        // the host sizes rings and arenas for every pair of a launch; one that it misjudged all the same gets no result
+        // instead of memory that is not its own
+        if ((uint32_t)wide + 2 > W) need = ~(size_t)0;
+        if (round == kRounds || rounds_bytes - used < need) {
+            finish();
+            if (need > rounds_bytes) {
+                if (run) status = kCap;
+                run = false;
+                wide = 0;
+            }
+        }
         int final_s = -1, s = 0;
         uint32_t entries = 0;   // of the round's history
         if (wide) {
@@ -532,7 +510,7 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
             st_windows += windows;
             entries = kDense ? filled : (uint32_t)s * stride;
         }
-        if (gl == 0 && (status == kRejected || status == kBad)) emit_failed(a, pi, status);
+        if (gl == 0 && (status == kRejected || status == kBad || status == kCap)) emit_failed(a, pi, status);
         // the pair's tracer takes what it needs (P == 1: every lane has it)
         if constexpr (P == 1) {
             if (lane == tracer(round))
@@ -631,10 +609,8 @@ size_t ring_warp_bytes(const WfaPlan& p, int G, uint32_t max_length) {
     size_t entries = 0;
     if (P > 1 || entry_form(max_length) == kWhole) {
         entries = ring_rows(p) * ((W * P + 31) / 32 * 32);
-    } else {   // row s: at most s - O diagonals from 0, at most S - s from the end diagonal, the window
-        const int64_t O = p.oe - p.e, S = (int64_t)ring_rows(p) - 1;
-        for (int64_t s = 0; s <= S; ++s)
-            entries += (size_t)std::min(std::min(2 * std::max<int64_t>(s - O, 0), 2 * (S - s)) + 1, (int64_t)W - 2);
+    } else {
+        entries = dense_entries((int64_t)ring_rows(p) - 1, p.oe - p.e, (int64_t)W);
     }
     return align_up(32 * p.runs_bytes + entries * entry_bytes(max_length) + 512, 256);
 }
