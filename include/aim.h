@@ -152,6 +152,7 @@ AIM_API int aim_pack_2bit(aim_ctx *ctx, const uint8_t *ascii, const uint64_t *ch
  *   algo, pen                  algorithm and costs (pen is a host pointer)
  *   max_edits                  edit threshold (see the threshold rule above); when max_edits_per_pair
  *                              is given it must bound every entry, and pairs above it are flagged BAD_PAIR
+ *                              (a negative entry takes max_edits itself in the wavefront algorithms and GenASM)
  *   max_edits_per_pair         optional (NULL): per-pair thresholds (int32, device)
  *   out_scores                 int32 per pair: optimum, or -1 if rejected / bad
  *   out_cigars, cigar_offsets  optional (both NULL: scores only).  Pair i's runs go to

@@ -58,6 +58,7 @@ struct GenasmArgs {
     uint8_t* scratch;
     size_t warp_bytes;              // stored columns of one warp
     int W, overlap;
+    int64_t max_limit;              // the call's largest threshold, which a pair without one of its own gets
     uint32_t nwarps;
     uint32_t* counter;
 };
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(128) genasm_kernel(GenasmArgs a) {
         ++st_pairs;
 
         const uint32_t n = a.P.read_len[pi], m = a.P.target_len[pi];
-        const int64_t k = pair_limit(a.L, pi);
+        const int64_t k = min((long long)pair_limit(a.L, pi), (long long)a.max_limit);
         if (pair_bad(a.P, pi) || n > a.P.max_length || m > a.P.max_length || k == -2) {
             write_header(a.O, pi, -1, AIM_F_BAD_PAIR, 0);
             continue;
@@ -305,6 +306,7 @@ cudaError_t launch_genasm(int W, int O, const PairsView& P, const LimitView& L, 
     GenasmArgs a;
     a.P = P; a.L = L; a.O = Ov;
     a.W = W; a.overlap = O;
+    a.max_limit = max_limit;
     a.counter = counter;
     a.warp_bytes = column_bytes(W, max_limit);
     // warp slots start on 256-byte boundaries so that every stored row is one aligned segment

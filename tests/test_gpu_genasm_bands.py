@@ -49,3 +49,19 @@ def test_windows_at_the_band_edge(oracle_lib, limit):
     dev = device_results(p, "genasm", oracle.UNIT, limit, aligner=a)
     a.close()
     assert_same(dev, want, what=f"genasm limit {limit}")
+
+
+def test_pairs_without_a_threshold_of_their_own(oracle_lib):
+    """A negative entry takes the call's largest threshold: at 14 the call's windows are kept as 32-bit bands alone."""
+    import paper_2208_01243_gb300 as aim
+    p = pairs()
+    per_pair = np.full(len(p), 14, np.int32)
+    per_pair[1::2] = -1
+    per_pair[::5] = 9
+    s, f, off, cig, lens = oracle.genasm_batch(p, np.where(per_pair < 0, 14, per_pair).astype(np.int64),
+                                               W=oracle.GENASM_W, O=oracle.GENASM_O)
+    want = s, f, [cig[off[i]:off[i] + lens[i]].astype(np.uint32) for i in range(len(p))]
+    a = aim.Aligner(0, 1 << 30)
+    dev = device_results(p, "genasm", oracle.UNIT, 14, per_pair=per_pair, aligner=a)
+    a.close()
+    assert_same(dev, want, what="genasm, negative entries")
