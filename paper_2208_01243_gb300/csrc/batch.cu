@@ -55,7 +55,6 @@
 // 4,000 pairs of 2-10 kbp 12.7 ms (31 ms; 18 ms; 23 ms before thin classes were merged); 1,000 pairs of 138-408 bp
 // 137 us (335 us; 312 us with the bound pass), 16,000 431 us (475 us; 548 us with a full batch's lanes).
 #include <algorithm>
-#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -67,13 +66,12 @@
 
 #include "aim_internal.cuh"
 #include "ranges.h"
+#include "ring_rows.h"
 
 namespace aim {
 namespace {
 
 constexpr int kBuckets = 32;
-constexpr int kWidthClasses = 4;
-constexpr int kWorkClasses = 8;
 constexpr int kCandidates[7] = {1, 2, 4, 8, 16, 32, 256};
 
 struct BucketParams {
@@ -102,14 +100,7 @@ __device__ __forceinline__ int bucket_of(const PairsView& P, const LimitView& L,
     const int64_t lim = pair_limit(L, i);
     int64_t S = lim < 0 ? 0 : lim / bp.g;
     if (S > bp.smax) S = bp.smax;
-    int64_t W = 2 * (S / bp.E) + 3;
-    W = min(W, n + m + 1);
-    if (bp.band >= 0) W = min(W, 2 * (int64_t)bp.band + 1);
-    const int64_t C = (S + 1) * W;
-    const int wc = W <= 64 ? 0 : W <= 128 ? 1 : W <= 256 ? 2 : 3;
-    int kc = (63 - __clzll((long long)(C + 1))) / 3;
-    if (kc > kWorkClasses - 1) kc = kWorkClasses - 1;
-    return bp.perm[(kWorkClasses - 1 - kc) * kWidthClasses + (kWidthClasses - 1 - wc)];
+    return bp.perm[work_bucket(n, m, S, bp.E, bp.band)];
 }
 
 // `capped` (optional): count and scatter only the pairs whose flag is AIM_F_STEP_CAP (the second pass's queues)
@@ -193,19 +184,10 @@ size_t bucket_pair_bytes(const WfaPlan& plan, int b, int G) {
     return wfa_pair_bytes_capped(plan, G, hist);
 }
 
-// the plan with what bucket b says of its pairs for wfa_ring.cu.  With C = (S + 1) W < 2^(3 (kc + 1)) and the window at
-// most W: W is at most 64 / 128 / 256 in the narrower width classes, and at most sqrt(2 C) + 1 in the widest (W <= 2 S + 3
-// there, so C >= W (W - 1) / 2); S + 1 is C over the class's least W.
+// the plan with what bucket b says of its pairs for wfa_ring.cu (E > 1 only narrows W for the same S; it needs E == 1)
 WfaPlan bucket_plan(const WfaPlan& plan, int b) {
-    const int kc = kWorkClasses - 1 - b / kWidthClasses;
-    const int wc = kWidthClasses - 1 - b % kWidthClasses;
     WfaPlan p = plan;
-    const int64_t cmax = ((int64_t)1 << (3 * (kc + 1))) - 2;
-    if (wc < kWidthClasses - 1) p.ring_diagonals = (int64_t)64 << wc;
-    else if (kc < kWorkClasses - 1) p.ring_diagonals = (int64_t)std::sqrt(2.0 * (double)cmax) + 2;
-    const int64_t wmin = wc == 0 ? 1 : ((int64_t)32 << wc) + 1;
-    // (E > 1 only narrows W for the same S; wfa_ring.cu needs E == 1)
-    if (kc < kWorkClasses - 1) p.ring_scores = std::max<int64_t>(cmax / wmin, 1);
+    bucket_limits(b, &p.ring_diagonals, &p.ring_scores);
     return p;
 }
 

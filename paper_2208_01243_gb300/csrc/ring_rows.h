@@ -1,7 +1,10 @@
-// Rows of a wavefront history: which positions row s of a pair covers, and where it starts when rows lie end to end.
-// Plain arithmetic for the host and the device (and for a test without either's compiler).
+// What wfa_ring.cu's memory is sized by: the window and rows of a pair, where a row starts when rows lie end to end, and
+// the work and width classes of batch plans with what each says of its pairs.  The kernel does not check its rows against
+// its memory again (checks in its loop over rounds cost 2 % by the registers they took), so this is plain arithmetic, kept
+// apart for a test that takes it through every kind of pair without a GPU.
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -13,8 +16,13 @@
 
 namespace aim {
 
+#ifdef __CUDACC__
+AIM_ROWS int least_of(int a, int b) { return min(a, b); }
+AIM_ROWS int most_of(int a, int b) { return max(a, b); }
+#else
 AIM_ROWS int least_of(int a, int b) { return a < b ? a : b; }
 AIM_ROWS int most_of(int a, int b) { return a > b ? a : b; }
+#endif
 
 // A pair's ring: diagonal k at position k - koff, position 1 the window's first diagonal and `last` its last one;
 // diagonal 0 at `zero`, the end diagonal at `end`.  Row s covers lo(s) .. hi(s).
@@ -24,14 +32,11 @@ struct Window {
     AIM_ROWS int hi(int s, int O) const { return least_of(least_of(zero + most_of(s - O, 0), end + (S - s)), last); }
 };
 
-// The window of a pair of n read and m target bases under scaled limit S (|m - n| no wider than the band or the limit
-// allows): 2 O + k + (k - kend) <= S beyond both 0 and kend = m - n, and likewise on the other side.
-AIM_ROWS Window window_of(int n, int m, int S, int O, int band) {
-    const int kend = m - n;
-    int right = least_of(most_of(most_of(0, kend), (S - 2 * O + kend) >> 1), m);
-    int left = least_of(most_of(most_of(0, -kend), (S - 2 * O - kend) >> 1), n);
-    if (band >= 0) { right = least_of(right, band); left = least_of(left, band); }
-    return Window{-left - 1, left + right + 1, left + 1, kend + left + 1, S};
+// Diagonals beyond 0 and `end` on the end's side that can lie on an alignment within scaled limit S, of `most` that the
+// matrix has: 2 O + k + (k - end) <= S, and no fewer than reach the end.
+AIM_ROWS int reach(int end, int most, int S, int O, int band) {
+    const int k = least_of(most_of(most_of(0, end), (S - 2 * O + end) >> 1), most);
+    return band >= 0 ? least_of(k, band) : k;
 }
 
 // Rows end to end: row c at the sum of hi(i) - lo(i) + 1 over i < c.  lo(i) is zero - min(g, zero - 1), g = max(i - O, 0),
@@ -74,6 +79,41 @@ inline size_t dense_entries(int64_t S, int64_t O, int64_t width) {
         n += (size_t)(w < width - 2 ? w : width - 2);
     }
     return n;
+}
+
+// Buckets of batch plans: with W = min(2 S / E + 3, n + m + 1, 2 band + 1) and C = (S + 1) W, bucket
+// (kWorkClasses - 1 - kc) kWidthClasses + kWidthClasses - 1 - wc holds the pairs of work class kc = log2(C + 1) / 3 and width
+// class wc, W <= 64, 128, 256 or more.
+constexpr int kWidthClasses = 4;
+constexpr int kWorkClasses = 8;
+
+AIM_ROWS int work_bucket(int64_t n, int64_t m, int64_t S, int E, int band) {
+    int64_t W = 2 * (S / E) + 3;
+    if (n + m + 1 < W) W = n + m + 1;
+    if (band >= 0 && 2 * (int64_t)band + 1 < W) W = 2 * (int64_t)band + 1;
+    const uint64_t C = (uint64_t)(S + 1) * (uint64_t)W;
+    const int wc = W <= 64 ? 0 : W <= 128 ? 1 : W <= 256 ? 2 : 3;
+#ifdef __CUDA_ARCH__
+    const int zeros = __clzll((long long)(C + 1));
+#else
+    const int zeros = __builtin_clzll(C + 1);
+#endif
+    const int kc = (63 - zeros) / 3;
+    return (kWorkClasses - 1 - least_of(kc, kWorkClasses - 1)) * kWidthClasses + (kWidthClasses - 1 - wc);
+}
+
+// No pair of bucket b has a window of more diagonals, or a larger scaled limit (0: the bucket says nothing).  With
+// C = (S + 1) W < 2^(3 (kc + 1)) - 1 and the window at most W: W is at most 64 / 128 / 256 in the narrower width classes, and
+// at most sqrt(2 C) + 1 in the widest (W <= 2 S + 3, so C >= W (W - 1) / 2); S + 1 is C over the class's least W.
+inline void bucket_limits(int b, int64_t* diagonals, int64_t* scores) {
+    const int kc = kWorkClasses - 1 - b / kWidthClasses;
+    const int wc = kWidthClasses - 1 - b % kWidthClasses;
+    const int64_t cmax = ((int64_t)1 << (3 * (kc + 1))) - 2;
+    *diagonals = *scores = 0;
+    if (wc < kWidthClasses - 1) *diagonals = (int64_t)64 << wc;
+    else if (kc < kWorkClasses - 1) *diagonals = (int64_t)std::sqrt(2.0 * (double)cmax) + 2;
+    const int64_t wmin = wc == 0 ? 1 : ((int64_t)32 << wc) + 1;
+    if (kc < kWorkClasses - 1) *scores = cmax / wmin > 1 ? cmax / wmin : 1;
 }
 
 }  // namespace aim

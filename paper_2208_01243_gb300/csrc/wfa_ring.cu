@@ -348,9 +348,10 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
         bool run = status == kRun;
         Window win{0, 0, 0, 0, S};
         if (run) {
-            win = window_of(n, m, S, O, a.band);
+            const int right = reach(kend, m, S, O, a.band), left = reach(-kend, n, S, O, a.band);
+            win = Window{-left - 1, left + right + 1, left + 1, kend + left + 1, S};
         }
-        int wide = P == 1 ? win.last : __reduce_max_sync(kFull, win.last);   // 0: no pair to run
+        const int wide = P == 1 ? win.last : __reduce_max_sync(kFull, win.last);   // 0: no pair to run
         // entry (s, t-th of its row) of the history at [s * stride + t * P]
         const uint32_t stride = ((uint32_t)wide * P + 31u) & ~31u;
         // what rows 0 .. S take, from the pairs' own limits and windows: the arena holds more rounds than of the worst case
@@ -361,17 +362,7 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
             const int rows = P == 1 ? S : __reduce_max_sync(kFull, run ? S : 0);
             if (wide) need = (size_t)(rows + 1) * stride * sizeof(E);
         }
-        // the host sizes rings and arenas for every pair of a launch; one that it misjudged all the same gets no result
-        // instead of memory that is not its own
-        if ((uint32_t)wide + 2 > W) need = ~(size_t)0;
-        if (round == kRounds || rounds_bytes - used < need) {
-            finish();
-            if (need > rounds_bytes) {
-                if (run) status = kCap;
-                run = false;
-                wide = 0;
-            }
-        }
+        if (round == kRounds || rounds_bytes - used < need) finish();
         int final_s = -1, s = 0;
         uint32_t entries = 0;   // of the round's history
         if (wide) {
@@ -510,7 +501,7 @@ __global__ void __launch_bounds__(kBlockThreads<G>) wfa_ring_kernel(RingArgs r) 
             st_windows += windows;
             entries = kDense ? filled : (uint32_t)s * stride;
         }
-        if (gl == 0 && (status == kRejected || status == kBad || status == kCap)) emit_failed(a, pi, status);
+        if (gl == 0 && (status == kRejected || status == kBad)) emit_failed(a, pi, status);
         // the pair's tracer takes what it needs (P == 1: every lane has it)
         if constexpr (P == 1) {
             if (lane == tracer(round))

@@ -1,6 +1,7 @@
 """Where the ring kernel's history rows lie (ring_rows.h), compiled for the CPU with overflow checks: row starts in closed
 form against the sum of the rows' widths, every pair's rows within the entries that the host reserves, and its window
-within the ring's width, over limits, bands, gap openings and end diagonals up to the largest that a launch can hold."""
+within the ring's width, over limits, bands, gap openings and end diagonals up to the largest that a launch can hold; the
+same by what a batch plan's bucket says of its pairs."""
 import os
 import subprocess
 
@@ -12,6 +13,10 @@ HARNESS = r"""
 #include <algorithm>
 #include "ring_rows.h"
 using namespace aim;
+static Window window_of(int n, int m, int kend, int S, int O, int band) {
+    const int right = reach(kend, m, S, O, band), left = reach(-kend, n, S, O, band);
+    return Window{-left - 1, left + right + 1, left + 1, kend + left + 1, S};
+}
 static int64_t width_of(int64_t smax, int64_t O, int64_t band, int64_t len) {   // the host's ring width
     int64_t w = smax - O + 1;
     if (band >= 0) w = std::min<int64_t>(w, 2 * band + 1);
@@ -20,7 +25,7 @@ static int64_t width_of(int64_t smax, int64_t O, int64_t band, int64_t len) {   
 static void check(int n, int m, int S, int O, int band, int64_t smax, int64_t len, size_t reserved) {
     const int kend = m - n;
     if ((band >= 0 && std::abs(kend) > band) || (kend && std::abs(kend) + O > S)) return;   // rejected at once
-    const Window w = window_of(n, m, S, O, band);
+    const Window w = window_of(n, m, kend, S, O, band);
     const DenseRows d(w, O);
     uint64_t sum = 0;
     const int step = S > 20000 ? 97 : 1;
@@ -34,6 +39,19 @@ static void check(int n, int m, int S, int O, int band, int64_t smax, int64_t le
     if (d.start(S + 1) != sum || sum >> 32 || sum > reserved || w.last + 2 > width_of(smax, O, band, len)) {
         std::printf("total %d %d %d %d %d: %llu %u of %zu, last %d\n", n, m, S, O, band, (unsigned long long)sum, d.start(S + 1),
                     reserved, w.last);
+        std::exit(1);
+    }
+}
+static void check_bucket(int n, int m, int S, int O, int band) {
+    const int kend = m - n;
+    if ((band >= 0 && std::abs(kend) > band) || (kend && std::abs(kend) + O > S)) return;
+    int64_t diagonals, scores;
+    const int b = work_bucket(n, m, S, 1, band);
+    bucket_limits(b, &diagonals, &scores);
+    const Window w = window_of(n, m, kend, S, O, band);
+    if (b < 0 || b >= kWorkClasses * kWidthClasses || (diagonals && w.last > diagonals) || (scores && S > scores)) {
+        std::printf("bucket %d of %d %d %d %d %d: %d of %lld, %d of %lld\n", b, n, m, S, O, band, w.last, (long long)diagonals, S,
+                    (long long)scores);
         std::exit(1);
     }
 }
@@ -52,6 +70,13 @@ int main() {
         const int len = 1 + rnd(2000), smax = rnd(3000), O = 1 + rnd(4), band = rnd(3) ? -1 : rnd(300);
         const size_t reserved = dense_entries(smax, O, width_of(smax, O, band, len));
         for (int j = 0; j < 8; ++j) check(rnd(len + 1), rnd(len + 1), rnd(smax + 1), O, band, smax, len, reserved);
+    }
+    for (int S = 0; S < 4000; ++S)   // across every line between classes
+        for (int len : {0, 1, 31, 32, 63, 64, 127, 128, 300, 3000})
+            for (int band : {-1, 0, 31, 32, 63, 64, 127, 128, 1000}) check_bucket(len, len + (S & 1), S, 1 + (S & 3), band);
+    for (int i = 0; i < 2000000; ++i) {
+        const int len = 1 + rnd(1 << (1 + rnd(15))), S = rnd(1 << (1 + rnd(18)));
+        check_bucket(rnd(len + 1), rnd(len + 1), S, 1 + rnd(4), rnd(2) ? -1 : rnd(1 << (1 + rnd(14))));
     }
     // the most a launch can hold: 32,000 bp without a threshold at mismatch 4, opening 4 (scaled), the widest band whose
     // ring fits 226 KB, and the widest limit without a band
