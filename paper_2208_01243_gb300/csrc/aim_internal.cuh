@@ -230,12 +230,13 @@ cudaError_t launch_wfa(const WfaPlan& plan, int group, const PairsView& P, const
                        int* warps_used);
 
 // the form of wfa_ring.cu (state in shared memory): whether the costs and lengths allow it, whether a launch with G
-// lanes per pair (1..32, 256: a block) fits shared memory and the scratch, the lanes suited to a batch (0: does not fit), one launch
+// lanes per pair (1..32, 256: a block) fits shared memory and the scratch, the lanes suited to a batch (0: does not fit;
+// alone: no other launch shares the scratch), one launch
 // over all pairs, or over the queue range bounds[0..1] of order
 bool ring_ok(const WfaPlan& p, uint32_t max_length);
 bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_bytes);
 size_t ring_warp_bytes(const WfaPlan& p, int G, uint32_t max_length);   // the least scratch of a warp (G = 256: a block)
-int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes);
+int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes, bool alone);
 cudaError_t launch_wfa_ring(const WfaPlan& plan, int G, const PairsView& P, const LimitView& L, const OutView& O,
                             const uint32_t* order, const uint32_t* bounds, uint8_t* scratch, size_t scratch_bytes,
                             uint32_t* counters, int num_sms, cudaStream_t st, int* warps_used);

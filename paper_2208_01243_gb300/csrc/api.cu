@@ -208,7 +208,7 @@ int align_packed(aim_ctx* ctx, const aim::PairsView& P, int algo, const aim_pena
             int ring = 0;
             if (aim::ring_ok(plan, P.max_length)) {
                 ring = ctx->wfa_group ? ctx->wfa_group
-                                      : aim::ring_group(plan, P.max_length, P.num_pairs, ctx->num_sms, scratch_bytes);
+                                      : aim::ring_group(plan, P.max_length, P.num_pairs, ctx->num_sms, scratch_bytes, true);
                 if (ctx->wfa_group && !aim::ring_fits(plan, ring, P.max_length, scratch_bytes)) ring = 0;
             }
             slot = time_begin(ctx, 1, st);

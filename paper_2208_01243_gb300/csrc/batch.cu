@@ -395,7 +395,7 @@ bool ring_layout(aim_batch* b) {
         const WfaPlan p = class_plan(b, k);
         // lanes by the rule of wfa_ring.cu for the class's pairs, and a bound pass with one pair per lane, or a warp per
         // pair for longer reads.  The rule looks at this batch, so cached choices, made for another, are not taken.
-        b->groups[k] = ring_group(p, b->max_length, b->class_pairs[k], b->ctx->num_sms, b->scratch_bytes);
+        b->groups[k] = ring_group(p, b->max_length, b->class_pairs[k], b->ctx->num_sms, b->scratch_bytes, false);
         const int mode = b->ctx->batch_bound;
         const int gb = mode == 1 ? kBoundDefaultGroup : p.smax < kBoundScore || b->few ? 0 : 1;
         b->bound1[k] = mode == 2 ? 0 : gb;

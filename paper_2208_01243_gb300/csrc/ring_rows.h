@@ -72,13 +72,11 @@ struct DenseRows {
 // entries of rows 0 .. S of any pair whose ring takes `width` positions, two of them padding: row s has at most s - O
 // diagonals on either side of 0 and S - s of the end diagonal, inside the window
 inline size_t dense_entries(int64_t S, int64_t O, int64_t width) {
-    size_t n = 0;
-    for (int64_t s = 0; s <= S; ++s) {
-        const int64_t up = 2 * (s > O ? s - O : 0), down = 2 * (S - s);
-        const int64_t w = (up < down ? up : down) + 1;
-        n += (size_t)(w < width - 2 ? w : width - 2);
-    }
-    return n;
+    const int64_t n = S - O, c = width - 3, a = c / 2;   // t = s - O rises to n; beside the middle one, 2 t or 2 (n - t), at most c
+    const auto half = [&](int64_t k) -> int64_t {        // sum of min(2 t, c) over t = 0 .. k
+        return k < 0 ? 0 : k <= a ? k * (k + 1) : a * (a + 1) + (k - a) * c;
+    };
+    return (size_t)(S + 1 + (n > 0 ? half(n / 2) + half(n - n / 2 - 1) : 0));
 }
 
 // Buckets of batch plans: with W = min(2 S / E + 3, n + m + 1, 2 band + 1) and C = (S + 1) W, bucket

@@ -539,15 +539,22 @@ void (*ring_kernel_for(int G))(RingArgs) {
 }
 
 // Lanes per pair: the fewest whose warps fit an SM at least 16 at a time (14 KB of shared memory each), since one lane
-// per pair wastes no lane on a row's end and shares a row's fixed work between the most pairs; more when the batch
-// would otherwise give the device less than 8 warps per SM, where the pair's own serial chain is what counts, up to the
-// lanes that the widest row gives work to (1,270 pairs, 2 edits: 18.0 us with 8 lanes, 18.1 with 32).
+// per pair wastes no lane on a row's end and shares a row's fixed work between the most pairs; more when the batch, or
+// the pairs that the scratch holds at once, would otherwise give the device less than 8 warps per SM, where the pair's
+// own serial chain is what counts, up to the lanes that the widest row gives work to (1,270 pairs, 2 edits: 18.0 us with 8
+// lanes, 18.1 with 32).
 // Measured, ms at 1 / 2 / 4 / 8 / 16 lanes: 1M x 150 bp, 6 edits (12 KB at 1 lane) 1.15 / 1.24 / 1.50 / 1.99 / 2.89;
 // 1M x 250 bp, 25 edits, band 25 (12 KB at 4) 13.4 / 10.7 / 9.8 / 10.4 / 12.8; 300k x 300 bp, 30 edits (11 KB at 8)
 // 12.6 / 12.2 / 5.7 / 4.6 / 4.9; 10k x 150 bp 0.080 / 0.067 / 0.060 / 0.064 / 0.073; 61 x 150 bp 0.072 / 0.056 /
 // 0.045 / 0.039 / 0.037.
 constexpr size_t kGoodSmem = 14u << 10;
+// Short of scratch, ms at 8 / 16 / 32 / 256 lanes: 10k x 1,000 bp, 50 edits, 16 MB 25.0 / 16.9 / 11.8 / 9.1, 256 MB 1.79 /
+// 1.25 / 0.92 / 1.54, 1 GB 0.71 / 0.59 / 0.57 / 1.40; at 32 / 256: 500 x 5 kbp, 250 edits, 64 MB 12.4 / 6.5, 1 GB 1.55 / 1.26;
+// 5,000 of them, 1 GB 8.9 / 8.3, 2 GB 6.4 / 7.7.  (wfa.cu: 500 x 5 kbp, 64 MB, 11.1; the rule had taken 32 there.)  A batch
+// plan's classes run side by side and share scratch and device, so there the scratch has no say.
 constexpr int kGoodWarps = 8;
+constexpr int kThinWarps = 4;              // a block per pair below so many warps an SM for want of scratch
+constexpr int64_t kBlockWidth = 128;       // narrower rows leave half a block without work
 constexpr size_t kBlockSmem = 20u << 10;   // a whole block per pair where a warp's state takes more
 constexpr size_t kMaxSmem = 226u << 10;   // dynamic shared memory a block may use (227 KB, less its static few bytes)
 constexpr size_t kPlainSmem = 47u << 10;  // ... and without asking for it (48 KB, less the same)
@@ -620,14 +627,20 @@ bool ring_fits(const WfaPlan& p, int G, uint32_t max_length, size_t scratch_byte
            units_of(G) * ring_warp_bytes(p, G, max_length) <= scratch_bytes;
 }
 
-int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes) {
+int ring_group(const WfaPlan& p, uint32_t max_length, uint32_t num_pairs, int num_sms, size_t scratch_bytes, bool alone) {
+    const int64_t widest = ring_width(p, max_length) - 2;
+    auto held = [&](int G) -> uint64_t {   // pairs that the scratch holds at once
+        return alone ? scratch_bytes / ring_warp_bytes(p, G, max_length) * pairs_of(G) : UINT32_MAX;
+    };
+    auto thin = [&](int G) {   // the pairs at work leave SMs short of warps
+        return std::min<uint64_t>(num_pairs, held(G)) * G < (uint64_t)num_sms * kGoodWarps * 32;
+    };
     int G = 1;
-    while (G < 32 && (ring_smem_per_warp(p, G, max_length) > kGoodSmem ||
-                      ((uint64_t)num_pairs * G < (uint64_t)num_sms * kGoodWarps * 32 &&
-                       G < ring_width(p, max_length) - 2)))
-        G *= 2;
+    while (G < 32 && (ring_smem_per_warp(p, G, max_length) > kGoodSmem || (G < widest && thin(G)))) G *= 2;
     while (G <= 32 && !ring_fits(p, G, max_length, scratch_bytes)) G *= 2;
-    if (G > 32 || (G == 32 && ring_smem_per_warp(p, G, max_length) > kBlockSmem)) G = 256;
+    if (G > 32 || (G == 32 && (ring_smem_per_warp(p, G, max_length) > kBlockSmem ||
+                              (widest > kBlockWidth && held(G) < (uint64_t)num_sms * kThinWarps))))
+        G = 256;
     return ring_fits(p, G, max_length, scratch_bytes) ? G : 0;
 }
 

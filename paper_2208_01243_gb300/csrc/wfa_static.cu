@@ -121,7 +121,7 @@ extern "C" int aim_wfa_align_static(const uint64_t* packed_reads, const uint64_t
     int sms = 0;
     const int rc = scratch_for_current_device((cudaStream_t)stream, &base, &sms);
     if (rc) return rc;
-    const int ring = aim::ring_ok(plan, max_length) ? aim::ring_group(plan, max_length, num_pairs, sms, capacity) : 0;
+    const int ring = aim::ring_ok(plan, max_length) ? aim::ring_group(plan, max_length, num_pairs, sms, capacity, true) : 0;
     if (ring) group = ring;
 
     cudaStream_t st = (cudaStream_t)stream;

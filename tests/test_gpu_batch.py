@@ -276,7 +276,7 @@ def test_cached_choices_for_longer_reads(oracle_lib, gen_lib):
     al.close()
 
 
-@pytest.mark.parametrize("scratch_mb,compact", [(48, 0), (48, 1), (160, 0), (160, 2)])
+@pytest.mark.parametrize("scratch_mb,compact", [(48, 0), (48, 1), (48, 2), (32, 0)])
 def test_plans_short_of_scratch(oracle_lib, gen_lib, scratch_mb, compact):
     """Scratch too small for classes of limits: buckets tuned by trials, each on the kernels that then run it.  The bound
     pass of these costs has one form, reported as 1 lane; results are the plain form's."""

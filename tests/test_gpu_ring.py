@@ -108,3 +108,14 @@ assert_same(dev, oracle_results(p, w.penalties, np.full(len(p), 8 * {edits}, np.
     env = dict(os.environ, PYTHONPATH=os.pathsep.join([here, os.path.dirname(here)]))
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("length,edits,count,megabytes", [(300, 30, 200, 2), (1000, 50, 120, 8), (1000, 50, 120, 64),
+                                                          (2500, 130, 30, 16), (2500, 130, 30, 400)])
+def test_ring_short_of_scratch(length, edits, count, megabytes):
+    """Workspaces that hold few pairs at once take more lanes for each, up to a block."""
+    w = gen.Workload("ring_scratch", 41, count, length - 40, length - 40, 0.7 * edits / length, 0.7 * edits / length, 0.1,
+                     "wfa", (0, 4, 6, 2), edits)
+    p = gen.generate(w)
+    dev = device_results(p, "wfa", w.penalties, edits, max_length=length, workspace=megabytes << 20)
+    assert_same(dev, oracle_results(p, w.penalties, np.full(len(p), 8 * edits, np.int64)), what=f"ring, {megabytes} MB")

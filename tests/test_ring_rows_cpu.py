@@ -55,7 +55,17 @@ static void check_bucket(int n, int m, int S, int O, int band) {
         std::exit(1);
     }
 }
+static size_t counted(int64_t S, int64_t O, int64_t width) {
+    size_t n = 0;
+    for (int64_t s = 0; s <= S; ++s)
+        n += (size_t)std::min(std::min(2 * std::max<int64_t>(s - O, 0), 2 * (S - s)) + 1, width - 2);
+    return n;
+}
 int main() {
+    for (int S = 0; S < 70; ++S)
+        for (int O = 1; O <= 4; ++O)
+            for (int width = 3; width < 90; ++width)
+                if (dense_entries(S, O, width) != counted(S, O, width)) { std::printf("entries %d %d %d\n", S, O, width); return 1; }
     for (int O = 1; O <= 4; ++O)
         for (int band : {-1, 0, 1, 3, 9})
             for (int n = 0; n <= 12; ++n)
