@@ -77,9 +77,11 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t s) {   // 0 f
     return r;
 }
 
-// parts: warps that share a batch (word lists of few, long sequences), each taking every parts-th turn; then `bad` is
-// zero at launch
-__global__ void __launch_bounds__(32 * kPackWarps, 6) pack_kernel(const uint8_t* __restrict__ ascii,
+// SHARED: `parts` warps share a batch (few sequences, which may be long), each taking every parts-th turn; batches are then
+// one sequence, the grid covers them at once, and the parts lie in one block of WARPS warps, which gather its flag.  (With
+// the flags zeroed by a memset before the launch 64 sequences of 150 bp took 6.2 us, 2.7 now.)
+template <int WARPS, bool SHARED>
+__global__ void __launch_bounds__(32 * WARPS, 48 / WARPS) pack_kernel(const uint8_t* __restrict__ ascii,
                                                                const uint64_t* __restrict__ char_off,
                                                                const uint32_t* __restrict__ len, uint32_t count,
                                                                uint32_t batch, uint32_t parts,
@@ -87,6 +89,8 @@ __global__ void __launch_bounds__(32 * kPackWarps, 6) pack_kernel(const uint8_t*
                                                                const uint64_t* __restrict__ word_off,
                                                                uint64_t word_stride, uint8_t* __restrict__ bad) {
     __shared__ uint4 s_first[17];   // [h]: ones in the first h bytes of a chunk
+    __shared__ uint32_t s_bad[WARPS];   // SHARED: whether a warp saw a byte that is none of the four
+    if (SHARED && threadIdx.x < WARPS) s_bad[threadIdx.x] = 0;
     if (threadIdx.x < 17) {
         auto word = [&](int q) -> uint32_t {
             const int h = (int)threadIdx.x - 4 * q;
@@ -97,7 +101,7 @@ __global__ void __launch_bounds__(32 * kPackWarps, 6) pack_kernel(const uint8_t*
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-    const uint64_t nbatches = (count + batch - 1) / batch;
+    const uint64_t nbatches = ((uint64_t)count + batch - 1) / batch;
     for (uint64_t work = warp; work < nbatches * parts; work += nwarps) {
         const uint32_t first = (uint32_t)(work / parts) * batch, part = (uint32_t)(work % parts);
         // this lane's sequence
@@ -112,10 +116,8 @@ __global__ void __launch_bounds__(32 * kPackWarps, 6) pack_kernel(const uint8_t*
             const uint32_t nw = (L + 31) >> 5;
             const bool fits = word_off || nw <= word_stride;   // longer than the fixed slot: flag, write nothing
             items = fits && nw ? nw + 1 : 0;
-            if (bad && part == 0) {
-                if (!fits) bad[i] = 1;
-                else if (parts == 1) bad[i] = 0;
-            }
+            if (SHARED && !fits) s_bad[threadIdx.x >> 5] = 1;
+            if (!SHARED && bad) bad[i] = !fits;
         }
         __syncwarp();   // bad[] starts at 0 before any lane sets it
         // all sequences at once, or one by one where the list's length might leave 32 bits (over 2 G bases in one)
@@ -166,8 +168,20 @@ __global__ void __launch_bounds__(32 * kPackWarps, 6) pack_kernel(const uint8_t*
                                         ~shr_clamp(~0u, 2 * max(nb, 16u) - 32);
                     packed[sto + w] = ((uint64_t)hi << 32) | lo;
                 }
-                if (bad && b) bad[first + s] = 1;
+                if (bad && b) {
+                    if (SHARED) s_bad[threadIdx.x >> 5] = 1;
+                    else bad[first + s] = 1;
+                }
             }
+        }
+    }
+    if (SHARED && bad) {
+        __syncthreads();
+        const uint64_t i = (uint64_t)blockIdx.x * (WARPS / parts) + threadIdx.x;   // parts divides a block's warps
+        if (threadIdx.x < WARPS / parts && i < count) {
+            uint32_t any = 0;
+            for (uint32_t k = 0; k < parts; ++k) any |= s_bad[threadIdx.x * parts + k];
+            bad[i] = any != 0;
         }
     }
 }
@@ -184,17 +198,16 @@ cudaError_t launch_pack(const uint8_t* ascii, const uint64_t* char_off, const ui
     // batches of up to 32 sequences, smaller (and then shared by several warps) while that leaves SMs without 16 warps
     const uint32_t want = (uint32_t)sms * 16;
     uint32_t batch = 32, parts = 1;
-    while (batch > 1 && (count + batch - 1) / batch < want) batch /= 2;
-    const uint32_t batches = (count + batch - 1) / batch;
-    while (parts < 16 && batches * parts < want / 2) parts *= 2;
-    if (bad && parts > 1) {
-        const cudaError_t e = cudaMemsetAsync(bad, 0, count, st);
-        if (e != cudaSuccess) return e;
-    }
-    const uint64_t warps = (uint64_t)batches * parts;
-    const uint64_t blocks = std::min<uint64_t>((warps + kPackWarps - 1) / kPackWarps, (uint64_t)sms * 32);
-    pack_kernel<<<(unsigned)blocks, 32 * kPackWarps, 0, st>>>(ascii, char_off, len, count, batch, parts, packed, word_off,
-                                                             word_stride, bad);
+    while (batch > 1 && ((uint64_t)count + batch - 1) / batch < want) batch /= 2;
+    const uint64_t batches = ((uint64_t)count + batch - 1) / batch;
+    // (no more than a slot's words keep busy, where slots are fixed: 61 pairs of 150 bp 28.7 us a call, 31.8 with 16)
+    while (parts < 16 && batches * parts < want / 2 && (word_off || 31ull * parts <= word_stride)) parts *= 2;
+    const uint64_t warps = batches * parts;
+    const int per_block = std::max(kPackWarps, (int)parts);
+    const uint64_t blocks = std::min<uint64_t>((warps + per_block - 1) / per_block, (uint64_t)sms * 32);
+    auto kernel = parts == 1 ? pack_kernel<kPackWarps, false> : parts <= kPackWarps ? pack_kernel<kPackWarps, true> : pack_kernel<16, true>;
+    kernel<<<(unsigned)blocks, 32 * per_block, 0, st>>>(ascii, char_off, len, count, batch, parts, packed, word_off,
+                                                        word_stride, bad);
     return cudaGetLastError();
 }
 
