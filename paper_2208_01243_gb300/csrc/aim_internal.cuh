@@ -117,17 +117,21 @@ struct DpPlan {
     size_t slot_bytes;   // per-warp scratch
 };
 DpPlan plan_dp(bool unit, int band, uint32_t max_length, int64_t max_limit_hint);
+size_t dp_slot_bytes(const DpPlan& plan, const Costs& c, uint32_t max_length, int64_t max_limit);   // one pair's scratch
+// evenness (see dp_lane_evenness): if not 0, the launch aligns the batch only if its reads are less even than that
 cudaError_t launch_dp(const DpPlan& plan, const Costs& c, const PairsView& P, const LimitView& L, const OutView& O,
-                      int64_t max_limit, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter,
+                      int64_t max_limit, uint32_t evenness, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter,
                       int num_sms, cudaStream_t st, int* warps_used);
 
-// the same alignments with one pair per lane (dp_lane.cu): whether costs, band, lengths and scratch allow it and the batch
-// is large enough; the launch
-bool dp_lane_ok(bool unit, int band, const Costs& c, uint32_t max_length, int64_t max_limit, uint32_t num_pairs,
-                int num_sms, size_t scratch_bytes);
+// the same alignments with one pair per lane (dp_lane.cu): how even the batch's reads have to be for that to be the faster
+// form, as their mean length in 256ths of the longest one's (0: it is whatever the lengths; kNeverEven: it is not, or costs,
+// band, lengths or scratch don't allow it); the launch, which aligns the batch only if its reads are that even
+constexpr uint32_t kNeverEven = 257;
+uint32_t dp_lane_evenness(const DpPlan& plan, const Costs& c, uint32_t max_length, int64_t max_limit, uint32_t num_pairs,
+                          int num_sms, size_t scratch_bytes);
 cudaError_t launch_dp_lane(bool unit, int band, const Costs& c, const PairsView& P, const LimitView& L, const OutView& O,
-                           int64_t max_limit, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms,
-                           cudaStream_t st, int* warps_used);
+                           int64_t max_limit, uint32_t evenness, uint8_t* scratch, size_t scratch_bytes,
+                           uint32_t* counter, int num_sms, cudaStream_t st, int* warps_used);
 
 constexpr int kMaxBuckets = 32;
 // wavefront history: one entry per (score, diagonal) holds M~, I~, D~ and a spare slot as four int16, so an entry
@@ -330,6 +334,27 @@ __device__ __forceinline__ void warp_stat_add(unsigned long long* stats, int slo
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     if (stats && lane == 0 && v) atomicAdd(stats + slot, v);
+}
+
+}  // namespace aim
+
+namespace aim {
+
+// Whole warp: whether the mean length of the batch's reads is at least evenness / 256 of the longest one's, by a sample of
+// 128 spread over the batch.  Every warp of every kernel that asks looks at the same reads, so two launches, of which the
+// first aligns even batches and the second the others, need nothing from the host, which does not see device lengths.
+__device__ __forceinline__ bool reads_even(const PairsView& P, uint32_t evenness) {
+    uint32_t sum = 0, most = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i) {
+        const uint32_t at = (uint32_t)((uint64_t)(i * 32 + (threadIdx.x & 31)) * P.num_pairs / 128);
+        const uint32_t n = min(__ldg(P.read_len + at), P.max_length);
+        sum += n;
+        most = max(most, n);
+    }
+    sum = __reduce_add_sync(kFull, sum);
+    most = __reduce_max_sync(kFull, most);
+    return (uint64_t)sum * 256 >= (uint64_t)most * 128 * evenness;
 }
 
 }  // namespace aim

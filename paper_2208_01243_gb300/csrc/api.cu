@@ -229,16 +229,17 @@ int align_packed(aim_ctx* ctx, const aim::PairsView& P, int algo, const aim_pena
         }
         if (b > aim::kMaxDpBand) return AIM_ERR_UNSUPPORTED;
         const aim::DpPlan plan = aim::plan_dp(unit, (int)b, P.max_length, r.max_limit);
-        const bool lanes = aim::dp_lane_ok(unit, (int)b, r.costs, P.max_length, r.max_limit, P.num_pairs,
-                                           ctx->num_sms, scratch_bytes);
+        const uint32_t even = aim::dp_lane_evenness(plan, r.costs, P.max_length, r.max_limit, P.num_pairs, ctx->num_sms,
+                                                    scratch_bytes);
         if (plan.slot_bytes > scratch_bytes) return AIM_ERR_NOMEM;
         slot = time_begin(ctx, 1, st);
-        if (lanes)
-            err = aim::launch_dp_lane(unit, (int)b, r.costs, P, r.lim, O, r.max_limit, scratch, scratch_bytes, counter,
-                                      ctx->num_sms, st, &warps);
-        else
-            err = aim::launch_dp(plan, r.costs, P, r.lim, O, r.max_limit, scratch, scratch_bytes, counter,
-                                 ctx->num_sms, st, &warps);
+        // between the two, both are launched, and the lengths say which of them aligns the batch (the other ends at once)
+        if (even < aim::kNeverEven)
+            err = aim::launch_dp_lane(unit, (int)b, r.costs, P, r.lim, O, r.max_limit, even, scratch, scratch_bytes,
+                                      counter, ctx->num_sms, st, &warps);
+        if (err == cudaSuccess && even && (even >= aim::kNeverEven || warps > 0))
+            err = aim::launch_dp(plan, r.costs, P, r.lim, O, r.max_limit, even < aim::kNeverEven ? even : 0, scratch,
+                                 scratch_bytes, counter, ctx->num_sms, st, &warps);
     }
     time_end(ctx, 1, slot, st);
     if (err != cudaSuccess) return cuda_status(err);

@@ -59,6 +59,7 @@ struct DpArgs {
     uint32_t defer;          // slots per warp: finished pairs wait in them and are traced back side by side
     uint32_t runs_cap;
     uint32_t nwarps;
+    uint32_t evenness;       // not 0: batches of reads at least this even are dp_lane.cu's
     uint32_t* counter;
 };
 
@@ -171,6 +172,7 @@ __device__ __forceinline__ void dp_finish(const DpArgs& a, uint8_t* warp_slots, 
 template <bool UNIT, int R, int SUB, bool CAP>
 __global__ void __launch_bounds__(256, R == 1 ? 4 : R == 2 ? 2 : 1) dp_kernel(DpArgs a) {
     static_assert(SUB == 1 || R == 1, "several pairs per warp only for one lane block");
+    if (a.evenness && reads_even(a.P, a.evenness)) return;
     using TB = typename std::conditional<UNIT, uint8_t, uint16_t>::type;
     constexpr int GS = 32 / SUB;    // lanes per pair (a segment of the warp)
     constexpr int RW = GS * R;      // trace entries per anti-diagonal row
@@ -537,24 +539,33 @@ DpPlan plan_dp(bool unit, int band, uint32_t max_length, int64_t max_limit) {
     return p;
 }
 
+// staged runs: every edit run costs at least min(x, o+e), and runs alternate with match runs
+static int64_t runs_of(const DpPlan& plan, const Costs& c, uint32_t max_length, int64_t max_limit) {
+    const int64_t minc = plan.unit ? 1 : (c.x < c.o + c.e ? c.x : c.o + c.e);
+    int64_t cap = 2 * (int64_t)max_length + 1;
+    if (max_limit < kUnbounded && minc > 0) {
+        const int64_t by_cost = 2 * (max_limit / minc) + 1;
+        if (by_cost < cap) cap = by_cost;
+    }
+    return cap;
+}
+
+size_t dp_slot_bytes(const DpPlan& plan, const Costs& c, uint32_t max_length, int64_t max_limit) {
+    return align_up(plan.slot_bytes + (size_t)runs_of(plan, c, max_length, max_limit) * 4, 128);
+}
+
 cudaError_t launch_dp(const DpPlan& plan, const Costs& c, const PairsView& P, const LimitView& L, const OutView& O,
-                      int64_t max_limit, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms,
-                      cudaStream_t st, int* warps_used) {
+                      int64_t max_limit, uint32_t evenness, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter,
+                      int num_sms, cudaStream_t st, int* warps_used) {
     *warps_used = 0;
     if (P.num_pairs == 0) return cudaSuccess;
     DpArgs a;
     a.c = c; a.P = P; a.L = L; a.O = O; a.band = plan.band;
     a.scratch = scratch; a.counter = counter; a.nwarps = 0;
-    // staged runs: every edit run costs at least min(x, o+e), and runs alternate with match runs
-    const int64_t minc = plan.unit ? 1 : (c.x < c.o + c.e ? c.x : c.o + c.e);
-    int64_t cap = 2 * (int64_t)P.max_length + 1;
-    if (max_limit < kUnbounded && minc > 0) {
-        const int64_t by_cost = 2 * (max_limit / minc) + 1;
-        if (by_cost < cap) cap = by_cost;
-    }
-    a.runs_cap = (uint32_t)cap;
+    a.evenness = evenness;
+    a.runs_cap = (uint32_t)runs_of(plan, c, P.max_length, max_limit);
     a.trace_bytes = plan.slot_bytes;
-    a.slot_bytes = align_up(plan.slot_bytes + (size_t)cap * 4, 128);
+    a.slot_bytes = dp_slot_bytes(plan, c, P.max_length, max_limit);
     // values need no cap when kInf + (anti-diagonals + 1) * (largest cost) fits int32
     const int64_t maxc = plan.unit ? 1 : std::max<int64_t>(std::max<int64_t>(c.x, (int64_t)c.o + c.e), c.e);
     const bool need_cap = (2 * (int64_t)P.max_length + 2) * maxc >= (int64_t)INT32_MAX - kInf - maxc;

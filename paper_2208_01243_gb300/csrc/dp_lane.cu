@@ -1,5 +1,5 @@
 // Banded global DP with one pair per lane: NW edit distance (unit costs) and gap-affine Gotoh, the same alignments as
-// dp_banded.cu's, for bands and costs that fit (dp_lane_ok).
+// dp_banded.cu's, for bands and costs that fit (dp_lane_evenness).
 //
 // Values carry their traceback.  The canonical traceback takes, in each cell, the first of X < I < D < M among the
 // states that meet the cost the rest must have.  Values are 4 * cost + rank, where the rank says which op the state
@@ -56,6 +56,7 @@ struct LaneArgs {
     size_t warp_bytes, trace_bytes;   // a warp's scratch: trace rows, then 32 lanes' runs
     uint32_t runs_cap;
     uint32_t nwarps;
+    uint32_t evenness;        // reads of an EVEN instance
     uint32_t* counter;
 };
 
@@ -64,8 +65,10 @@ extern __shared__ __align__(16) uint8_t s_lane[];
 // the two low bits of v pushed into the top of a trace word
 __device__ __forceinline__ void push(uint32_t& word, int v) { word = __funnelshift_r(word, (uint32_t)v, 2); }
 
-template <bool UNIT>
+// EVEN: only batches of reads at least a.evenness even (an instance of its own: the test alone cost unit costs 12 %)
+template <bool UNIT, bool EVEN>
 __global__ void __launch_bounds__(32 * kLaneWarps) dp_lane_kernel(LaneArgs a) {
+    if (EVEN && !reads_even(a.P, a.evenness)) return;
     const int lane = (int)(threadIdx.x & 31);
     const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (gwarp >= a.nwarps) return;
@@ -304,26 +307,53 @@ constexpr size_t kLaneSmem = 226u << 10;   // dynamic shared memory a block may 
 
 }  // namespace
 
-// From 27 pairs per SM on: a warp takes as long for one pair as for 32, and below that dp_banded.cu's warp per pair
-// ends sooner.  The two meet (ms, dp_banded.cu / here) at 250 bp, band 25: 2,500 pairs 0.37 / 0.46, 5,000 0.53 / 0.46;
-// 250 bp, band 60: 2,500 0.66 / 0.80, 5,000 0.94 / 0.82; 100 bp, band 8: 2,500 0.148 / 0.139; edit distance 100 bp,
-// band 10: 2,500 0.100 / 0.101, 5,000 0.139 / 0.101; 250 bp, band 25: 2,500 0.27 / 0.29, 5,000 0.37 / 0.29.
-bool dp_lane_ok(bool unit, int band, const Costs& c, uint32_t max_length, int64_t max_limit, uint32_t num_pairs,
-                int num_sms, size_t scratch_bytes) {
-    if (num_pairs < 27u * (uint32_t)num_sms) return false;
+// Where this form is the faster one.  A warp takes as long for one pair as for 32, rho times a lone pair's warp in
+// dp_banded.cu, and runs in waves of the pairs that shared memory and scratch hold.  dp_banded.cu's time grows with the
+// pairs' own lengths: of y = pairs * mean / longest, as many as the scratch holds are at work, and sat of them on every SM
+// double the time of each.  In a lone pair's times:
+//   here rho * waves,   there max(1, y / held) (1 + min(y, held) / (sat * SMs)).
+// The two are equal at the share of the mean in the longest that this returns; the launches look at the lengths.  Fitted to
+// (ms, dp_banded.cu / here, 1 GB unless stated) 250 bp, band 25: 2,500 pairs 0.37 / 0.46, 5,000 0.53 / 0.46; 1,000 bp, 8,000
+// pairs, 64 MB: band 25 13.8 / 10.3, band 60 40.3 / 36.6, band 120 121 / 128, at 256 MB 33.5 / 36.1, 1 GB 15.1 / 10.6; 3,000
+// bp, band 25, 8,000 pairs 12.1 / 9.1; 50-1,000 bp, band 25: 4,200 pairs 1.19 / 1.54, 8,000 1.45 / 1.58, 10,000 1.59 / 1.56;
+// band 60: 4,200 1.73 / 2.94, 16,000 3.82 / 2.98; band 120: 8,000 5.19 / 5.22, 16,000 8.97 / 10.1; edit distance, 100 bp, band
+// 10: 2,500 0.100 / 0.101, 5,000 0.139 / 0.101; 50-1,000 bp, band 12: 4,200 0.567 / 0.587, 6,000 0.706 / 0.594.
+// Below 27 pairs an SM it has not been measured throughout.  A share below a quarter counts as none, such batches being
+// rare, and so does any below 1 with unit costs, where little is lost, or where the second launch's 4 us would show (250
+// rows of band 25 take 0.41 ms).
+uint32_t dp_lane_evenness(const DpPlan& plan, const Costs& c, uint32_t max_length, int64_t max_limit, uint32_t num_pairs,
+                          int num_sms, size_t scratch_bytes) {
+    const bool unit = plan.unit;
+    const int band = plan.band;
+    if (num_pairs < 27u * (uint32_t)num_sms) return kNeverEven;
     const int64_t maxc = unit ? 1 : std::max<int64_t>(c.x, (int64_t)c.o + c.e);
-    return (2 * (int64_t)max_length + 2 * (int64_t)band + 8) * maxc < (int64_t)1 << 26 &&
-           kLaneWarps * lane_smem(unit, band, max_length) <= kLaneSmem &&
-           kLaneWarps * lane_warp(unit, band, c, max_length, max_limit) <= scratch_bytes;
+    const size_t smem = kLaneWarps * lane_smem(unit, band, max_length), warp = lane_warp(unit, band, c, max_length, max_limit);
+    if ((2 * (int64_t)max_length + 2 * (int64_t)band + 8) * maxc >= (int64_t)1 << 26 || smem > kLaneSmem ||
+        kLaneWarps * warp > scratch_bytes)
+        return kNeverEven;
+    const size_t held = scratch_bytes / dp_slot_bytes(plan, c, max_length, max_limit);   // pairs at once in dp_banded.cu
+    if (held < (size_t)plan.pairs_per_warp) return 0;   // it has room for none
+    const int r = plan.blocks == 1 ? 0 : plan.blocks == 2 ? 1 : 2;
+    const double rho = unit ? (r == 0 ? 1.7 : r == 1 ? 2.2 : 2.7) : (r == 0 ? 2.0 : r == 1 ? 2.3 : 3.0);
+    const double sat = (unit ? 13.0 : r == 0 ? 27.0 : r == 1 ? 19.0 : 10.0) * num_sms;
+    const size_t warps = std::min((size_t)num_sms * std::min<size_t>(kLaneSmem / smem * kLaneWarps, 16), scratch_bytes / warp);
+    const size_t waves = ((size_t)num_pairs + 32 * warps - 1) / (32 * warps);
+    const double here = rho * (double)waves;
+    double y = (here - 1.0) * sat;
+    if (y > (double)held) y = here / (1.0 / (double)held + 1.0 / sat);
+    const double share = y / (double)num_pairs;
+    if (share >= 1.0) return kNeverEven;
+    return unit || share <= 0.25 || (uint64_t)max_length * (2 * band + 1) < 250 * 51 ? 0 : (uint32_t)(share * 256.0);
 }
 
 cudaError_t launch_dp_lane(bool unit, int band, const Costs& c, const PairsView& P, const LimitView& L, const OutView& O,
-                           int64_t max_limit, uint8_t* scratch, size_t scratch_bytes, uint32_t* counter, int num_sms,
-                           cudaStream_t st, int* warps_used) {
+                           int64_t max_limit, uint32_t evenness, uint8_t* scratch, size_t scratch_bytes,
+                           uint32_t* counter, int num_sms, cudaStream_t st, int* warps_used) {
     *warps_used = 0;
     if (P.num_pairs == 0) return cudaSuccess;
     LaneArgs a{};
     a.c = c; a.P = P; a.L = L; a.O = O;
+    a.evenness = evenness;
     a.band = band;
     a.groups = groups_of(band);
     a.row_words = row_words_of(unit, band);
@@ -335,7 +365,8 @@ cudaError_t launch_dp_lane(bool unit, int band, const Costs& c, const PairsView&
     a.warp_bytes = lane_warp(unit, band, c, P.max_length, max_limit);
     a.runs_cap = lane_runs(unit, c, P.max_length, max_limit);
     a.counter = counter;
-    void (*kernel)(LaneArgs) = unit ? dp_lane_kernel<true> : dp_lane_kernel<false>;
+    void (*kernel)(LaneArgs) = unit ? dp_lane_kernel<true, false>
+                               : evenness ? dp_lane_kernel<false, true> : dp_lane_kernel<false, false>;
     const size_t smem = (size_t)kLaneWarps * a.smem_warp;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLaneSmem);
     if (e != cudaSuccess) return e;

@@ -61,3 +61,29 @@ def test_lane_dp_leaves_large_costs_to_the_other_kernel(aligner):
     k = 8000 // len(p) + 1
     dev = device_results(gen.concat([p] * k), "gotoh", pen, -1, band=12, max_score=1 << 24, aligner=aligner)
     assert_same(dev, oracle_results(p, pen, lim, band=12), what="large costs")
+
+
+@pytest.mark.parametrize("band", [0, 1, 3, 8, 15, 16, 25, 31, 32, 63, 64, 127])
+@pytest.mark.parametrize("algo,penalties", [("edit", (0, 1, 0, 1)), ("gotoh", (0, 4, 6, 2)), ("gotoh", (0, 3, 0, 2))])
+@pytest.mark.parametrize("long_share", [0.8, 0.05])
+def test_lane_dp_by_evenness(aligner, algo, penalties, band, long_share):
+    """The form is chosen by how even the reads are: batches of mostly long reads go to a pair per lane, whatever short,
+    empty and one-base pairs are among them, and mostly short ones with a few long reads to a warp per pair."""
+    rng = np.random.default_rng(band)
+    short = gen.concat([_mixed([1, 2, 15, 16, 17, 31, 33, 64], 300 + band),
+                        gen.from_strings([b"", b"ACGT", b"", b"A" * 70], [b"", b"", b"ACG", b"A" * 75])])
+    long = _mixed([150, 159, 160, 161, 190], 500 + band)
+    k_long = max(int(long_share / (1 - long_share) * len(short) / len(long) * 4), 1)
+    p = gen.concat([short] * 4 + [long] * k_long)
+    order = rng.permutation(len(p))
+    p = gen.from_strings([p.read(i) for i in order], [p.target(i) for i in order])
+    most = 40
+    per_pair = rng.integers(0, most + 1, len(p)).astype(np.int32)
+    per_pair[::2] = most
+    x, o, e = penalties[1:]
+    lim = per_pair.astype(np.int64) * (1 if algo == "edit" else max(x, o + e))
+    k = 6000 // len(p) + 1
+    dev = device_results(gen.concat([p] * k), algo, penalties, most, per_pair=np.tile(per_pair, k), band=band,
+                         aligner=aligner)
+    assert_same(dev, oracle_results(p, penalties, lim, band=band), what=f"{algo} {penalties}, band {band}")
+    assert np.array_equal(dev[0], np.tile(dev[0][:len(p)], k)) and np.array_equal(dev[3], np.tile(dev[3][:len(p)], k))
