@@ -175,15 +175,17 @@ int align_packed(aim_ctx* ctx, const aim::PairsView& P, int algo, const aim_pena
             int ga = aim::adapt_group(plan, P.max_length, P.num_pairs, ctx->num_sms, scratch_bytes);
             if (ga && ctx->wfa_group)
                 ga = aim::adapt_group_fits(plan, ctx->wfa_group, P.max_length, scratch_bytes) ? ctx->wfa_group : 0;
-            // That form loses on narrow scores (1,000 bp, 2 %, smax 100: 4.93 ms against 4.57; 2,000 bp, 2 %, smax 200: 2.93
-            // against 3.27; 1,000 bp, 5 %: 13.5 against 14.2), and beyond 2,048 bp wherever the scratch holds the compact
-            // pass at three quarters of 24 warps an SM (5 kbp, 5 %: 12.1 against 30.6 ms on 2 GiB, 8.2 on 32 GiB; 10 kbp,
-            // 5 %: 12.9 against 17.9 on 8 GiB, 9.5 on 32)
+            // That form loses on narrow scores (1,000 bp, 2 %, smax 100: 4.93 ms against 4.57), and where the scratch holds the
+            // compact pass at three quarters of 24 warps an SM: beyond 2,048 bp always (5 kbp, 5 %: 12.1 against 30.6 ms on 2
+            // GiB, 8.2 on 32 GiB; 10 kbp, 5 %: 12.9 against 17.9 on 8 GiB, 9.5 on 32), below unless pairs enough keep its groups
+            // busy to the end whatever their lengths (40k pairs of 200-1,000 bp, 5 %, 1.84 against 1.72 ms, 200k 7.36 against
+            // 7.49; 200k of 1,000 bp, 5 %, 13.9 against 14.6, 1-5 % 8.48 against 8.96, a tenth unrelated 18.5 against 18.0)
             if (ga && !ctx->wfa_group) {
                 const size_t per_warp = (size_t)std::max(1, 32 / g1);
                 const size_t full = std::min<size_t>((size_t)ctx->num_sms * 24, (P.num_pairs + per_warp - 1) / per_warp);
                 const size_t fit = scratch_bytes / aim::wfa_warp_bytes(g1, aim::wfa_pair_bytes(compact, g1));
-                if (plan.smax < 150 || (ga == 32 && 4 * fit >= 3 * full)) ga = 0;
+                const bool many = ga == 8 && P.num_pairs >= 768u * (uint32_t)ctx->num_sms;
+                if (plan.smax < 150 || (4 * fit >= 3 * full && !many)) ga = 0;
             }
             slot = time_begin(ctx, 1, st);
             err = ga ? aim::launch_wfa_adapt(plan, ga, P, r.lim, O, scratch, scratch_bytes, counter, ctx->num_sms, st,
