@@ -292,3 +292,51 @@ def test_plans_short_of_scratch(oracle_lib, gen_lib, scratch_mb, compact):
     for o in outs:
         assert np.array_equal(o[0], plain[0]) and np.array_equal(o[1], plain[1])
         assert all(np.array_equal(x, y) for x, y in zip(o[2], plain[2]))
+
+
+@pytest.mark.parametrize("autotune", [False, True])
+def test_replay_moves_pairs_between_classes(oracle_lib, gen_lib, autotune):
+    """A plan of classes of limits, made on short reads with few errors, replayed over longer and noisier ones and over other
+    thresholds, which put its pairs into classes that were empty or merged at planning, and back."""
+    import torch
+    import paper_2208_01243_gb300 as aim
+    slot, n = 700, 2500
+    rng = np.random.default_rng(8)
+
+    def content(lo, hi, r0, r1, unrelated, seed):
+        p = gen.generate(gen.Workload("classes", seed, n, lo, hi, r0, r1, unrelated, "wfa", AFF, 60))
+        buf = np.full(2 * n * slot, ord("A"), np.uint8)
+        for i in range(n):
+            r, t = p.read(i), p.target(i)
+            buf[2 * i * slot:2 * i * slot + len(r)] = np.frombuffer(r, np.uint8)
+            buf[(2 * i + 1) * slot:(2 * i + 1) * slot + len(t)] = np.frombuffer(t, np.uint8)
+        return p, buf
+    easy, mixed, hard = (content(80, 200, 0.0, 0.01, 0.0, 3), content(80, 600, 0.0, 0.1, 0.1, 4),
+                         content(500, 600, 0.08, 0.1, 0.2, 5))
+    steps = [(easy, np.full(n, 60)), (hard, np.full(n, 60)), (mixed, rng.integers(0, 61, n)), (easy, rng.integers(0, 8, n)),
+             (hard, np.where(rng.random(n) < 0.5, 60, 5)), (easy, np.full(n, 60))]
+    ro = np.arange(n, dtype=np.int64) * 2 * slot
+    buf, ro_d, to_d, rl, tl, pp = aim.upload(easy[1], ro, ro + slot, easy[0].read_len, easy[0].target_len,
+                                             np.full(n, 60, np.int32))
+    al = aim.Aligner(0, 1 << 30)
+    cap = np.full(n, 260, np.int64)
+    out = al.outputs(n, cigar_capacity=torch.from_numpy(cap))
+    coff = np.concatenate([[0], np.cumsum(cap)])
+    plan = aim.aim_batch_plan(al.ctx, buf, buf, ro_d, to_d, rl, tl, slot, aim.penalties(4, 6, 2), 60, pp, out["scores"],
+                              out["cigars"], out["cigar_offsets"], out["cigar_lens"], out["flags"], autotune=autotune)
+    for step, ((p, text), me) in enumerate(steps):
+        me = me.astype(np.int32)
+        buf.copy_(torch.from_numpy(text)); pp.copy_(torch.from_numpy(me))
+        rl.copy_(torch.from_numpy(p.read_len.view(np.int32))); tl.copy_(torch.from_numpy(p.target_len.view(np.int32)))
+        aim.aim_batch_run(plan); torch.cuda.synchronize()
+        s, f = out["scores"].cpu().numpy(), out["flags"].cpu().numpy()
+        ln, cg = out["cigar_lens"].cpu().numpy(), out["cigars"].cpu().numpy().view(np.uint32)
+        plain = device_results(p, "wfa", AFF, 60, per_pair=me)
+        assert np.array_equal(s, plain[0]) and np.array_equal(f, plain[1]), step
+        assert all(np.array_equal(cg[coff[i]:coff[i] + ln[i]], plain[2][i]) for i in range(n)), step
+        idx = rng.choice(n, 60, replace=False)
+        sub = gen.concat([gen.from_strings([p.read(i)], [p.target(i)]) for i in idx])
+        assert_same((s, f, [cg[coff[i]:coff[i] + ln[i]] for i in range(n)]),
+                    oracle_results(sub, AFF, me[idx].astype(np.int64) * 8), idx=idx, what=f"replay {step}")
+    aim.aim_batch_destroy(plan)
+    al.close()
