@@ -201,7 +201,7 @@ AIM_API int aim_align_batch_ascii(aim_ctx *ctx, const uint8_t *reads, const uint
  * The batch goes through the device in chunks, two device slots in turn: while
  * one chunk aligns, the next one's inputs copy in and the previous one's
  * results copy out.  AIM_ALGO_WFA_AFFINE runs the batched form (each slot holds
- * a batch plan, autotuned on the first chunk; a short last chunk is padded with
+ * a batch plan, planned on its first chunk; a short last chunk is padded with
  * empty pairs; each slot's plan takes half of the context workspace as its
  * scratch, so one chunk's launches overlap the next one's); the other
  * algorithms run the plain form per chunk.  The slots, streams and plans stay
@@ -363,8 +363,8 @@ AIM_API int aim_set_batch_compact(aim_ctx *ctx, int mode);
  * a diamond around the optimal paths.  Scores, flags and CIGARs are those of
  * the exact pass alone.  aim_batch_bound_passes reports, per bucket, the
  * bound pass's lanes per pair (0: none; 1: the form with its few diagonals in
- * registers, a lane or a warp per pair) and returns the number of buckets with
- * one.  aim_set_batch_bound sets how later plans of the context choose: 0
+ * registers, a lane or a warp per pair; a forced one is reported as 4 whichever
+ * form runs) and returns the number of buckets with one.  aim_set_batch_bound sets how later plans of the context choose: 0
  * (default) by timed trials when autotuning, or, with wavefronts in shared
  * memory, for every class that may reach a scaled score of 48 (but not for a
  * batch that makes one small class); 1 always (reads up to 32,000 bp), 2

@@ -20,10 +20,15 @@
 // range, of the kernel compiled for that group size alone (one kernel holding
 // every group size spilled registers and ran 14 % slower).
 //
-// Autotuner.  For every non-empty bucket, timed trial launches on a sample of
-// its pairs large enough to fill the device several times try the group sizes that suit its width class (so
-// that no lane walks more than about 64 diagonals per score step; the widest
-// class may also use a whole block per pair) and keep the fastest; choices are cached in the context per (costs, band, bucket).
+// Autotuner (plans of these buckets only; plans of wfa_ring.cu, below, choose by
+// rule).  For every non-empty bucket, timed trial launches on a sample of its
+// pairs large enough to fill the device several times try the group sizes that
+// suit its width class (so that no lane walks more than about 64 diagonals per
+// score step; the widest class may also use a whole block per pair) and keep
+// the fastest; choices are cached in the context per (costs, band, bucket).
+// Trials run the kernels that the plan would: buckets that fit wfa_ring.cu run
+// it in plans of one pass, and wfa.cu's kernels where any bucket has a compact
+// first pass, so such costs are tried both ways.
 //
 // Two passes.  A bucket's scratch is sized for its worst case, which for long
 // pairs under a loose threshold only fits one pair per warp.  Most pairs end

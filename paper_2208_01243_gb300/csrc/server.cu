@@ -568,8 +568,8 @@ int aim_server_submit(aim_server* s, const aim_request* q, uint64_t* ticket) {
             job.warp_bytes = wfa_pair_bytes(job.plan, 32);
         }
         // a bound pass before the exact one for the heaviest classes (work class >= 5, wavefronts over 256
-        // diagonals), where the batched form's tuner keeps one: 4 lanes per pair before groups of up to 32 lanes,
-        // 16 before whole blocks.  Results are the exact pass's either way.
+        // diagonals): wfa_bound.cu's form, or, for costs that it does not take, 4 lanes per pair before groups of up to
+        // 32 lanes and 16 before whole blocks.  Results are the exact pass's either way.
         const int key = keyed[i].first, kc = 7 - key / 4, wc = 3 - key % 4;
         job.bound_group = kc >= 5 && wc == 3 && jl <= kMaxWfaLength16 ? (job.group > 32 ? 16 : 4) : 0;
         // warps wanted: every pair in flight at once (a 256-lane group uses 8 warps), within the device's capacity
