@@ -25,9 +25,9 @@
 // computed but nothing at or left of column m reads them; the diagonal after the last one is set infinite.  Infinity
 // is 2^30 + 2^29, and the host checks that four times the costs along a path stay below 2^28, so infinite values,
 // which move by as much, stay apart from others.
-// What bounds it: the integer pipe (70 % busy), 24 lane instructions a cell of which the three 3-input minima, three
-// shifts into the trace and three ranks are most.  1M pairs of 250 bp, band 25: 13.4 ms, 9,700 warp instructions a
-// pair (dp_banded.cu: 51.3 ms and 55,400); edit distance, 1M x 100 bp, band 10: 1.45 ms (9.3 ms).  With ranks compared
+// What bounds it: the integer pipe and issue (59 % and 1.8 per cycle over 50k pairs, whose second wave is a third full),
+// 24 lane instructions a cell of which the three 3-input minima, three shifts into the trace and three ranks are most.  1M
+// pairs of 250 bp, band 25: 13.4 ms, 9,700 warp instructions a pair (dp_banded.cu: 51.3 ms and 55,400); edit distance, 1M x 100 bp, band 10: 1.45 ms (9.3 ms).  With ranks compared
 // by equality and six bits assembled per cell it took 15.3 ms, with costs not relative to 4 e (v + h) 15.1 ms.
 #include <algorithm>
 #include <cstdint>

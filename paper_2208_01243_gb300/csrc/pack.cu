@@ -16,7 +16,7 @@
 // Bytes next to a sequence are converted like its own: the shift drops those before it and a mask those after it;
 // only a chunk that shows a byte other than the four is looked at again, with the bytes outside the sequence masked.
 //
-// What bounds it: the latency of the 16-byte loads and the integer pipe (58 % busy) about evenly; 40 registers, for 48
+// What bounds it: the latency of the 16-byte loads (6.3 of 14 stalls an issue) and the integer pipe (59 % busy); 40 registers, for 48
 // warps on an SM, measured better than more registers or loads issued a turn ahead (136 us with 55 registers, 132 us
 // with the loads ahead).  1M sequences of 100-1,000 bp (391 MB) in 123 us, 4.2 TB/s of 6.8, from 901 us with a warp
 // per sequence and a byte per lane; 1M of 150 bp 62 us (from 392 us; a thread per word in fixed slots 63 us, and 105

@@ -20,6 +20,9 @@
 // and whether J and K came from the extension (on ties they do: the traceback takes an extension before an opening).
 // Following these bits is the source-following traceback: at each step the word of one entry says where to go, and a
 // gap's offset is the M~ at its opening.  A table holds each row's place and each pair's first diagonal in it.
+//
+// What bounds it: issue and the integer pipe (2.4 per cycle, 53-58 % busy) with 20 to 23 of 32 lanes at work: 56,600 warp
+// instructions a pair of 1,000 bp at 5 % and 8 lanes, two reductions of three shuffles and the votes in every score.
 #include <algorithm>
 #include <cstdint>
 

@@ -11,8 +11,9 @@
 // limit gets no bound (-1), and its exact pass runs under the limit alone.
 // Pairs end at scores far apart, so idle lanes take new pairs while the others carry on (kRefill).  1M pairs of
 // 100-1,000 bp, 1-10 %: 3.8 ms in step with the slowest lane (16 of 32 lanes at work), 2.3 ms with refills; wfa.cu's
-// groups of four lanes took about 11 ms over the same pairs.  That form is issue bound (400 instructions a score for 32
-// pairs); a warp per pair is bound by one score's chain of loads and shuffles, about 0.15 us: 4,000 pairs of 1-10 kbp in
+// groups of four lanes took about 11 ms over the same pairs.  That form runs 400 instructions a score for 32 pairs with the
+// few warps that their copies leave room for (1.3 per cycle, 14 of 32 lanes at work over 50k pairs); a warp per pair is
+// bound by one score's chain of loads and shuffles, about 0.15 us (0.66 per cycle): 4,000 pairs of 1-10 kbp in
 // 11.0 ms all told (14.3 with wfa.cu's 32-lane groups, 14.2 without a bound pass; 16 lanes a pair and a window of 16
 // diagonals, which loses the end more often, 11.8), a server's burst of 24 requests in 31 ms (36).
 #include <algorithm>

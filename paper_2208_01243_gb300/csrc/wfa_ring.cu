@@ -27,9 +27,11 @@
 // traceback computes where that is (RowMap).  A round of P pairs leaves its history in its unit's arena; after
 // 32 pairs (or when the arena may not hold another round) a lane each traces them back, by the tests of wfa.cu.
 //
-// What bounds it: instruction issue.  1M pairs of 150 bp at 6 edits take 900 warp instructions a pair at 2.7 per
-// cycle (wfa.cu's 4-lane groups: 1,790 at 2.2), 1.03 ms against 2.43 ms; 250 bp, band 25, 25 edits 9.6 ms against
-// 21.4 ms (all on one launch, packing apart).
+// What bounds it: instruction issue at short reads.  150 bp at 6 edits take 931 warp instructions a pair, 22 of 32 lanes
+// at work, 95 thread instructions for each of some 217 entries, at 2.2 per cycle (100k pairs; wfa.cu's 4-lane groups 1,790);
+// 250 bp, band 25, 4 lanes, 9,480 at 2.8.  1M pairs of the first in 1.03 ms against 2.43 ms, of the second in 9.6 ms against
+// 21.4 ms (all on one launch, packing apart).  Wide windows leave shared memory for few warps (10-13 % of an SM's at 16 and
+// 32 lanes: 1.6-1.9 per cycle), and a block per pair waits at its barrier (4.0 of 7.8 stalls an issue at 5 kbp, 1.7).
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
